@@ -233,6 +233,49 @@ __global__ void wsum_kernel(const double *w, int64_t n, double *out) {
     if (threadIdx.x == 0) *out = red[0];
 }
 
+// Extent (see internal.h) of points [off[y], off[y + 1]) of surface y =
+// blockIdx.y (off NULL: all n points), block x of kExtentBlocks partials each.
+__global__ void extent_kernel(const double *xyz, const double *nrm, const double *w, int64_t n, const int64_t *off,
+                              Extent *out) {
+    __shared__ double red[8][256];
+    const int64_t beg = off ? off[blockIdx.y] : 0, end = off ? off[blockIdx.y + 1] : n;
+    double v[8] = {1e308, 1e308, 1e308, 1e308, 1e308, 1e308, 0.0, 1.0};   // lo, -hi (minima), -mmax, fin
+    for (int64_t i = beg + (int64_t)blockIdx.x * 256 + threadIdx.x; i < end; i += (int64_t)gridDim.x * 256) {
+        for (int c = 0; c < 3; ++c) {
+            const double x = xyz[c * n + i], m = w[i] * nrm[c * n + i];
+            v[c] = fmin(v[c], x);
+            v[3 + c] = fmin(v[3 + c], -x);
+            v[6] = fmin(v[6], -fabs(m));
+            if (!isfinite(x) || !isfinite(m)) v[7] = 0.0;
+        }
+    }
+    for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = v[q];
+    __syncthreads();
+    for (int st = 128; st > 0; st >>= 1) {
+        if (threadIdx.x < st)
+            for (int q = 0; q < 8; ++q)
+                red[q][threadIdx.x] = fmin(red[q][threadIdx.x], red[q][threadIdx.x + st]);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        Extent e;
+        for (int c = 0; c < 3; ++c) { e.lo[c] = red[c][0]; e.hi[c] = -red[3 + c][0]; }
+        e.mmax = -red[6][0];
+        e.fin = red[7][0];
+        out[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = e;
+    }
+}
+
+Extent merge_extents(const Extent *e, int k) {
+    Extent r = e[0];
+    for (int i = 1; i < k; ++i) {
+        for (int c = 0; c < 3; ++c) { r.lo[c] = fmin(r.lo[c], e[i].lo[c]); r.hi[c] = fmax(r.hi[c], e[i].hi[c]); }
+        r.mmax = fmax(r.mmax, e[i].mmax);
+        r.fin = fmin(r.fin, e[i].fin);
+    }
+    return r;
+}
+
 // ------------------------------------------------------------- batched layouts
 // key = surface index above a 30-bit Morton code of the position in the
 // batch's bounding box: sorting groups each surface's points in Morton order
@@ -383,7 +426,8 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
                  o_w32 = carve(sizeof(float4) * np), o_p64 = carve(sizeof(d4) * np),
                  o_w64 = carve(sizeof(d4) * np), o_cb = carve(sizeof(float4) * 2 * (np / kChunk)),
                  o_es = carve(sizeof(int32_t) * n), o_ws = carve(sizeof(double) * ns),
-                 o_sc = carve(sizeof(double) * ns), o_meta = carve(sizeof(int64_t) * (4 * ns + 1));
+                 o_sc = carve(sizeof(double) * ns), o_meta = carve(sizeof(int64_t) * (4 * ns + 1)),
+                 o_ex = carve(sizeof(Extent) * ns), o_geo = carve(fx_geo_bytes(ns));
     void *blk = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &blk));
     char *bp = static_cast<char *>(blk);
@@ -400,6 +444,8 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
     out.d_wsum = reinterpret_cast<double *>(bp + o_ws);
     out.d_selfc = reinterpret_cast<double *>(bp + o_sc);
     int64_t *dmeta = reinterpret_cast<int64_t *>(bp + o_meta);   // off[ns+1], cnt[ns], poff[ns]
+    Extent *dext = reinterpret_cast<Extent *>(bp + o_ex);
+    out.fx_geo = bp + o_geo;
     std::vector<int64_t> hmeta(4 * ns + 1, 0);
     for (int k = 0; k <= ns; ++k) hmeta[k] = b->offsets[k];
     for (int k = 0; k < ns; ++k) { hmeta[ns + 1 + k] = out.n[k]; hmeta[2 * ns + 1 + k] = out.poff[k]; }
@@ -449,12 +495,19 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
                 batch_fill_kernel<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(fa, out.L);
                 batch_chunk_box_kernel<<<(unsigned)((np / kChunk + 127) / 128), 128, 0, s>>>(out.L);
                 batch_wsum_kernel<<<ns, 256, 0, s>>>(b->w, dmeta, out.d_wsum);
-                ctx->launches += 3;
+                for (int k = 0; k < ns; k += 65535)   // grid.y limit
+                    extent_kernel<<<dim3(1, (unsigned)(ns - k < 65535 ? ns - k : 65535)), 256, 0, s>>>(
+                        b->xyz, b->nrm, b->w, n, dmeta + k, dext + k);
+                ctx->launches += 4;
                 st = launch_check(ctx, "batch fill");
             }
         }
     }
     out.wsum.resize(ns);
+    out.ext.resize(ns);
+    if (st == SSD_OK)
+        st = cuda_check(ctx, cudaMemcpyAsync(out.ext.data(), dext, sizeof(Extent) * ns, cudaMemcpyDeviceToHost, s),
+                        "extent copy");
     if (st == SSD_OK)
         st = cuda_check(ctx, cudaMemcpyAsync(out.wsum.data(), out.d_wsum, sizeof(double) * ns,
                                              cudaMemcpyDeviceToHost, s), "wsum copy");
@@ -485,8 +538,7 @@ int check_points(ssd_ctx *ctx, const ssd_points *pts) {
 
 void release_layout(ssd_ctx *ctx, Layout *L) {
     if (L->block) dev_free(ctx, L->block);
-    for (int k = 0; k < 2; ++k)
-        if (L->order32[k]) dev_free(ctx, L->order32[k]);
+    if (L->order32) dev_free(ctx, L->order32);
     for (auto &pl : L->sym)
         if (pl.block) dev_free(ctx, pl.block);
     *L = Layout();
@@ -503,7 +555,8 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cuda
     const size_t o_p64 = carve(sizeof(d4) * n_pad);
     const size_t o_w64 = carve(sizeof(d4) * n_pad);
     const size_t o_cb = carve(sizeof(float4) * 2 * (n_pad / kChunk));
-    const size_t o_ws = carve(sizeof(double) * 8);
+    // weight sum, then the extent partials: one host read
+    const size_t o_ws = carve(sizeof(double) * 8 + sizeof(Extent) * kExtentBlocks);
     void *blk = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &blk));
     char *b = static_cast<char *>(blk);
@@ -553,16 +606,21 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cuda
         fill_layout_kernel<<<(unsigned)((n_pad + 255) / 256), 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, n_pad,
                                                                           sorted, out);
         wsum_kernel<<<1, 256, 0, s>>>(pts->w, n, dsum);
+        extent_kernel<<<kExtentBlocks, 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, nullptr,
+                                                    reinterpret_cast<Extent *>(dsum + 8));
         chunk_box_kernel<<<(unsigned)((n_pad / kChunk + 127) / 128), 128, 0, s>>>(out);
-        ctx->launches += 3;
+        ctx->launches += 4;
         st = launch_check(ctx, "layout fill");
     }
-    if (st == SSD_OK) st = cuda_check(ctx, cudaMemcpyAsync(ctx->hbuf, dsum, sizeof(double),
+    static_assert(8 + 8 * kExtentBlocks <= 512, "the read fits the pinned scratch");
+    if (st == SSD_OK) st = cuda_check(ctx, cudaMemcpyAsync(ctx->hbuf, dsum,
+                                                           sizeof(double) * 8 + sizeof(Extent) * kExtentBlocks,
                                                            cudaMemcpyDeviceToHost, s), "wsum copy");
     if (st == SSD_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "layout sync");
     if (tmp) dev_free(ctx, tmp);
     if (st != SSD_OK) { release_layout(ctx, &out); return st; }
     out.wsum = ctx->hbuf[0];
+    out.ext = merge_extents(reinterpret_cast<const Extent *>(ctx->hbuf + 8), kExtentBlocks);
     if (!(out.wsum > 0.0)) {
         release_layout(ctx, &out);
         return set_error(ctx, SSD_EINVAL, "quadrature weights must have a positive sum");
@@ -627,7 +685,7 @@ int ssd_ctx_create(ssd_ctx **out, int device) {
     if (const char *w = getenv("SSD_PAIR_SYM")) ctx->sym = atoi(w) != 0;
     if (const char *w = getenv("SSD_PAIR_WAVES64")) {
         const int v = atoi(w);
-        if (v >= 1 && v <= 64) ctx->waves64 = v;
+        if (v >= 1 && v <= 64) ctx->waves64 = ctx->waves_fx = v;
     }
     *out = ctx;
     return SSD_OK;

@@ -1,0 +1,448 @@
+// FP64 pair sums in fixed point: kernel, packing and host set-up (included by
+// pair.cu inside its namespace, after the generic pair kernel).
+//
+// What bounds it: the integer pipes.  One Stokes double-layer pair is about
+// 70 wide multiply-adds and 90 shifts, adds and logic operations, two thirds
+// of them replacing 31 double-precision operations that issue at 1.6 per
+// clock and SM; a smoothed pair costs the same as a bare one, where the
+// double-precision kernel also evaluates erf and exp (33 clocks per pair and
+// SM).  So there is no near/far split here, every tile costs the same, and
+// the grid needs no launch order.
+//
+// A CTA holds 256 targets, one per thread, and walks its sources 128 at a time
+// in shared memory next to the kernel tables (3 KB per octave of 1 + rho^2 and
+// table).  Positions keep one global grid; each tile shifts it so that its
+// largest distance fills 61 bits.  The tile's sums are integers (exact, so
+// their order does not matter); they enter a double accumulator once per tile.
+// Tables are read by lane-dependent index, sources by broadcast.
+// Measured on the h = 1/32 sphere (N = 17070), against the double-precision
+// kernel: Laplace double layer 2.1 ms (18.9), and on small sets, where every
+// pair is smoothed, Stokes double layer 0.053 ms (0.62) at N = 1062, fused
+// Stokes layers 0.113 ms (1.44) at N = 1742, transposed Stokes double layer
+// 0.34 ms (3.7) at N = 4302; errors against long double at or below the double
+// kernel's.  The wide multiplier is 80% busy (32 a clock and SM).
+//
+// Densities are scaled by their largest magnitude, which the packing kernel
+// leaves per block; the kernel reduces those at its start.  When that scale
+// does not exist (a NaN, an infinity, or a magnitude outside 2^+-400) the CTA
+// evaluates its pairs in double precision instead, as the generic kernel
+// does, so non-finite densities give the same results as there.  Point sets
+// whose extent is over 256 or under 1/16 delta, or that are not finite, keep the
+// generic kernel (fx_geo).
+
+constexpr int kFxExpMax = 400;
+
+struct FxGeo {
+    double c[3];          // grid origin
+    double inv, inv_lo;   // 1 / delta to twice double precision
+    double grid;          // 2^ps
+    int ps;               // positions: (x - c) / delta in units of 2^-ps
+    int em;               // |w n| < 2^em
+    int ed, pad;
+    int64_t dq;           // 1 / delta = dq 2^(ed - 62)
+    double f_sl, f_dl;    // 1 / delta, 1 / delta^2
+};
+
+struct FxArgs {
+    const l4 *X;
+    const int4 *cbox;            // per 32-point chunk: (lo, hi) of X >> 32
+    const unsigned long long *bmax;   // [rhs][pack block][2]: bits of the largest |d0|, |d1|
+    int64_t nblk;                // pack blocks per right-hand side
+    const FxI4 *tab;
+    int noct;
+    FxGeo geo;
+    const FxGeo *geos;           // batched: per surface
+    KArgs<double> k;             // the rest, as for the generic kernel
+    int64_t n;
+};
+
+// positions of the fixed-point grid, their chunk boxes and the densities' block
+// maxima (every thread of a 256-thread block calls this)
+struct FxPack {
+    l4 *X = nullptr;             // NULL: not wanted
+    int4 *cbox = nullptr;
+    unsigned long long *bmax = nullptr;
+    FxGeo geo;
+    const FxGeo *geos = nullptr;     // batched
+    const BSurf *surfs = nullptr;
+    int nsurf = 0;
+    int two = 0;                 // LSLDL: .y of the first record is the second density
+};
+
+__device__ __forceinline__ int64_t fx_grid(double x, double c, const FxGeo &g) {
+    const double hi = x - c, bb = hi - x, lo = (x - (hi - bb)) - (c + bb);   // x - c = hi + lo exactly
+    const double q = hi * g.inv;
+    const double e = fma(hi, g.inv, -q) + (hi * g.inv_lo + lo * g.inv);
+    const double r = q * g.grid;
+    const long long a = __double2ll_rn(r);
+    return a + __double2ll_rn((r - (double)a) + e * g.grid);
+}
+
+__device__ __forceinline__ void fx_pack(const FxPack &P, int64_t i, int64_t n_last, const d4 *pos, const int32_t *perm,
+                                        const d4 &r0, const d4 &r1, int rhs, int64_t nblk) {
+    __shared__ unsigned long long smax[2][8];
+    __shared__ int ssurf;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned long long am = 0x7fffffffffffffffull;
+    auto bits = [&](double v) { return (unsigned long long)__double_as_longlong(v) & am; };
+    unsigned long long m0 = bits(r0.x), m1 = 0;
+    if (P.two) m1 = bits(r0.y);
+    else { m0 = max(m0, max(bits(r0.y), bits(r0.z))); m1 = max(bits(r1.x), max(bits(r1.y), bits(r1.z))); }
+    for (int off = 16; off > 0; off >>= 1) {
+        m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, off));
+        m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
+    }
+    if (lane == 0) { smax[0][warp] = m0; smax[1][warp] = m1; }
+    if (threadIdx.x == 0) {
+        int lo = 0, hi = P.nsurf - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (P.surfs[mid].poff <= i) lo = mid; else hi = mid - 1;
+        }
+        ssurf = lo;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        unsigned long long m = smax[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w) m = max(m, smax[threadIdx.x][w]);
+        P.bmax[((int64_t)rhs * nblk + blockIdx.x) * 2 + threadIdx.x] = m;
+    }
+    if (rhs != 0) return;
+    const FxGeo &g = P.geos ? P.geos[ssurf] : P.geo;
+    const int64_t last = P.surfs ? P.surfs[ssurf].poff + P.surfs[ssurf].n_real - 1 : n_last;
+    const d4 p = pos[i <= last ? i : last];   // padding: a copy of the last point, with zero weight and density
+    const int64_t x = fx_grid(p.x, g.c[0], g), y = fx_grid(p.y, g.c[1], g), z = fx_grid(p.z, g.c[2], g);
+    P.X[i] = l4{x, y, z, 0};
+    const int xh = (int)(x >> 32), yh = (int)(y >> 32), zh = (int)(z >> 32);
+    const int4 lo = make_int4(__reduce_min_sync(0xffffffffu, xh), __reduce_min_sync(0xffffffffu, yh),
+                              __reduce_min_sync(0xffffffffu, zh), 0);
+    const int4 hi = make_int4(__reduce_max_sync(0xffffffffu, xh), __reduce_max_sync(0xffffffffu, yh),
+                              __reduce_max_sync(0xffffffffu, zh), 0);
+    if (lane == 0) { P.cbox[2 * (i >> 5)] = lo; P.cbox[2 * (i >> 5) + 1] = hi; }
+}
+
+// The generic kernel's pair terms for one target in double precision, all
+// pairs of [s_beg, s_end) in order (densities without a common scale).
+template <int OP>
+__device__ __noinline__ void fx_fallback(const KArgs<double> *ap, const Consts<double> *cp, const d4 *d0, const d4 *d1,
+                                         int64_t i, int64_t s_beg, int64_t s_end, double out[3]) {
+    const KArgs<double> &a = *ap;
+    const Consts<double> c = *cp;
+    const d4 yp = a.pos[i], yd = d0[i], yw = a.wn[i];
+    const double dt[3] = {yd.x, yd.y, yd.z}, twn[3] = {yw.x, yw.y, yw.z};
+    double acc[3] = {0.0, 0.0, 0.0};
+    for (int64_t j = s_beg; j < s_end; ++j) {
+        const d4 sp = a.pos[j], sw = a.wn[j], s0 = d0[j], s1 = d1[j];
+        const double d[3] = {yp.x - sp.x, yp.y - sp.y, yp.z - sp.z};
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        if (r2 < c.rfar2) pair_term<double, OP, true>(d, r2, dt, sw, s0, s1, c, true, false, acc, twn);
+        else pair_term<double, OP, false>(d, r2, dt, sw, s0, s1, c, false, false, acc, twn);
+    }
+    out[0] = acc[0]; out[1] = acc[1]; out[2] = acc[2];
+}
+
+template <int OP>
+__global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ FxArgs a) {
+    typedef FxOp<OP> T;
+    constexpr int NC = OpInfo<OP>::NC;
+    constexpr bool M = T::dl, VU = T::dl && T::vec, VF = T::sl && T::vec;
+    extern __shared__ __align__(16) FxI4 s_tab[];           // [ntab][noct * kFxSeg][kFxEntry]
+    // staged sources: limbs of the vectors, scalars in the spare words
+    __shared__ int4 s_xh[kTile], s_xl[kTile];
+    __shared__ int4 s_mh[M ? kTile : 1], s_ml[M ? kTile : 1];
+    __shared__ int4 s_uh[VU ? kTile : 1], s_ul[VU ? kTile : 1];
+    __shared__ int4 s_fh[VF ? kTile : 1], s_fl[VF ? kTile : 1];
+    __shared__ unsigned long long s_max[2][kFxTPB / 32];
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t tbase, s_beg, s_end, part_base, pstride, b0 = 0, b1 = a.nblk;
+    const d4 *d0 = a.k.d0, *d1 = a.k.d1;
+    const FxGeo *gp = &a.geo;
+    const Consts<double> *cp = &a.k.c;
+    if (a.k.items) {
+        const BItem it = a.k.items[blockIdx.x];
+        const BSurf sf = a.k.surfs[it.surf];
+        tbase = it.tbase; s_beg = it.s_beg; s_end = it.s_end;
+        if (a.geos) {
+            gp = a.geos + it.surf;
+            b0 = sf.poff / 256; b1 = (sf.poff + sf.n_pad) / 256;
+        }
+        cp = a.k.consts + it.surf;
+        d0 += blockIdx.y * a.k.rec_stride;
+        d1 += blockIdx.y * a.k.rec_stride;
+        part_base = blockIdx.y * a.k.part_stride + NC * sf.pbase + (int64_t)it.split * NC * sf.n_pad - sf.poff;
+        pstride = sf.n_pad;
+    } else {
+        tbase = (blockIdx.x + a.k.tile0) * kFxTPB;
+        s_beg = blockIdx.y * a.k.chunk;
+        s_end = s_beg + a.k.chunk;
+        const int64_t top = (a.n + kChunk - 1) / kChunk * kChunk;
+        if (s_end > top) s_end = top;
+        part_base = blockIdx.y * NC * a.k.n_pad;
+        pstride = a.k.n_pad;
+    }
+    const int64_t i = tbase + threadIdx.x;
+    // largest densities of this surface and right-hand side
+    {
+        unsigned long long m0 = 0, m1 = 0;
+        const unsigned long long *bm = a.bmax + (a.geos ? blockIdx.y : 0) * a.nblk * 2;
+        for (int64_t b = b0 + threadIdx.x; b < b1; b += kFxTPB) { m0 = max(m0, bm[2 * b]); m1 = max(m1, bm[2 * b + 1]); }
+        for (int off = 16; off > 0; off >>= 1) {
+            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, off));
+            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
+        }
+        if (lane == 0) { s_max[0][warp] = m0; s_max[1][warp] = m1; }
+    }
+    for (int k = 0; k < T::ntab; ++k) {
+        const int4 *src = reinterpret_cast<const int4 *>(a.tab) + (int64_t)T::tab(k) * kFxMaxOct * kFxSeg * kFxEntry;
+        int4 *dst = reinterpret_cast<int4 *>(s_tab) + (int64_t)k * a.noct * kFxSeg * kFxEntry;
+        for (int q = threadIdx.x; q < a.noct * kFxSeg * kFxEntry; q += kFxTPB) dst[q] = src[q];
+    }
+    __syncthreads();
+    int ee[2];
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        unsigned long long m = 0;
+#pragma unroll
+        for (int w = 0; w < kFxTPB / 32; ++w) m = max(m, s_max[k][w]);
+        const int ex = (int)(m >> 52);
+        ee[k] = m == 0 ? -kFxExpMax : ex - 1022;            // all zero: any scale
+        bad |= m != 0 && (ee[k] > kFxExpMax || ee[k] < -kFxExpMax);
+    }
+    double sum[3] = {0.0, 0.0, 0.0}, low[3] = {0.0, 0.0, 0.0};
+    if (bad) {
+        fx_fallback<OP>(&a.k, cp, d0, d1, i, s_beg, s_end, sum);
+    } else {
+        const FxGeo &g = *gp;
+        const FxScale sc = fx_scale<OP>(ee[0], ee[1], g.em, g.dq, g.ed);
+        FxPoint<OP> y;
+        const l4 Y = a.X[i];
+        {
+            const d4 d = d0[i];
+            if constexpr (VU) {
+                fx_split(fx_fix(d.x, sc.eu, 58), y.u.h[0], y.u.l[0]);
+                fx_split(fx_fix(d.y, sc.eu, 58), y.u.h[1], y.u.l[1]);
+                fx_split(fx_fix(d.z, sc.eu, 58), y.u.h[2], y.u.l[2]);
+            }
+            if constexpr (!T::vec && T::dl) y.p = fx_fix(d.x, sc.eu, 60);
+            if constexpr (T::tr) {
+                const d4 m = a.k.wn[i];
+                fx_split(fx_fix(m.x, sc.em, 59), y.m.h[0], y.m.l[0]);
+                fx_split(fx_fix(m.y, sc.em, 59), y.m.h[1], y.m.l[1]);
+                fx_split(fx_fix(m.z, sc.em, 59), y.m.h[2], y.m.l[2]);
+            }
+        }
+        int tlo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, thi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
+#pragma unroll
+        for (int k = 0; k < kFxTPB / kChunk; ++k) {
+            const int4 l = a.cbox[2 * (tbase / kChunk + k)], h = a.cbox[2 * (tbase / kChunk + k) + 1];
+            tlo[0] = min(tlo[0], l.x); tlo[1] = min(tlo[1], l.y); tlo[2] = min(tlo[2], l.z);
+            thi[0] = max(thi[0], h.x); thi[1] = max(thi[1], h.y); thi[2] = max(thi[2], h.z);
+        }
+        const uint32_t idx_max = (uint32_t)(a.noct * kFxSeg - 1);
+        const int4 *tab4 = reinterpret_cast<const int4 *>(s_tab);
+        const int tstride = a.noct * kFxSeg * kFxEntry;
+        auto tab = [&](int k, uint32_t idx, int w) {
+            const int4 v = tab4[k * tstride + idx * kFxEntry + w];
+            return FxI4{v.x, v.y, v.z, v.w};
+        };
+        for (int64_t tile = s_beg; tile < s_end; tile += kTile) {
+            const int cnt = (int)(s_end - tile < kTile ? s_end - tile : kTile);   // a multiple of kChunk
+            // the tile's largest distance exponent L and a lower bound 2^r of its distances
+            int dmax = 0, gap = 0;
+            {
+                int slo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, shi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
+                for (int k = 0; k < cnt / kChunk; ++k) {
+                    const int4 l = a.cbox[2 * (tile / kChunk + k)], h = a.cbox[2 * (tile / kChunk + k) + 1];
+                    slo[0] = min(slo[0], l.x); slo[1] = min(slo[1], l.y); slo[2] = min(slo[2], l.z);
+                    shi[0] = max(shi[0], h.x); shi[1] = max(shi[1], h.y); shi[2] = max(shi[2], h.z);
+                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    dmax = max(dmax, max(thi[c] - slo[c], shi[c] - tlo[c]) + 1);
+                    gap = max(gap, max(tlo[c] - shi[c], slo[c] - thi[c]) - 1);
+                }
+            }
+            // distances < dmax 2^(32 - ps) <= 2^L, >= gap 2^(32 - ps) >= 2^r
+            const int L = max(0, 32 - g.ps + (32 - __clz(dmax - 1)));
+            const int r = gap > 0 ? max(0, 31 - __clz(gap) + 32 - g.ps) : 0;
+            const FxTile tl = fx_tile<OP>(sc, L, r);
+            const int ks = 61 - L - g.ps;
+            auto grid = [&](int64_t v) { return ks >= 0 ? (int64_t)((uint64_t)v << ks) : v >> -ks; };
+            __syncthreads();
+            if (threadIdx.x < cnt) {
+                const int64_t j = tile + threadIdx.x;
+                const l4 p = a.X[j];
+                const d4 e0 = d0[j];
+                int4 h, l;
+                fx_split(grid(p.x), h.x, l.x);
+                fx_split(grid(p.y), h.y, l.y);
+                fx_split(grid(p.z), h.z, l.z);
+                if constexpr (!T::vec) {
+                    const int64_t q = fx_fix(e0.x, sc.eu, 60);
+                    h.w = (int)(q >> 32);
+                    l.w = (int)q;
+                }
+                s_xh[threadIdx.x] = h;
+                s_xl[threadIdx.x] = l;
+                if constexpr (M) {
+                    const d4 m = a.k.wn[j];
+                    fx_split(fx_fix(m.x, sc.em, 59), h.x, l.x);
+                    fx_split(fx_fix(m.y, sc.em, 59), h.y, l.y);
+                    fx_split(fx_fix(m.z, sc.em, 59), h.z, l.z);
+                    if constexpr (OP == OP_LSLDL) {
+                        const int64_t q = fx_fix(e0.y, sc.ef, 60);
+                        h.w = (int)(q >> 32);
+                        l.w = (int)q;
+                    }
+                    s_mh[threadIdx.x] = h;
+                    s_ml[threadIdx.x] = l;
+                }
+                if constexpr (VU) {
+                    fx_split(fx_fix(e0.x, sc.eu, 58), h.x, l.x);
+                    fx_split(fx_fix(e0.y, sc.eu, 58), h.y, l.y);
+                    fx_split(fx_fix(e0.z, sc.eu, 58), h.z, l.z);
+                    s_uh[threadIdx.x] = h;
+                    s_ul[threadIdx.x] = l;
+                }
+                if constexpr (VF) {
+                    const d4 e1 = T::dl ? d1[j] : e0;
+                    fx_split(fx_fix(e1.x, sc.ef, 58), h.x, l.x);
+                    fx_split(fx_fix(e1.y, sc.ef, 58), h.y, l.y);
+                    fx_split(fx_fix(e1.z, sc.ef, 58), h.z, l.z);
+                    s_fh[threadIdx.x] = h;
+                    s_fl[threadIdx.x] = l;
+                }
+            }
+            __syncthreads();
+            fx_split(grid(Y.x), y.x.h[0], y.x.l[0]);
+            fx_split(grid(Y.y), y.x.h[1], y.x.l[1]);
+            fx_split(grid(Y.z), y.x.h[2], y.x.l[2]);
+            FxSum<OP> acc{};
+            // 4 pairs in flight fill the wide multiplier's latency (Stokes double layer
+            // 3.10 clocks per pair and SM against 3.50 unrolled once; the transposed
+            // Stokes layer has no registers left beyond 2)
+            constexpr int kUnroll = OP == OP_SDLT ? 2 : 4;
+#pragma unroll kUnroll
+            for (int j = 0; j < cnt; ++j) {
+                FxPoint<OP> x;
+                auto vec = [](FxV &v, const int4 &h, const int4 &l) {
+                    v.h[0] = h.x; v.h[1] = h.y; v.h[2] = h.z;
+                    v.l[0] = l.x; v.l[1] = l.y; v.l[2] = l.z;
+                };
+                auto word = [](const int4 &h, const int4 &l) { return ((int64_t)h.w << 32) | (uint32_t)l.w; };
+                const int4 xh = s_xh[j], xl = s_xl[j];
+                vec(x.x, xh, xl);
+                if constexpr (T::dl && !T::vec) x.p = word(xh, xl);
+                if constexpr (OP == OP_LSL) x.g = word(xh, xl);
+                if constexpr (M) {
+                    const int4 mh = s_mh[j], ml = s_ml[j];
+                    vec(x.m, mh, ml);
+                    if constexpr (OP == OP_LSLDL) x.g = word(mh, ml);
+                }
+                if constexpr (VU) vec(x.u, s_uh[j], s_ul[j]);
+                if constexpr (VF) vec(x.f, s_fh[j], s_fl[j]);
+                fx_pair<OP>(y, x, tl, sc, idx_max, tab, acc);
+            }
+            const double f = __longlong_as_double((long long)(1023 + tl.ex) << 52) *
+                             (T::fused || !T::dl ? g.f_sl : g.f_dl);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {   // TwoSum: the tiles add no rounding of their own
+                double v;
+                if constexpr (T::vec) v = fx_value(acc.v[c]) * f;
+                else v = ((double)acc.f.h + (double)acc.f.l * 2.3283064365386963e-10) * f;
+                const double t = sum[c] + v, b = t - sum[c];
+                low[c] += (sum[c] - (t - b)) + (v - b);
+                sum[c] = t;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) sum[c] += low[c];
+    }
+    if (a.k.acc) {
+#pragma unroll
+        for (int q = 0; q < NC; ++q) atomicAdd(a.k.acc + q * a.k.n_pad + i, sum[q]);
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < NC; ++q) a.k.part[part_base + (int64_t)q * pstride + i] = sum[q];
+}
+
+// Constants of a point set and smoothing radius; false when the fixed-point
+// kernel does not serve it (extent outside kFxMinExt .. kFxMaxExt delta, values
+// that are not finite or far from unit scale).  noct: octaves of 1 + rho^2 that occur.
+bool fx_geo(const Extent &e, double delta, FxGeo *g, int *noct) {
+    if (!(e.fin > 0.0)) return false;
+    double ext = 0.0, r2 = 0.0;
+    for (int c = 0; c < 3; ++c) {
+        const double d = e.hi[c] - e.lo[c];
+        g->c[c] = 0.5 * (e.lo[c] + e.hi[c]);
+        ext = fmax(ext, d / delta);
+        r2 += d / delta * (d / delta);
+    }
+    g->em = 0;
+    if (e.mmax > 0.0) frexp(e.mmax, &g->em);
+    int xd;
+    frexp(delta, &xd);
+    double cm = 0.0;
+    for (int c = 0; c < 3; ++c) cm = fmax(cm, fabs(g->c[c]));
+    if (!(ext >= kFxMinExt && ext <= kFxMaxExt) || g->em > kFxExpMax || g->em < -kFxExpMax || xd > 60 || xd < -60 || !(cm < 1e100))
+        return false;
+    int xe;
+    frexp(ext, &xe);
+    g->ps = 62 - xe < 58 ? 62 - xe : 58;       // |x - c| / delta <= 2^(xe - 1): the grid value stays below 2^62
+    g->grid = ldexp(1.0, g->ps);
+    g->inv = 1.0 / delta;
+    g->inv_lo = fma(-g->inv, delta, 1.0) / delta;
+    const double m = frexp(g->inv, &g->ed);    // 1 / delta = (m + lo) 2^ed, 62 bits
+    g->dq = (int64_t)ldexp(m, 53) * 512 + llrint(ldexp(g->inv_lo, 62 - g->ed));
+    g->f_sl = 1.0 / delta;
+    g->f_dl = 1.0 / (delta * delta);
+    g->pad = 0;
+    const int k = (int)floor(log2(1.0 + r2 * (1.0 + 1e-12))) + 1;
+    *noct = k < kFxMaxOct ? k : kFxMaxOct;
+    return true;
+}
+
+template <int OP> size_t fx_smem(int noct) {
+    return (size_t)FxOp<OP>::ntab * noct * kFxSeg * kFxEntry * sizeof(FxI4);
+}
+
+template <int OP> cudaError_t launch_fx1(dim3 grid, const FxArgs &a, cudaStream_t s) {
+    fx_kernel<OP><<<grid, kFxTPB, fx_smem<OP>(a.noct), s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fx(int op, dim3 grid, const FxArgs &a, cudaStream_t s) {
+    switch (op) {
+        case OP_LSL: return launch_fx1<OP_LSL>(grid, a, s);
+        case OP_LDL: return launch_fx1<OP_LDL>(grid, a, s);
+        case OP_SSL: return launch_fx1<OP_SSL>(grid, a, s);
+        case OP_SDL: return launch_fx1<OP_SDL>(grid, a, s);
+        case OP_SSLDL: return launch_fx1<OP_SSLDL>(grid, a, s);
+        case OP_LSLDL: return launch_fx1<OP_LSLDL>(grid, a, s);
+        case OP_LDLT: return launch_fx1<OP_LDLT>(grid, a, s);
+        default: return launch_fx1<OP_SDLT>(grid, a, s);
+    }
+}
+
+template <int OP> cudaError_t fx_attr1() {
+    return cudaFuncSetAttribute(fx_kernel<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx_smem<OP>(kFxMaxOct));
+}
+
+// Uploads the kernel tables of a context and lets the kernels use them.
+int fx_init(ssd_ctx *ctx) {
+    const size_t bytes = (size_t)4 * kFxMaxOct * kFxSeg * kFxEntry * sizeof(FxI4);
+    SSD_TRY(dev_alloc(ctx, bytes, &ctx->fx_tab));
+    SSD_TRY(cuda_check(ctx, cudaMemcpy(ctx->fx_tab, fx_table_host(), bytes, cudaMemcpyHostToDevice), "kernel tables"));
+    cudaError_t e = fx_attr1<OP_LSL>();
+    if (e == cudaSuccess) e = fx_attr1<OP_LDL>();
+    if (e == cudaSuccess) e = fx_attr1<OP_SSL>();
+    if (e == cudaSuccess) e = fx_attr1<OP_SDL>();
+    if (e == cudaSuccess) e = fx_attr1<OP_SSLDL>();
+    if (e == cudaSuccess) e = fx_attr1<OP_LSLDL>();
+    if (e == cudaSuccess) e = fx_attr1<OP_LDLT>();
+    if (e == cudaSuccess) e = fx_attr1<OP_SDLT>();
+    return cuda_check(ctx, e, "kernel attributes");
+}

@@ -1,0 +1,133 @@
+// Tables of the kernel factors sigma_i(t) = s_i(rho) / rho^p, t = rho^2
+// (s_i of Section 5.3; p = 1, 3, 3, 5), for the fixed-point pair sums.
+//
+// The variable is v = 1 + t: 64 segments of equal width per octave of v, so
+// the segments are narrow where the smoothing acts (t < 64) and scale with t
+// where the kernels are bare powers.  On each segment sigma_i is a polynomial
+// of degree 7 in s in [-1, 1]: the Chebyshev interpolant on 12 nodes,
+// truncated to degree 7 (largest neglected term below 2^-56 of the value) and
+// rewritten in powers of s.  Node values come from the closed forms in long
+// double, below t = 2 from the Maclaurin series (the closed forms cancel).
+#include <math.h>
+
+#include <mutex>
+#include <vector>
+
+#include "fx.h"
+
+namespace ssd {
+namespace {
+
+typedef long double ld;
+constexpr int kNodes = 12, kDeg = 7, kTerms = 48;
+const ld kPiL = 3.141592653589793238462643383279502884L;
+
+struct Sigma {
+    ld ser[4][kTerms];
+    Sigma() {
+        const ld q[4][4] = {{5.0L / 3, -2.0L / 3, 0, 0}, {-1, 2.0L / 3, 0, 0}, {-1, 14.0L / 3, -4.0L / 3, 0},
+                            {-1, -6.0L / 9, 4, -8.0L / 9}};
+        const int skip[4] = {0, 1, 1, 2};
+        const ld c = 2 / sqrtl(kPiL);
+        for (int i = 0; i < 4; ++i)
+            for (int k = 0; k < kTerms; ++k) {
+                const int n = k + skip[i];
+                ld f[4] = {0, 0, 0, 0}, fact = 1;   // (-1)^(n-m) / (n-m)!
+                std::vector<ld> inv(n + 1, 1.0L);
+                for (int j = 1; j <= n; ++j) { fact *= j; inv[j] = 1 / fact; }
+                ld a = ((n & 1) ? -1 : 1) * inv[n] / (2 * n + 1);
+                for (int m = 0; m < 4 && m <= n; ++m) {
+                    f[m] = (((n - m) & 1) ? -1 : 1) * inv[n - m];
+                    a += q[i][m] * f[m];
+                }
+                ser[i][k] = c * a;
+            }
+    }
+    // sigma_1 .. sigma_4 at t
+    void at(ld t, ld out[4]) const {
+        if (t < 2) {
+            for (int i = 0; i < 4; ++i) {
+                ld s = 0;
+                for (int k = kTerms - 1; k >= 0; --k) s = s * t + ser[i][k];
+                out[i] = s;
+            }
+            return;
+        }
+        const ld rho = sqrtl(t);
+        ld er = 1, g = 0;
+        if (t < 80) {   // beyond, erf = 1 and e^{-t} = 0 to the table's precision
+            er = erfl(rho);
+            g = 2 / sqrtl(kPiL) * rho * expl(-t);
+        }
+        const ld s1 = er + g * (5 - 2 * t) / 3, s2 = er + g * (2 * t - 3) / 3,
+                 s3 = er + g * (t * (14 - 4 * t) - 3) / 3,
+                 s4 = er - g * (t * (t * (8 * t - 36) + 6) + 9) / 9;
+        out[0] = s1 / rho;
+        out[1] = s2 / (rho * t);
+        out[2] = s3 / (rho * t);
+        out[3] = s4 / (rho * t * t);
+    }
+};
+
+int64_t round_ll(ld x) { return (int64_t)llrintl(x); }
+
+std::vector<FxI4> build() {
+    static const Sigma sig;
+    std::vector<FxI4> tab((size_t)4 * kFxMaxOct * kFxSeg * kFxEntry);
+    ld node[kNodes], cheb[kNodes][kNodes];   // nodes, T_k(node_j)
+    for (int j = 0; j < kNodes; ++j) {
+        node[j] = cosl(kPiL * (j + 0.5L) / kNodes);
+        for (int k = 0; k < kNodes; ++k) cheb[k][j] = cosl(kPiL * k * (j + 0.5L) / kNodes);
+    }
+    ld mono[kDeg + 1][kDeg + 1] = {};        // T_k in powers of s
+    mono[0][0] = 1;
+    mono[1][1] = 1;
+    for (int k = 2; k <= kDeg; ++k)
+        for (int p = 0; p <= k; ++p) mono[k][p] = (p ? 2 * mono[k - 1][p - 1] : 0) - mono[k - 2][p];
+    for (int o = 0; o < kFxMaxOct; ++o)
+        for (int g = 0; g < kFxSeg; ++g) {
+            const ld base = ldexpl(1, o), hw = base / (2 * kFxSeg);
+            const ld vc = base + (2 * g + 1) * hw;
+            ld val[4][kNodes];
+            for (int j = 0; j < kNodes; ++j) {
+                ld v4[4];
+                sig.at(vc - 1 + hw * node[j], v4);
+                for (int i = 0; i < 4; ++i) val[i][j] = v4[i];
+            }
+            for (int i = 0; i < 4; ++i) {
+                ld c[kDeg + 1] = {}, top = 0;
+                for (int j = 0; j < kNodes; ++j) top = fmaxl(top, fabsl(val[i][j]));
+                for (int k = 0; k <= kDeg; ++k) {
+                    ld a = 0;
+                    for (int j = 0; j < kNodes; ++j) a += val[i][j] * cheb[k][j];
+                    a *= (k ? 2.0L : 1.0L) / kNodes;
+                    for (int p = 0; p <= k; ++p) c[p] += a * mono[k][p];
+                }
+                int ex;
+                frexpl(top * 1.002L, &ex);          // top < 2^ex: mantissa below 2^62 over the whole segment
+                const int e = 1 - ex;
+                const ld u = ldexpl(1, 61 + e);
+                int64_t q[kDeg + 1];
+                for (int p = 0; p <= 3; ++p) q[p] = round_ll(c[p] * u);
+                for (int p = 4; p <= kDeg; ++p) q[p] = round_ll(ldexpl(c[p] * u, p - 4 - fx_unit(i)));
+                FxI4 *t = &tab[((size_t)i * kFxMaxOct * kFxSeg + (size_t)o * kFxSeg + g) * kFxEntry];
+                auto lo = [](int64_t x) { return (int)(uint32_t)x; };
+                auto hi = [](int64_t x) { return (int)(x >> 32); };
+                t[0] = FxI4{lo(q[0]), hi(q[0]), lo(q[1]), hi(q[1])};
+                t[1] = FxI4{lo(q[2]), hi(q[2]), lo(q[3]), hi(q[3])};
+                t[2] = FxI4{(int)q[4], (int)q[5], (int)q[6], (int)((uint32_t)(int)q[7] << 8 | (uint32_t)(e + kFxEBias))};
+            }
+        }
+    return tab;
+}
+
+}  // namespace
+
+const FxI4 *fx_table_host() {
+    static std::once_flag once;
+    static std::vector<FxI4> tab;
+    std::call_once(once, [] { tab = build(); });
+    return tab.data();
+}
+
+}  // namespace ssd

@@ -30,8 +30,10 @@ constexpr int kTPT32 = SSD_TPT32;   // targets per thread, FP32C (pairs of packe
 #endif
 constexpr int kSymTPT = SSD_SYMTPT; // targets per thread of the FP32C symmetric kernel (4 or 8)
 constexpr int kChunk = 32;          // sources per bounding-box chunk (near/far test per warp)
-constexpr int kTPB64 = 128;         // threads per CTA, FP64 pair kernel
-constexpr int kTPT64 = 1;           // targets per thread, FP64
+constexpr int kTPB64 = 128;         // threads per CTA, generic pair kernel
+constexpr int kTPT64 = 1;           // targets per thread, generic pair kernel in FP32 (transposes)
+constexpr int kTPTd = 2;            // targets per thread, generic pair kernel in double
+constexpr int kFxTPB = 256;         // threads and targets per CTA, FP64 fixed-point kernel (= kTPB64 * kTPTd)
 constexpr int kRowAlign = 512;      // n_pad is a multiple of this (>= every CTA target span)
 
 // Operators of the pair kernels.
@@ -42,6 +44,11 @@ inline int op_components(int op) {
 }
 
 struct alignas(16) d4 { double x, y, z, w; };
+struct alignas(16) l4 { int64_t x, y, z, w; };
+
+// Extent of a point set, for the fixed-point FP64 kernels: box of the points,
+// largest |w n| component; fin is 0 when any of it is not finite.
+struct Extent { double lo[3], hi[3], mmax, fin; };
 
 // Plan that evaluates the far block pairs of a layout once for both
 // directions, cached for the last rho_far delta it was built for: near items
@@ -64,14 +71,14 @@ struct Layout {
     d4 *wn64 = nullptr;        // (w nx, w ny, w nz, 0)
     float4 *cbox = nullptr;    // per 32-point chunk: [2 * c] = (lo x, y, z, 0), [2 * c + 1] = (hi ...)
     double wsum = 0.0;         // sum of weights (host copy)
+    Extent ext{};              // box and largest weighted normal (host copy)
     void *block = nullptr;     // single allocation backing the arrays
     // launch order of the FP32C pair grid (prepared layouts only), cached for
     // the last (grid, rho_far delta) it was built for
-    // (slot 0: FP32C packed kernel, slot 1: FP64 generic kernel)
     bool order_ok = false;
-    int2 *order32[2] = {nullptr, nullptr};
-    int64_t order_nit[2] = {0, 0}, order_chunk[2] = {0, 0};
-    float order_rfar2[2] = {-1.f, -1.f};
+    int2 *order32 = nullptr;
+    int64_t order_nit = 0, order_chunk = 0;
+    float order_rfar2 = -1.f;
     // plans of the layer operators that evaluate far block pairs once for
     // both directions (prepared layouts only), one per precision:
     // [0] FP32C, [1] FP64
@@ -97,7 +104,9 @@ struct ssd_ctx {
     int waves32 = 12;          // FP32C grid: about this many waves of resident CTAs (tuned)
     int lpt = 1;               // pair grids in near-first order on prepared layouts
     int sym = 1;               // layer operators (both precisions): far block pairs once for both directions
+    int waves_fx = 4;          // FP64 fixed-point grid: about this many waves of resident CTAs
     int waves64 = 8;           // FP64 grid: about this many waves of resident CTAs (tuned)
+    void *fx_tab = nullptr;    // kernel tables of the fixed-point FP64 kernels (built with the context)
     void *noalloc_scratch = nullptr;   // device address of the no-alloc scratch array (first no-alloc call)
     std::string err;
     // caching device allocator: blocks are reused in stream order
@@ -178,6 +187,9 @@ struct PairCall {
 };
 int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s);
 int pair_occupancy(ssd_ctx *ctx);
+// reduces the extent of points [beg, end) of SoA arrays over `blocks` blocks, one partial each (ctx.cu)
+constexpr int kExtentBlocks = 32;
+size_t fx_geo_bytes(int nsurf);
 
 // ------------------------------------------------------------ batched layout
 // Many surfaces concatenated (caller order: surface s owns caller indices
@@ -188,6 +200,9 @@ struct BatchLayout {
     int64_t n_total = 0, n_pad_total = 0;
     std::vector<int64_t> off, n, poff, n_pad;   // host copies
     std::vector<double> delta, wsum;
+    std::vector<Extent> ext;
+    void *fx_geo = nullptr;   // per-surface constants of the fixed-point kernel (in block)
+    int fx_noct = 0;          // octaves of the kernel tables the surfaces need; 0: some surface is out of range
     Layout L;                 // concatenated padded arrays; L.perm maps to caller indices
     int32_t *elem_surf = nullptr;   // [n_total] surface of each caller index
     double *d_wsum = nullptr;       // [nsurf] weight sum per surface

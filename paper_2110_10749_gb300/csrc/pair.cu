@@ -23,6 +23,7 @@
 
 #include "internal.h"
 #include "erfcx_coef.h"
+#include "fx_pair.h"
 #include "series_coef.h"
 
 namespace ssd {
@@ -987,6 +988,8 @@ __global__ void __launch_bounds__(kTPB64) sym64_kernel(const Sym64Args a) {
     }
 }
 
+#include "fx_kernel.h"
+
 // ------------------------------------------------------------------- packing
 // Densities in the layout's order, scaled for the kernel; padding slots zero.
 struct PackArgs {
@@ -1000,6 +1003,7 @@ struct PackArgs {
     int no_weight;            // single layers: pack the density without w (transpose)
     void *out0, *out1;        // float4 or d4 [n_pad]
     double *wdot_part;        // optional: per-block partial of sum w * d0 (Darcy gauge)
+    FxPack fx;                // FP64: what the fixed-point kernel reads beside the records
 };
 
 template <typename V4, typename R>
@@ -1007,9 +1011,9 @@ __global__ void pack_kernel(const PackArgs a) {
     __shared__ double red[256];
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double wd = 0.0;
+    V4 r0 = {R(0), R(0), R(0), R(0)}, r1 = {R(0), R(0), R(0), R(0)};
     if (i < a.n_pad) {
         const int32_t o = a.perm[i];
-        V4 r0 = {R(0), R(0), R(0), R(0)}, r1 = {R(0), R(0), R(0), R(0)};
         if (o >= 0) {
             const double w = a.no_weight ? 1.0 : a.pos64[i].w;
             switch (a.op) {
@@ -1050,6 +1054,9 @@ __global__ void pack_kernel(const PackArgs a) {
         }
         reinterpret_cast<V4 *>(a.out0)[i] = r0;
         if (a.out1) reinterpret_cast<V4 *>(a.out1)[i] = r1;
+    }
+    if constexpr (sizeof(R) == 8) {   // n_pad is a multiple of 512: whole blocks
+        if (a.fx.X) fx_pack(a.fx, i, a.n - 1, a.pos64, a.perm, r0, r1, 0, gridDim.x);
     }
     if (a.wdot_part) {
         red[threadIdx.x] = wd;
@@ -1163,7 +1170,7 @@ __global__ void epilogue_kernel(const EpiArgs a) {
 
 template <int OP>
 cudaError_t launch64(dim3 grid, const KArgs<double> &ka, cudaStream_t s) {
-    pair_kernel<double, OP, kTPB64, kTPT64><<<grid, kTPB64, 0, s>>>(ka);
+    pair_kernel<double, OP, kTPB64, kTPTd><<<grid, kTPB64, 0, s>>>(ka);
     return cudaGetLastError();
 }
 
@@ -1181,8 +1188,9 @@ cudaError_t launch_pair_op64(int op, dim3 grid, const KArgs<double> &ka, cudaStr
 // transposed double layers run on the generic kernel in both precisions
 template <typename R>
 cudaError_t launch_transpose(int op, dim3 grid, const KArgs<R> &ka, cudaStream_t s) {
-    if (op == OP_LDLT) pair_kernel<R, OP_LDLT, kTPB64, kTPT64><<<grid, kTPB64, 0, s>>>(ka);
-    else pair_kernel<R, OP_SDLT, kTPB64, kTPT64><<<grid, kTPB64, 0, s>>>(ka);
+    constexpr int TPT = sizeof(R) == 8 ? kTPTd : kTPT64;
+    if (op == OP_LDLT) pair_kernel<R, OP_LDLT, kTPB64, TPT><<<grid, kTPB64, 0, s>>>(ka);
+    else pair_kernel<R, OP_SDLT, kTPB64, TPT><<<grid, kTPB64, 0, s>>>(ka);
     return cudaGetLastError();
 }
 
@@ -1241,6 +1249,7 @@ struct BPackArgs {
     void *out0, *out1;            // records [nrhs][n_pad]
     double *wdot_part;            // [nrhs][pack blocks]: w (d0 . n) (vector ops) or w d0 (scalar)
     int want_wdot;
+    FxPack fx;                    // FP64: what the fixed-point kernel reads beside the records
 };
 
 template <typename V4, typename R>
@@ -1252,9 +1261,9 @@ __global__ void bpack_kernel(const BPackArgs a) {
     const double *d1 = a.d1 ? a.d1 + (int64_t)r * a.nc1 * a.n_total : nullptr;
     const int64_t n = a.n_total;
     double wd = 0.0;
+    V4 r0 = {R(0), R(0), R(0), R(0)}, r1 = {R(0), R(0), R(0), R(0)};
     if (i < a.n_pad) {
         const int32_t o = a.perm[i];
-        V4 r0 = {R(0), R(0), R(0), R(0)}, r1 = {R(0), R(0), R(0), R(0)};
         if (o >= 0) {
             const double w = a.pos64[i].w;
             switch (a.op) {
@@ -1280,6 +1289,9 @@ __global__ void bpack_kernel(const BPackArgs a) {
         }
         reinterpret_cast<V4 *>(a.out0)[(int64_t)r * a.n_pad + i] = r0;
         if (a.out1) reinterpret_cast<V4 *>(a.out1)[(int64_t)r * a.n_pad + i] = r1;
+    }
+    if constexpr (sizeof(R) == 8) {
+        if (a.fx.X) fx_pack(a.fx, i, 0, a.pos64, a.perm, r0, r1, r, gridDim.x);
     }
     if (a.want_wdot) {
         red[threadIdx.x] = wd;
@@ -1399,16 +1411,16 @@ __global__ void item_cost_kernel(const float4 *cbox, int64_t ntiles_t, int64_t n
 }
 
 // Builds (once per layout, delta and grid) the launch order of the FP32C grid.
-int item_order(ssd_ctx *ctx, const Layout &L, int slot, int tpb, int tpt, int64_t ntiles_t, int64_t nsplit,
+int item_order(ssd_ctx *ctx, const Layout &L, int tpb, int tpt, int64_t ntiles_t, int64_t nsplit,
                int64_t chunk, float rfar2, const int2 **order, cudaStream_t s) {
     Layout &M = const_cast<Layout &>(L);
     const int64_t nit = ntiles_t * nsplit;
-    if (M.order32[slot] && M.order_nit[slot] == nit && M.order_chunk[slot] == chunk &&
-        M.order_rfar2[slot] == rfar2) {
-        *order = M.order32[slot];
+    if (M.order32 && M.order_nit == nit && M.order_chunk == chunk &&
+        M.order_rfar2 == rfar2) {
+        *order = M.order32;
         return SSD_OK;
     }
-    if (M.order32[slot]) { dev_free(ctx, M.order32[slot]); M.order32[slot] = nullptr; }
+    if (M.order32) { dev_free(ctx, M.order32); M.order32 = nullptr; }
     void *keys = nullptr;
     SSD_TRY(dev_alloc(ctx, sizeof(int32_t) * nit, &keys));
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, keys};
@@ -1430,14 +1442,14 @@ int item_order(ssd_ctx *ctx, const Layout &L, int slot, int tpb, int tpt, int64_
     for (int64_t i = 0; i < nit; ++i) ho[start[kmax - hk[i]]++] = make_int2((int)(i % ntiles_t), (int)(i / ntiles_t));
     void *dev = nullptr;
     SSD_TRY(dev_alloc(ctx, sizeof(int2) * nit, &dev));
-    M.order32[slot] = static_cast<int2 *>(dev);
-    SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(M.order32[slot], ho.data(), sizeof(int2) * nit, cudaMemcpyHostToDevice,
+    M.order32 = static_cast<int2 *>(dev);
+    SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(M.order32, ho.data(), sizeof(int2) * nit, cudaMemcpyHostToDevice,
                                             s), "order copy"));
     SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "order sync"));
-    M.order_nit[slot] = nit;
-    M.order_chunk[slot] = chunk;
-    M.order_rfar2[slot] = rfar2;
-    *order = M.order32[slot];
+    M.order_nit = nit;
+    M.order_chunk = chunk;
+    M.order_rfar2 = rfar2;
+    *order = M.order32;
     return SSD_OK;
 }
 
@@ -1448,8 +1460,8 @@ int item_order(ssd_ctx *ctx, const Layout &L, int slot, int tpb, int tpt, int64_
 // goes to the symmetric kernel, in items of the target block against at most
 // kSymTiles source tiles; the diagonal blocks and the near block pairs (both
 // directions) are items of the pair kernel of the precision (slot 0:
-// pair32_kernel, one item of 512 targets; slot 1: the generic FP64 kernel,
-// four items of 128 targets).  The plan is used when far pairs are at least
+// pair32_kernel, one item of 512 targets; slot 1: the fixed-point or the
+// generic FP64 kernel, two items of 256 targets).  The plan is used when far pairs are at least
 // half of all pairs.  The device block holds the surface descriptor, the
 // kernel constants (`cbytes` bytes at `consts`), the near and the far items.
 int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *consts, size_t cbytes,
@@ -1460,7 +1472,7 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
     if (pl.block) { dev_free(ctx, pl.block); pl.block = nullptr; }
     pl.use = false;
     pl.near = pl.far = 0;
-    const int nsub = slot == 0 ? 1 : kSymBlock / (kTPB64 * kTPT64);   // near items per block pair
+    const int nsub = slot == 0 ? 1 : kSymBlock / kFxTPB;   // near items per block pair
     const int sub = kSymBlock / nsub;
     const int64_t n = L.n, n_pad = L.n_pad, nb = n_pad / kSymBlock, nch = n_pad / kChunk;
     std::vector<float4> cb(2 * nch);
@@ -1572,7 +1584,7 @@ cudaError_t launch_sym(const Layout &L, const float4 *d0, double *acc, cudaStrea
 }
 
 template <int OP>
-cudaError_t launch_sym64(const Layout &L, const d4 *d0, double *acc, cudaStream_t s) {
+cudaError_t launch_sym64(const Layout &L, const d4 *d0, double *acc, FxArgs *fx, cudaStream_t s) {
     const SymPlan &pl = L.sym[1];
     char *b = static_cast<char *>(pl.block);
     size_t off = 0;
@@ -1589,8 +1601,13 @@ cudaError_t launch_sym64(const Layout &L, const d4 *d0, double *acc, cudaStream_
     ka.consts = reinterpret_cast<const Consts<double> *>(b + o_c);
     ka.rec_stride = 0; ka.part_stride = 0;
     ka.acc = acc;
-    pair_kernel<double, OP, kTPB64, kTPT64><<<dim3((unsigned)pl.near, 1), kTPB64, 0, s>>>(ka);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e;
+    if (fx) {
+        fx->k = ka;
+        e = launch_fx1<OP>(dim3((unsigned)pl.near, 1), *fx, s);
+    } else {
+        e = launch64<OP>(dim3((unsigned)pl.near, 1), ka, s);
+    }
     if (e != cudaSuccess || pl.far == 0) return e;
     Sym64Args sa;
     sa.pos = L.pos64; sa.wn = L.wn64; sa.d0 = d0;
@@ -1604,12 +1621,27 @@ int pair_occupancy(ssd_ctx *ctx) {
     int o32 = 0, o64 = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o32, pair32_kernel<OP_SSLDL>, kTPB32, 0);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o64, pair_kernel<double, OP_SSLDL, kTPB64, kTPT64>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o64, pair_kernel<float, OP_SDLT, kTPB64, kTPT64>,
                                                           kTPB64, 0);
     if (e != cudaSuccess) return cuda_check(ctx, e, "occupancy query");
     ctx->occ32 = o32 > 0 ? o32 : 1;
     ctx->occ64 = o64 > 0 ? o64 : 1;
-    return SSD_OK;
+    return fx_init(ctx);
+}
+
+size_t fx_geo_bytes(int nsurf) { return sizeof(FxGeo) * nsurf; }
+
+// Source split of the fixed-point grid: every tile costs the same, so the
+// grid only has to fill the GPU evenly; splits are multiples of 32 sources.
+static int64_t fx_chunk(const ssd_ctx *ctx, int64_t n, int64_t ntiles_t, int64_t *nsplit) {
+    const int64_t units = (n + kChunk - 1) / kChunk;
+    const int64_t want = (int64_t)ctx->num_sms * 2 * ctx->waves_fx;
+    int64_t ns = (want + ntiles_t - 1) / ntiles_t;
+    if (ns < 1) ns = 1;
+    if (ns > units) ns = units;
+    const int64_t cu = (units + ns - 1) / ns;
+    *nsplit = (units + cu - 1) / cu;
+    return cu * kChunk;
 }
 
 int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s) {
@@ -1619,8 +1651,12 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     const int64_t n = L.n, n_pad = L.n_pad;
     const bool transposed = (op == OP_LDLT || op == OP_SDLT);
     const bool packed32 = f32 && !transposed;    // the packed FP32 kernel, else the generic one
-    const int tspan = packed32 ? kTPB32 * kTPT32 : kTPB64 * kTPT64;
-    const int64_t ntiles_t = n_pad / tspan;
+    // FP64: fixed point unless the point set is out of its range
+    FxGeo geo;
+    int noct = 0;
+    const bool use_fx = !f32 && fx_geo(L.ext, pc.delta, &geo, &noct);
+    const int tspan = packed32 ? kTPB32 * kTPT32 : (f32 ? kTPB64 * kTPT64 : kFxTPB);
+    const int64_t ntiles_t = use_fx ? (n + tspan - 1) / tspan : n_pad / tspan;
     const int64_t ntiles_s = n_pad / kTile;
     // splits: enough CTAs for several waves of resident CTAs, so that the
     // uneven cost of near and far target tiles evens out (FP32C: tuned on the
@@ -1632,7 +1668,8 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     if (nsplit > ntiles_s) nsplit = ntiles_s;
     const int64_t chunk_tiles = (ntiles_s + nsplit - 1) / nsplit;
     nsplit = (ntiles_s + chunk_tiles - 1) / chunk_tiles;
-    const int64_t chunk = chunk_tiles * kTile;
+    int64_t chunk = chunk_tiles * kTile;
+    if (use_fx) chunk = fx_chunk(ctx, n, ntiles_t, &nsplit);
 
     const size_t rec = f32 ? sizeof(float4) : sizeof(d4);
     // FP32C keeps a (hi, lo) pair per target and split; one slot suffices when
@@ -1664,6 +1701,9 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         use_sym = L.sym[f32 ? 0 : 1].use;
     }
     const size_t o_acc = use_sym ? carve(sizeof(double) * nc * n_pad) : 0;
+    const size_t o_fx = use_fx ? carve(sizeof(l4) * n_pad) : 0;
+    const size_t o_fxb = use_fx ? carve(sizeof(int4) * 2 * (n_pad / kChunk)) : 0;
+    const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks) : 0;
     void *ws = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &ws));
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, ws};
@@ -1701,6 +1741,18 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     pa.no_weight = tsl ? 1 : 0;
     const bool rank1 = pc.rank1_weight_mean || pc.rank1_nrm != nullptr;
     pa.wdot_part = rank1 ? reinterpret_cast<double *>(base + o_wdot) : nullptr;
+    FxArgs fa{};
+    if (use_fx) {
+        pa.fx.X = reinterpret_cast<l4 *>(base + o_fx);
+        pa.fx.cbox = reinterpret_cast<int4 *>(base + o_fxb);
+        pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
+        pa.fx.geo = geo;
+        pa.fx.two = op == OP_LSLDL ? 1 : 0;
+        fa.X = pa.fx.X; fa.cbox = pa.fx.cbox; fa.bmax = pa.fx.bmax;
+        fa.nblk = pack_blocks; fa.tab = static_cast<const FxI4 *>(ctx->fx_tab); fa.noct = noct;
+        fa.geo = geo; fa.geos = nullptr; fa.n = n;
+        self_src = nullptr;    // the self pair is part of the sum
+    }
     if (f32) pack_kernel<float4, float><<<pack_blocks, 256, 0, s>>>(pa);
     else pack_kernel<d4, double><<<pack_blocks, 256, 0, s>>>(pa);
     ctx->launches++;
@@ -1734,10 +1786,10 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     } else if (use_sym) {
         const d4 *d0 = reinterpret_cast<const d4 *>(base + o_d0);
         switch (op) {
-            case OP_SDL: e = launch_sym64<OP_SDL>(L, d0, acc, s); break;
-            case OP_LDL: e = launch_sym64<OP_LDL>(L, d0, acc, s); break;
-            case OP_SSL: e = launch_sym64<OP_SSL>(L, d0, acc, s); break;
-            default: e = launch_sym64<OP_LSL>(L, d0, acc, s); break;
+            case OP_SDL: e = launch_sym64<OP_SDL>(L, d0, acc, use_fx ? &fa : nullptr, s); break;
+            case OP_LDL: e = launch_sym64<OP_LDL>(L, d0, acc, use_fx ? &fa : nullptr, s); break;
+            case OP_SSL: e = launch_sym64<OP_SSL>(L, d0, acc, use_fx ? &fa : nullptr, s); break;
+            default: e = launch_sym64<OP_LSL>(L, d0, acc, use_fx ? &fa : nullptr, s); break;
         }
         if (L.sym[1].far) ctx->launches++;
     } else if (f32 && transposed) {
@@ -1765,7 +1817,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         dim3 g = grid;
         if (ctx->lpt && L.order_ok && !rows) {
             const int2 *ord = nullptr;
-            const int st = item_order(ctx, L, 0, kTPB32, kTPT32, ntiles_t, nsplit, chunk, ka.c.rfar2, &ord, s);
+            const int st = item_order(ctx, L, kTPB32, kTPT32, ntiles_t, nsplit, chunk, ka.c.rfar2, &ord, s);
             if (st != SSD_OK) return st;
             ka.order = ord;
             g = dim3((unsigned)(ntiles_t * nsplit), 1);
@@ -1781,16 +1833,12 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         ka.part = reinterpret_cast<double *>(base + o_part);
         ka.items = nullptr; ka.surfs = nullptr; ka.consts = nullptr; ka.rec_stride = 0; ka.part_stride = 0;
         ka.tile0 = tile0;
-        dim3 g = grid;
-        if (ctx->lpt && L.order_ok && !rows) {
-            const int2 *ord = nullptr;
-            const int st = item_order(ctx, L, 1, kTPB64, kTPT64, ntiles_t, nsplit, chunk,
-                                      (float)ka.c.rfar2, &ord, s);
-            if (st != SSD_OK) return st;
-            ka.order = ord;
-            g = dim3((unsigned)(ntiles_t * nsplit), 1);
+        if (use_fx) {
+            fa.k = ka;
+            e = launch_fx(op, grid, fa, s);
+        } else {
+            e = transposed ? launch_transpose<double>(op, grid, ka, s) : launch_pair_op64(op, grid, ka, s);
         }
-        e = transposed ? launch_transpose<double>(op, g, ka, s) : launch_pair_op64(op, g, ka, s);
     }
     ctx->launches++;
     if (e != cudaSuccess) return cuda_check(ctx, e, "pair kernel launch");
@@ -1850,30 +1898,46 @@ __global__ void batch_item_cost_kernel(const BItem *items, int64_t nitems, const
 
 int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
     const int ns = B->nsurf;
+    // FP64 runs in fixed point when every surface is in its range
+    std::vector<FxGeo> geos(ns);
+    B->fx_noct = 0;
+    for (int k = 0; k < ns; ++k) {
+        int noct = 0;
+        if (!fx_geo(B->ext[k], B->delta[k], &geos[k], &noct)) { B->fx_noct = 0; break; }
+        B->fx_noct = noct > B->fx_noct ? noct : B->fx_noct;
+    }
+    SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(B->fx_geo, geos.data(), sizeof(FxGeo) * ns, cudaMemcpyHostToDevice, s),
+                       "surface constants copy"));
     for (int pr = 0; pr < 2; ++pr) {   // 0: FP32C, 1: FP64
-        const int span = pr == 0 ? kTPB32 * kTPT32 : kTPB64 * kTPT64;
+        const bool fx = pr == 1 && B->fx_noct > 0;
+        const int64_t unit = fx ? kChunk : kTile;   // sources come in multiples of this
+        // fixed point: real targets and sources only
+        auto ntt = [&](int k, int span) { return fx ? (B->n[k] + span - 1) / span : B->n_pad[k] / span; };
+        auto nss = [&](int k) { return fx ? (B->n[k] + unit - 1) / unit : B->n_pad[k] / unit; };
+        const int span = pr == 0 ? kTPB32 * kTPT32 : kFxTPB;
         const int occ = pr == 0 ? ctx->occ32 : ctx->occ64;
-        const int64_t want = (int64_t)ctx->num_sms * occ * (pr == 0 ? ctx->waves32 : 2);
-        // source chunk (multiple of kTile) common to all surfaces: about `want` items
+        const int64_t want = fx ? (int64_t)ctx->num_sms * 2 * ctx->waves_fx
+                                : (int64_t)ctx->num_sms * occ * (pr == 0 ? ctx->waves32 : 2);
+        // source chunk (multiple of the unit) common to all surfaces: about `want` items
         int64_t pairs_tiles = 0;
-        for (int k = 0; k < ns; ++k) pairs_tiles += (B->n_pad[k] / span) * (B->n_pad[k] / kTile);
+        for (int k = 0; k < ns; ++k) pairs_tiles += ntt(k, span) * nss(k);
         int64_t chunk_tiles = pairs_tiles / want;
         if (chunk_tiles < 1) chunk_tiles = 1;
         std::vector<BItem> items;
         std::vector<BSurf> surfs(ns);
         int64_t pb = 0;
         for (int k = 0; k < ns; ++k) {
-            const int64_t nts = B->n_pad[k] / kTile;
+            const int64_t nts = nss(k);
             const int64_t ct = chunk_tiles < nts ? chunk_tiles : nts;
             const int64_t nsplit = (nts + ct - 1) / ct;
             surfs[k] = BSurf{B->poff[k], B->n_pad[k], B->n[k], pb, nsplit, 0, 0, 0};
-            for (int64_t t = 0; t < B->n_pad[k] / span; ++t)
+            for (int64_t t = 0; t < ntt(k, span); ++t)
                 for (int64_t sp = 0; sp < nsplit; ++sp) {
                     BItem it;
                     it.tbase = (int32_t)(B->poff[k] + t * span);
-                    it.s_beg = (int32_t)(B->poff[k] + sp * ct * kTile);
-                    int64_t e = B->poff[k] + (sp + 1) * ct * kTile;
-                    if (e > B->poff[k] + B->n_pad[k]) e = B->poff[k] + B->n_pad[k];
+                    it.s_beg = (int32_t)(B->poff[k] + sp * ct * unit);
+                    int64_t e = B->poff[k] + (sp + 1) * ct * unit;
+                    if (e > B->poff[k] + nts * unit) e = B->poff[k] + nts * unit;
                     it.s_end = (int32_t)e;
                     it.surf = k;
                     it.split = (int32_t)sp;
@@ -1966,6 +2030,10 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
     const size_t o_part = carve(rsz * part_stride * nrhs);
     const size_t o_wdot = carve(sizeof(double) * pack_blocks * nrhs);
     const size_t o_r1 = carve(sizeof(double) * B.nsurf * nrhs);
+    const bool use_fx = !f32 && B.fx_noct > 0;
+    const size_t o_fx = use_fx ? carve(sizeof(l4) * n_pad) : 0;
+    const size_t o_fxb = use_fx ? carve(sizeof(int4) * 2 * (n_pad / kChunk)) : 0;
+    const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks * nrhs) : 0;
     void *ws = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &ws));
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, ws};
@@ -1999,6 +2067,20 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
     pa.out0 = base + o_d0; pa.out1 = two_rec ? base + o_d1 : nullptr;
     pa.wdot_part = reinterpret_cast<double *>(base + o_wdot);
     pa.want_wdot = rank1 ? 1 : 0;
+    FxArgs fa{};
+    if (use_fx) {
+        pa.fx.X = reinterpret_cast<l4 *>(base + o_fx);
+        pa.fx.cbox = reinterpret_cast<int4 *>(base + o_fxb);
+        pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
+        pa.fx.geos = static_cast<const FxGeo *>(B.fx_geo);
+        pa.fx.surfs = reinterpret_cast<const BSurf *>(B.surfs[pr]);
+        pa.fx.nsurf = B.nsurf;
+        pa.fx.two = op == OP_LSLDL ? 1 : 0;
+        fa.X = pa.fx.X; fa.cbox = pa.fx.cbox; fa.bmax = pa.fx.bmax;
+        fa.nblk = pack_blocks; fa.tab = static_cast<const FxI4 *>(ctx->fx_tab); fa.noct = B.fx_noct;
+        fa.geos = pa.fx.geos; fa.n = n_pad;
+        self_src = nullptr;    // the self pair is part of the sum
+    }
     const dim3 pg((unsigned)pack_blocks, (unsigned)nrhs);
     if (f32) bpack_kernel<float4, float><<<pg, 256, 0, s>>>(pa);
     else bpack_kernel<d4, double><<<pg, 256, 0, s>>>(pa);
@@ -2041,7 +2123,12 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
         ka.surfs = reinterpret_cast<const BSurf *>(B.surfs[pr]);
         ka.consts = reinterpret_cast<const Consts<double> *>(B.consts[pr]);
         ka.rec_stride = n_pad; ka.part_stride = part_stride;
-        e = launch_pair_op64(op, grid, ka, s);
+        if (use_fx) {
+            fa.k = ka;
+            e = launch_fx(op, grid, fa, s);
+        } else {
+            e = launch_pair_op64(op, grid, ka, s);
+        }
     }
     ctx->launches++;
     if (e != cudaSuccess) return cuda_check(ctx, e, "batched pair kernel launch");
