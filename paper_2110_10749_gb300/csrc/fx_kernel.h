@@ -141,9 +141,22 @@ __device__ __noinline__ void fx_fallback(const KArgs<double> *ap, const Consts<d
     out[0] = acc[0]; out[1] = acc[1]; out[2] = acc[2];
 }
 
-template <int OP>
+// FAR: all items are block pairs at least 8 delta apart (the second launch of a
+// plan).  Only the octaves from there on are staged, and the Stokes single
+// layer takes sigma_3 from sigma_1: one table of noct - 6 octaves instead of two
+// of noct.  Stokes single layer at N = 68166: 58.9 ms with the plan against 64.9
+// with every tile on the general kernel; the other layers gain 1-2%.  (The
+// double-precision symmetric kernel that ran the far pairs before took 154 of
+// the 164 ms of this operator at N = 78106; both directions in fixed point take
+// it to 76 ms.)
+constexpr int kFxFarOct = 6;                     // 1 + 8^2 > 2^6
+template <int OP, bool FAR> constexpr int fx_ntab() { return FAR && OP == OP_SSL ? 1 : FxOp<OP>::ntab; }
+
+template <int OP, bool FAR>
 __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ FxArgs a) {
     typedef FxOp<OP> T;
+    constexpr int kOct0 = FAR ? kFxFarOct : 0;
+    const int tstride = (a.noct - kOct0) * kFxSeg * kFxEntry;
     constexpr int NC = OpInfo<OP>::NC;
     constexpr bool M = T::dl, VU = T::dl && T::vec, VF = T::sl && T::vec;
     extern __shared__ __align__(16) FxI4 s_tab[];           // [ntab][noct * kFxSeg][kFxEntry]
@@ -193,10 +206,11 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
         }
         if (lane == 0) { s_max[0][warp] = m0; s_max[1][warp] = m1; }
     }
-    for (int k = 0; k < T::ntab; ++k) {
-        const int4 *src = reinterpret_cast<const int4 *>(a.tab) + (int64_t)T::tab(k) * kFxMaxOct * kFxSeg * kFxEntry;
-        int4 *dst = reinterpret_cast<int4 *>(s_tab) + (int64_t)k * a.noct * kFxSeg * kFxEntry;
-        for (int q = threadIdx.x; q < a.noct * kFxSeg * kFxEntry; q += kFxTPB) dst[q] = src[q];
+    for (int k = 0; k < fx_ntab<OP, FAR>(); ++k) {
+        const int4 *src = reinterpret_cast<const int4 *>(a.tab) +
+                          ((int64_t)T::tab(k) * kFxMaxOct + kOct0) * kFxSeg * kFxEntry;
+        int4 *dst = reinterpret_cast<int4 *>(s_tab) + (int64_t)k * tstride;
+        for (int q = threadIdx.x; q < tstride; q += kFxTPB) dst[q] = src[q];
     }
     __syncthreads();
     int ee[2];
@@ -240,9 +254,8 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
             tlo[0] = min(tlo[0], l.x); tlo[1] = min(tlo[1], l.y); tlo[2] = min(tlo[2], l.z);
             thi[0] = max(thi[0], h.x); thi[1] = max(thi[1], h.y); thi[2] = max(thi[2], h.z);
         }
-        const uint32_t idx_max = (uint32_t)(a.noct * kFxSeg - 1);
+        const uint32_t idx_max = (uint32_t)((a.noct - kOct0) * kFxSeg - 1);
         const int4 *tab4 = reinterpret_cast<const int4 *>(s_tab);
-        const int tstride = a.noct * kFxSeg * kFxEntry;
         auto tab = [&](int k, uint32_t idx, int w) {
             const int4 v = tab4[k * tstride + idx * kFxEntry + w];
             return FxI4{v.x, v.y, v.z, v.w};
@@ -267,7 +280,8 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
             // distances < dmax 2^(32 - ps) <= 2^L, >= gap 2^(32 - ps) >= 2^r
             const int L = max(0, 32 - g.ps + (32 - __clz(dmax - 1)));
             const int r = gap > 0 ? max(0, 31 - __clz(gap) + 32 - g.ps) : 0;
-            const FxTile tl = fx_tile<OP>(sc, L, r);
+            FxTile tl = fx_tile<OP>(sc, L, r);
+            tl.oct0 -= kOct0 * kFxSeg;
             const int ks = 61 - L - g.ps;
             auto grid = [&](int64_t v) { return ks >= 0 ? (int64_t)((uint64_t)v << ks) : v >> -ks; };
             __syncthreads();
@@ -343,7 +357,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
                 }
                 if constexpr (VU) vec(x.u, s_uh[j], s_ul[j]);
                 if constexpr (VF) vec(x.f, s_fh[j], s_fl[j]);
-                fx_pair<OP>(y, x, tl, sc, idx_max, tab, acc);
+                fx_pair<OP, FAR>(y, x, tl, sc, idx_max, tab, acc);
             }
             const double f = __longlong_as_double((long long)(1023 + tl.ex) << 52) *
                              (T::fused || !T::dl ? g.f_sl : g.f_dl);
@@ -405,12 +419,12 @@ bool fx_geo(const Extent &e, double delta, FxGeo *g, int *noct) {
     return true;
 }
 
-template <int OP> size_t fx_smem(int noct) {
-    return (size_t)FxOp<OP>::ntab * noct * kFxSeg * kFxEntry * sizeof(FxI4);
+template <int OP, bool FAR> size_t fx_smem(int noct) {
+    return (size_t)fx_ntab<OP, FAR>() * (noct - (FAR ? kFxFarOct : 0)) * kFxSeg * kFxEntry * sizeof(FxI4);
 }
 
-template <int OP> cudaError_t launch_fx1(dim3 grid, const FxArgs &a, cudaStream_t s) {
-    fx_kernel<OP><<<grid, kFxTPB, fx_smem<OP>(a.noct), s>>>(a);
+template <int OP, bool FAR = false> cudaError_t launch_fx1(dim3 grid, const FxArgs &a, cudaStream_t s) {
+    fx_kernel<OP, FAR><<<grid, kFxTPB, fx_smem<OP, FAR>(a.noct), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -427,8 +441,9 @@ cudaError_t launch_fx(int op, dim3 grid, const FxArgs &a, cudaStream_t s) {
     }
 }
 
-template <int OP> cudaError_t fx_attr1() {
-    return cudaFuncSetAttribute(fx_kernel<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx_smem<OP>(kFxMaxOct));
+template <int OP, bool FAR = false> cudaError_t fx_attr1() {
+    return cudaFuncSetAttribute(fx_kernel<OP, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)fx_smem<OP, FAR>(kFxMaxOct));
 }
 
 // Uploads the kernel tables of a context and lets the kernels use them.
@@ -444,5 +459,9 @@ int fx_init(ssd_ctx *ctx) {
     if (e == cudaSuccess) e = fx_attr1<OP_LSLDL>();
     if (e == cudaSuccess) e = fx_attr1<OP_LDLT>();
     if (e == cudaSuccess) e = fx_attr1<OP_SDLT>();
+    if (e == cudaSuccess) e = fx_attr1<OP_LSL, true>();
+    if (e == cudaSuccess) e = fx_attr1<OP_LDL, true>();
+    if (e == cudaSuccess) e = fx_attr1<OP_SSL, true>();
+    if (e == cudaSuccess) e = fx_attr1<OP_SDL, true>();
     return cuda_check(ctx, e, "kernel attributes");
 }

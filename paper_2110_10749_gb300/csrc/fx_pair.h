@@ -76,8 +76,10 @@ template <int OP> FX_HD FxTile fx_tile(const FxScale &s, int L, int r) {
 
 template <int OP> struct FxSum { FxMac v[FxOp<OP>::vec ? 3 : 1]; FxF f; };
 
+// FAR: every pair of the tile has rho >= 8, where sigma_3 = sigma_1^3 (bare
+// kernels): the Stokes single layer then needs one table instead of two.
 // tab(k, idx, w): word w of entry idx of staged table k
-template <int OP, typename Tab>
+template <int OP, bool FAR, typename Tab>
 FX_HD void fx_pair(const FxPoint<OP> &y, const FxPoint<OP> &x, const FxTile &t, const FxScale &s, uint32_t idx_max,
                    const Tab &tab, FxSum<OP> &acc) {
     typedef FxOp<OP> T;
@@ -87,7 +89,12 @@ FX_HD void fx_pair(const FxPoint<OP> &y, const FxPoint<OP> &x, const FxTile &t, 
     const uint32_t idx = a.idx < idx_max ? a.idx : idx_max;
     FxQ K1, K3, KD;
     if constexpr (T::k1 >= 0) K1 = fx_poly<fx_unit(0)>(tab(T::k1, idx, 0), tab(T::k1, idx, 1), tab(T::k1, idx, 2), a.sh, a.sl);
-    if constexpr (T::k3 >= 0) K3 = fx_poly<fx_unit(2)>(tab(T::k3, idx, 0), tab(T::k3, idx, 1), tab(T::k3, idx, 2), a.sh, a.sl);
+    if constexpr (T::k3 >= 0 && FAR) {
+        K3.m = fx_mul(fx_mul(K1.m, K1.m), K1.m);   // (m 2^-(61+e))^3 in units of 2^-(61 + e3)
+        K3.e = 3 * K1.e - 2;
+    } else if constexpr (T::k3 >= 0) {
+        K3 = fx_poly<fx_unit(2)>(tab(T::k3, idx, 0), tab(T::k3, idx, 1), tab(T::k3, idx, 2), a.sh, a.sl);
+    }
     if constexpr (T::kd >= 0)
         KD = fx_poly<fx_unit(T::vec ? 3 : 1)>(tab(T::kd, idx, 0), tab(T::kd, idx, 1), tab(T::kd, idx, 2), a.sh, a.sl);
     if constexpr (!T::vec) {

@@ -1464,7 +1464,9 @@ int item_order(ssd_ctx *ctx, const Layout &L, int tpb, int tpt, int64_t ntiles_t
 // generic FP64 kernel, two items of 256 targets).  The plan is used when far pairs are at least
 // half of all pairs.  The device block holds the surface descriptor, the
 // kernel constants (`cbytes` bytes at `consts`), the near and the far items.
-int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *consts, size_t cbytes,
+// `ordered` (the fixed-point FP64 kernels): the far list holds items of the
+// pair kernel as the near one does, in both directions.
+int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *consts, size_t cbytes, bool ordered,
              cudaStream_t s) {
     Layout &M = const_cast<Layout &>(L);
     SymPlan &pl = M.sym[slot];
@@ -1499,9 +1501,24 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
         }
         return g2 >= rfar2;
     };
-    std::vector<BItem> near;
+    std::vector<BItem> near, far2;
     std::vector<SymItem> far;
     int64_t far_blocks = 0;
+    if (ordered)   // runs of far blocks of every target block, both directions
+        for (int64_t i = 0; i < nb; ++i)
+            for (int64_t k = 0; k < nb;) {
+                if (k == i || !far_pair(i, k) || k * kSymBlock >= n) { ++k; continue; }
+                int64_t k1 = k;
+                while (k1 < nb && k1 != i && far_pair(i, k1) && k1 * kSymBlock < n) ++k1;
+                for (int64_t t = k * kSymBlock; t < k1 * kSymBlock; t += (int64_t)kSymTiles * kTile) {
+                    int64_t e = t + (int64_t)kSymTiles * kTile;
+                    if (e > k1 * kSymBlock) e = k1 * kSymBlock;
+                    for (int q = 0; q < nsub; ++q)
+                        if (i * kSymBlock + q * sub < n)
+                            far2.push_back(BItem{(int32_t)(i * kSymBlock + q * sub), (int32_t)t, (int32_t)e, 0, 0, 0, 0, 0});
+                }
+                k = k1;
+            }
     auto near_item = [&](int64_t ti, int64_t si) {   // targets of block ti against sources of block si
         for (int q = 0; q < nsub; ++q)
             near.push_back(BItem{(int32_t)(ti * kSymBlock + q * sub), (int32_t)(si * kSymBlock),
@@ -1534,7 +1551,8 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
     size_t off = 0;
     auto carve = [&](size_t b) { size_t o = off; off += (b + 255) & ~size_t(255); return o; };
     const size_t o_surf = carve(sizeof(BSurf)), o_c = carve(cbytes);
-    const size_t o_near = carve(sizeof(BItem) * near.size()), o_far = carve(sizeof(SymItem) * far.size());
+    const size_t o_near = carve(sizeof(BItem) * near.size()),
+                 o_far = carve(ordered ? sizeof(BItem) * far2.size() : sizeof(SymItem) * far.size());
     void *blk = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &blk));
     char *b = static_cast<char *>(blk);
@@ -1543,13 +1561,14 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
     memcpy(host.data() + o_surf, &sf, sizeof(sf));
     memcpy(host.data() + o_c, consts, cbytes);
     memcpy(host.data() + o_near, near.data(), sizeof(BItem) * near.size());
-    memcpy(host.data() + o_far, far.data(), sizeof(SymItem) * far.size());
+    if (ordered) memcpy(host.data() + o_far, far2.data(), sizeof(BItem) * far2.size());
+    else memcpy(host.data() + o_far, far.data(), sizeof(SymItem) * far.size());
     const int st = cuda_check(ctx, cudaMemcpyAsync(b, host.data(), off, cudaMemcpyHostToDevice, s), "plan copy");
     if (st == SSD_OK) SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "plan sync"));
     if (st != SSD_OK) { dev_free(ctx, blk); return st; }
     pl.block = blk;
     pl.near = (int64_t)near.size();
-    pl.far = (int64_t)far.size();
+    pl.far = ordered ? (int64_t)far2.size() : (int64_t)far.size();
     pl.use = true;
     return SSD_OK;
 }
@@ -1609,6 +1628,10 @@ cudaError_t launch_sym64(const Layout &L, const d4 *d0, double *acc, FxArgs *fx,
         e = launch64<OP>(dim3((unsigned)pl.near, 1), ka, s);
     }
     if (e != cudaSuccess || pl.far == 0) return e;
+    if (fx) {
+        fx->k.items = reinterpret_cast<const BItem *>(b + o_far);
+        return launch_fx1<OP, true>(dim3((unsigned)pl.far, 1), *fx, s);
+    }
     Sym64Args sa;
     sa.pos = L.pos64; sa.wn = L.wn64; sa.d0 = d0;
     sa.items = reinterpret_cast<const SymItem *>(b + o_far);
@@ -1693,10 +1716,10 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         L.order_ok) {
         if (f32) {
             const Consts<float> c = make_consts<float>(pc.delta, kRhoFar32);
-            SSD_TRY(sym_plan(ctx, L, 0, c.rfar2, &c, sizeof(c), s));
+            SSD_TRY(sym_plan(ctx, L, 0, c.rfar2, &c, sizeof(c), false, s));
         } else {
             const Consts<double> c = make_consts<double>(pc.delta, kRhoFar64);
-            SSD_TRY(sym_plan(ctx, L, 1, c.rfar2, &c, sizeof(c), s));
+            SSD_TRY(sym_plan(ctx, L, 1, c.rfar2, &c, sizeof(c), use_fx, s));
         }
         use_sym = L.sym[f32 ? 0 : 1].use;
     }
