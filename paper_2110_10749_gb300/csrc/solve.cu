@@ -186,6 +186,213 @@ __global__ void givens_kernel(double *H, int ldh, double *cs, double *sn, double
     for (int i = t; i <= j + 1; i += blockDim.x) hc[i] = col[i];
 }
 
+// One Arnoldi step in one cooperative launch: Gram-Schmidt against v_0 .. v_j
+// (w . w from the same sweep), the DGKS test, a second pass when it asks for
+// one, the norm, the Givens update and the scaling of v_{j+1}.  The separate
+// kernels of a step are 11 launches of 3-4 us each, most of them waiting on
+// latency; here the phases meet at grid barriers (about 1.5 us).  A block owns
+// `rows` rows and keeps them in shared memory; sums over the blocks are taken
+// by every block in the same order, so all hold the same h.  Four threads per
+// row share the vectors of an update; a warp takes whole vectors of a dot.
+// Time of an FP32C GMRES step outside its pair kernel: 49 us against 94 with
+// separate kernels at n = 6500, 57 against 100 at 26000, 73 against 118 at
+// 104000; longer vectors keep the separate kernels (kArnMaxN).
+constexpr int kArnTPB = 256;
+constexpr int kArnRows = 64;       // rows per block step: few, for FP64 adds are slow (1.6 per clock and SM)
+constexpr int kArnMaxRows = 1024;  // rows of a block
+constexpr int64_t kArnMaxN = 155648;   // vectors up to this length
+
+struct ArnoldiArgs {
+    double *V;            // [j + 2][n]; w = V + (j + 1) n holds A v_j
+    int64_t n;
+    int j, rows, ldh;
+    double *H, *cs, *sn, *g;
+    double *partial;      // [3][(j + 2) * gridDim.x]
+    unsigned *bar;        // three counters of this step, zero at launch
+    double *out;          // pinned host: residual estimate, norm
+};
+
+// Grid barrier with a bounded wait (every block is resident: cooperative
+// launch).  Returns false when the wait ran out.
+__device__ bool grid_barrier(unsigned *bar) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        int good = 0;
+        for (int it = 0; it < (1 << 22); ++it) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar));
+            if (v >= gridDim.x) { good = 1; break; }
+        }
+        __threadfence();
+        ok = good;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+__global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
+    __shared__ double w[kArnMaxRows], h1[kMaxRestart + 2], h2[kMaxRestart + 2];
+    __shared__ double al[2][kMaxRestart], be[2][kMaxRestart];
+    __shared__ double s_red[kArnTPB / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j = a.j;
+    const int64_t row0 = (int64_t)blockIdx.x * a.rows;
+    const int nr = (int)(a.n - row0 < a.rows ? a.n - row0 : a.rows);   // may be <= 0 (no rows)
+    double *wg = a.V + (int64_t)(j + 1) * a.n + row0;
+    for (int r = tid; r < nr; r += kArnTPB) w[r] = wg[r];
+    __syncthreads();
+    const double *Vb = a.V + row0;
+    // partial[v][block] = V[v] . w over the block's rows, v < nv (v = j + 1: w . w)
+    auto dots = [&](double *partial, int nv) {
+        for (int v = warp; v < nv; v += kArnTPB / 32) {
+            const double *x = Vb + (int64_t)v * a.n;
+            double s0 = 0.0, s1 = 0.0;
+            int r = lane;
+            if (v == j + 1) {
+                for (; r < nr; r += 32) s0 = fma(w[r], w[r], s0);
+            } else {
+                for (; r + 32 < nr; r += 64) {
+                    s0 = fma(x[r], w[r], s0);
+                    s1 = fma(x[r + 32], w[r + 32], s1);
+                }
+                if (r < nr) s0 = fma(x[r], w[r], s0);
+            }
+            double t = s0 + s1;
+            for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+            if (lane == 0) partial[(int64_t)v * gridDim.x + blockIdx.x] = t;
+        }
+    };
+    auto gather = [&](const double *partial, int nv, double *h) {
+        for (int v = warp; v < nv; v += kArnTPB / 32) {
+            double t = 0.0;
+            for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(partial + (int64_t)v * gridDim.x + b);
+            for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+            if (lane == 0) h[v] = t;
+        }
+        __syncthreads();
+    };
+    auto update = [&](const double *h) {
+        const int q = tid & 3;
+        for (int r0 = 0; r0 < nr; r0 += kArnTPB / 4) {
+            const int r = r0 + (tid >> 2);
+            double s0 = 0.0, s1 = 0.0;
+            if (r < nr) {
+                int v = q;
+                for (; v + 4 <= j; v += 8) {
+                    s0 = fma(h[v], Vb[(int64_t)v * a.n + r], s0);
+                    s1 = fma(h[v + 4], Vb[(int64_t)(v + 4) * a.n + r], s1);
+                }
+                if (v <= j) s0 = fma(h[v], Vb[(int64_t)v * a.n + r], s0);
+            }
+            double t = s0 + s1;
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            if (q == 0 && r < nr) w[r] -= t;
+        }
+        __syncthreads();
+    };
+    double *p0 = a.partial, *p1 = p0 + (int64_t)(j + 2) * gridDim.x, *p2 = p1 + (int64_t)(j + 2) * gridDim.x;
+    bool ok = true;
+    dots(p0, j + 2);
+    ok = grid_barrier(a.bar) && ok;
+    gather(p0, j + 2, h1);
+    update(h1);
+    // DGKS test, the same in every block: more than half of ||w||^2 removed?
+    {
+        double s = 0.0;
+        for (int i = tid; i <= j; i += kArnTPB) s = fma(h1[i], h1[i], s);
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) s_red[warp] = s;
+        __syncthreads();
+        s = 0.0;
+#pragma unroll
+        for (int k = 0; k < kArnTPB / 32; ++k) s += s_red[k];
+        __syncthreads();
+        if (ok && s > 0.5 * h1[j + 1]) {
+            dots(p1, j + 1);
+            ok = grid_barrier(a.bar + 1) && ok;
+            gather(p1, j + 1, h2);
+            update(h2);
+        } else {
+            for (int i = tid; i <= j; i += kArnTPB) h2[i] = 0.0;
+        }
+    }
+    if (!ok) {   // a barrier's wait ran out: report it as a residual that is not finite
+        if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
+        return;
+    }
+    {
+        double t = 0.0;
+        for (int r = tid; r < nr; r += kArnTPB) t = fma(w[r], w[r], t);
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        if (lane == 0) s_red[warp] = t;
+        __syncthreads();
+        if (tid == 0) {
+            t = 0.0;
+            for (int k = 0; k < kArnTPB / 32; ++k) t += s_red[k];
+            p2[blockIdx.x] = t;
+        }
+    }
+    if (!grid_barrier(a.bar + 2)) {
+        if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
+        return;
+    }
+    {
+        double t = 0.0;
+        for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(p2 + b);
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        const double hn = sqrt(fmax(t, 0.0));
+        const double f = hn != 0.0 ? 1.0 / hn : 1.0;
+        for (int r = tid; r < nr; r += kArnTPB) wg[r] = w[r] * f;
+        if (blockIdx.x != 0) return;
+        // H(:, j) and the rotations, as givens_kernel does; h1 becomes the column
+        for (int i = tid; i <= j; i += kArnTPB) h1[i] += h2[i];
+        __syncthreads();
+        for (int i = tid; i < j; i += kArnTPB) {
+            al[0][i] = -a.sn[i];
+            be[0][i] = a.cs[i] * h1[i + 1];
+        }
+        __syncthreads();
+        int cur = 0;
+        for (int off = 1; off < j; off <<= 1) {
+            for (int i = tid; i < j; i += kArnTPB) {
+                if (i >= off) {
+                    const double x = al[cur][i], y = be[cur][i];
+                    al[cur ^ 1][i] = x * al[cur][i - off];
+                    be[cur ^ 1][i] = x * be[cur][i - off] + y;
+                } else {
+                    al[cur ^ 1][i] = al[cur][i];
+                    be[cur ^ 1][i] = be[cur][i];
+                }
+            }
+            cur ^= 1;
+            __syncthreads();
+        }
+        const double a0 = h1[0];
+        double *hc = a.H + (int64_t)j * a.ldh;
+        for (int i = tid; i < j; i += kArnTPB) {
+            const double ai = i == 0 ? a0 : al[cur][i - 1] * a0 + be[cur][i - 1];
+            hc[i] = a.cs[i] * ai + a.sn[i] * h1[i + 1];
+        }
+        if (tid == 0) {
+            const double aj = j > 0 ? al[cur][j - 1] * a0 + be[cur][j - 1] : a0;
+            const double den = hypot(aj, hn);
+            const double cj = den != 0.0 ? aj / den : 1.0, sj = den != 0.0 ? hn / den : 0.0;
+            a.cs[j] = cj;
+            a.sn[j] = sj;
+            hc[j] = den;
+            hc[j + 1] = 0.0;
+            const double gj = a.g[j];
+            a.g[j + 1] = -sj * gj;
+            a.g[j] = cj * gj;
+            a.out[0] = fabs(sj * gj);
+            a.out[1] = hn;
+        }
+    }
+}
+
 // Back substitution H(0:k, 0:k) y = g(0:k), column by column: y_i is fixed,
 // then every earlier right-hand side entry drops H(l, i) y_i in parallel.
 __global__ void backsolve_kernel(const double *H, int ldh, const double *g, int k, double *y) {
@@ -354,14 +561,23 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
     Buf V, small;
     SSD_TRY(V.alloc(ctx, sizeof(double) * (size_t)(m + 1) * n));
     const int ldh = m + 1;
-    // small: H[(m+1)*m], cs[m], sn[m], g[m+1], h1[m+3], h2[m+3], y[m], scal[8]
-    const size_t nsmall = (size_t)ldh * m + 2 * m + (m + 1) + 2 * (m + 3) + m + 8;
+    // small: H[(m+1)*m], cs[m], sn[m], g[m+1], h1[m+3], h2[m+3], y[m], scal[8], and
+    // three barrier counters per Arnoldi step
+    const size_t nsmall = (size_t)ldh * m + 2 * m + (m + 1) + 2 * (m + 3) + m + 8 + (3 * m + 1) / 2;
     SSD_TRY(small.alloc(ctx, sizeof(double) * nsmall));
     double *H = small.d(), *cs = H + (size_t)ldh * m, *sn = cs + m, *g = sn + m, *h1 = g + m + 1,
            *h2 = h1 + m + 3, *y = h2 + m + 3, *scal = y + m;
+    unsigned *bar = reinterpret_cast<unsigned *>(scal + 8);
     Dots dots;
     SSD_TRY(dots.init(ctx, s, m + 2));
     const unsigned gb = grid_for(n);
+    // one launch per Arnoldi step while its blocks hold their rows in shared memory
+    int rows = (int)((n + ctx->num_sms - 1) / ctx->num_sms);
+    rows = (rows + kArnRows - 1) / kArnRows * kArnRows;
+    const unsigned arn_grid = (unsigned)((n + rows - 1) / rows);
+    // (with its three sets of (m + 2) * arn_grid partial sums in the dot buffer)
+    const bool fused = n <= kArnMaxN && rows <= kArnMaxRows &&
+                       3ll * (m + 2) * arn_grid <= (int64_t)kDotMaxBlocks * (m + 3);
 
     // ||b||
     SSD_TRY(dots.multi(b, 0, 1, b, n, scal));
@@ -379,23 +595,27 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
     int total = 0;
     bool first = true;
     for (;;) {
-        // r = b - A x  (r = b when x = 0 on the first cycle)
+        // r = b - A x  (r = b when x = 0 on the first cycle: its norm is known)
         double *v0 = V.d();
-        if (first && !warm) {
-            SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(v0, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s),
-                               "copy"));
-        } else {
+        const bool from_b = first && !warm;
+        if (!from_b) {
             SSD_TRY(A(x, v0));
             axpby_kernel<<<gb, 256, 0, s>>>(n, 1.0, b, -1.0, v0);
             ctx->launches++;
+            SSD_TRY(dots.multi(v0, 0, 1, v0, n, scal));
         }
         first = false;
-        SSD_TRY(dots.multi(v0, 0, 1, v0, n, scal));
         sqrt_kernel<<<1, 32, 0, s>>>(scal);
         gmres_init_kernel<<<1, 128, 0, s>>>(g, m, scal);
-        scale_inv_kernel<<<gb, 256, 0, s>>>(n, v0, scal, v0);
+        scale_inv_kernel<<<gb, 256, 0, s>>>(n, from_b ? b : v0, scal, v0);
         ctx->launches += 3;
-        SSD_TRY(read_scalars(ctx, scal, 1, hb, s));
+        if (fused) SSD_TRY(cuda_check(ctx, cudaMemsetAsync(bar, 0, sizeof(unsigned) * 3 * m, s), "memset"));
+        if (from_b) {
+            SSD_TRY(launch_check(ctx, "gmres start"));
+            hb[0] = bnorm;
+        } else {
+            SSD_TRY(read_scalars(ctx, scal, 1, hb, s));
+        }
         double rel = hb[0] / bnorm;
         res->relres = rel;
         if (!isfinite(rel)) return set_error(ctx, SSD_ENUMERIC, "non-finite residual");
@@ -415,6 +635,14 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
             double *w = V.d() + (size_t)(j + 1) * n;    // the new vector is built in its slot
             SSD_TRY(A(vj, w));
             ++total;
+            if (fused) {
+                ArnoldiArgs aa{V.d(), n, j, rows, ldh, H, cs, sn, g, dots.partial.d(), bar + 3 * j,
+                               slot + 2 * (j & 1)};
+                void *params[] = {&aa};
+                SSD_TRY(cuda_check(ctx, cudaLaunchCooperativeKernel((const void *)arnoldi_kernel, dim3(arn_grid),
+                                                                    dim3(kArnTPB), params, 0, s), "arnoldi step"));
+                ctx->launches++;
+            } else {
             // Gram-Schmidt pass (h1[j+1] = w . w from the same sweep), the
             // DGKS test, and a second pass only when the test asks for it
             SSD_TRY(dots.multi(V.d(), n, j + 2, w, n, h1));
@@ -431,6 +659,7 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
             SSD_TRY(launch_check(ctx, "arnoldi step"));
             SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(slot + 2 * (j & 1), scal, 2 * sizeof(double),
                                                     cudaMemcpyDeviceToHost, s), "residual copy"));
+            }
             SSD_TRY(cuda_check(ctx, cudaEventRecord(ev[j & 1], s), "event record"));
             if (pending >= 0) {
                 // step j was queued ahead: read step j - 1 now
