@@ -390,6 +390,7 @@ void batch_layout_release(ssd_ctx *ctx, BatchLayout *B) {
     for (int k = 0; k < 2; ++k) {
         if (B->items[k]) dev_free(ctx, B->items[k]);
     }
+    if (B->fx_pos) dev_free(ctx, B->fx_pos);
     *B = BatchLayout();
 }
 
@@ -539,6 +540,7 @@ int check_points(ssd_ctx *ctx, const ssd_points *pts) {
 void release_layout(ssd_ctx *ctx, Layout *L) {
     if (L->block) dev_free(ctx, L->block);
     if (L->order32) dev_free(ctx, L->order32);
+    if (L->fx_block) dev_free(ctx, L->fx_block);
     for (auto &pl : L->sym)
         if (pl.block) dev_free(ctx, pl.block);
     *L = Layout();

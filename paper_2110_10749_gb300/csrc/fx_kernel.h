@@ -31,6 +31,7 @@
 // generic kernel (fx_geo).
 
 constexpr int kFxExpMax = 400;
+constexpr int kFxGroups = 4;   // source groups of a CTA on small sets
 
 struct FxGeo {
     double c[3];          // grid origin
@@ -56,17 +57,10 @@ struct FxArgs {
     int64_t n;
 };
 
-// positions of the fixed-point grid, their chunk boxes and the densities' block
-// maxima (every thread of a 256-thread block calls this)
+// what the packing kernels leave for it: the densities' block maxima
 struct FxPack {
-    l4 *X = nullptr;             // NULL: not wanted
-    int4 *cbox = nullptr;
-    unsigned long long *bmax = nullptr;
-    FxGeo geo;
-    const FxGeo *geos = nullptr;     // batched
-    const BSurf *surfs = nullptr;
-    int nsurf = 0;
-    int two = 0;                 // LSLDL: .y of the first record is the second density
+    unsigned long long *bmax = nullptr;   // NULL: not wanted
+    int two = 0;                          // LSLDL: .y of the first record is the second density
 };
 
 __device__ __forceinline__ int64_t fx_grid(double x, double c, const FxGeo &g) {
@@ -78,10 +72,9 @@ __device__ __forceinline__ int64_t fx_grid(double x, double c, const FxGeo &g) {
     return a + __double2ll_rn((r - (double)a) + e * g.grid);
 }
 
-__device__ __forceinline__ void fx_pack(const FxPack &P, int64_t i, int64_t n_last, const d4 *pos, const int32_t *perm,
-                                        const d4 &r0, const d4 &r1, int rhs, int64_t nblk) {
+// block maxima (every thread of a 256-thread block calls this)
+__device__ __forceinline__ void fx_pack(const FxPack &P, const d4 &r0, const d4 &r1, int rhs, int64_t nblk) {
     __shared__ unsigned long long smax[2][8];
-    __shared__ int ssurf;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long am = 0x7fffffffffffffffull;
     auto bits = [&](double v) { return (unsigned long long)__double_as_longlong(v) & am; };
@@ -93,32 +86,50 @@ __device__ __forceinline__ void fx_pack(const FxPack &P, int64_t i, int64_t n_la
         m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
     }
     if (lane == 0) { smax[0][warp] = m0; smax[1][warp] = m1; }
-    if (threadIdx.x == 0) {
-        int lo = 0, hi = P.nsurf - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (P.surfs[mid].poff <= i) lo = mid; else hi = mid - 1;
-        }
-        ssurf = lo;
-    }
     __syncthreads();
     if (threadIdx.x < 2) {
         unsigned long long m = smax[threadIdx.x][0];
         for (int w = 1; w < 8; ++w) m = max(m, smax[threadIdx.x][w]);
         P.bmax[((int64_t)rhs * nblk + blockIdx.x) * 2 + threadIdx.x] = m;
     }
-    if (rhs != 0) return;
-    const FxGeo &g = P.geos ? P.geos[ssurf] : P.geo;
-    const int64_t last = P.surfs ? P.surfs[ssurf].poff + P.surfs[ssurf].n_real - 1 : n_last;
-    const d4 p = pos[i <= last ? i : last];   // padding: a copy of the last point, with zero weight and density
-    const int64_t x = fx_grid(p.x, g.c[0], g), y = fx_grid(p.y, g.c[1], g), z = fx_grid(p.z, g.c[2], g);
+}
+
+// Positions on the fixed-point grid and their chunk boxes, once per point set
+// and smoothing radius (32-thread blocks: about 50 double-precision operations
+// a point, so few points per SM).
+struct FxGrid {
+    const d4 *pos;
+    int64_t n_pad, n_last;       // one surface: last real point
+    FxGeo geo;
+    const FxGeo *geos;           // batched: per surface
+    const BSurf *surfs;
+    int nsurf;
+    l4 *X;
+    int4 *cbox;
+};
+
+__global__ void __launch_bounds__(kChunk) fx_grid_kernel(const __grid_constant__ FxGrid P) {
+    const int64_t i = (int64_t)blockIdx.x * kChunk + threadIdx.x;
+    int64_t last = P.n_last;
+    const FxGeo *g = &P.geo;
+    if (P.geos) {
+        int lo = 0, hi = P.nsurf - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (P.surfs[mid].poff <= i) lo = mid; else hi = mid - 1;
+        }
+        g = P.geos + lo;
+        last = P.surfs[lo].poff + P.surfs[lo].n_real - 1;
+    }
+    const d4 p = P.pos[i <= last ? i : last];   // padding: a copy of the last point, with zero weight and density
+    const int64_t x = fx_grid(p.x, g->c[0], *g), y = fx_grid(p.y, g->c[1], *g), z = fx_grid(p.z, g->c[2], *g);
     P.X[i] = l4{x, y, z, 0};
     const int xh = (int)(x >> 32), yh = (int)(y >> 32), zh = (int)(z >> 32);
     const int4 lo = make_int4(__reduce_min_sync(0xffffffffu, xh), __reduce_min_sync(0xffffffffu, yh),
                               __reduce_min_sync(0xffffffffu, zh), 0);
     const int4 hi = make_int4(__reduce_max_sync(0xffffffffu, xh), __reduce_max_sync(0xffffffffu, yh),
                               __reduce_max_sync(0xffffffffu, zh), 0);
-    if (lane == 0) { P.cbox[2 * (i >> 5)] = lo; P.cbox[2 * (i >> 5) + 1] = hi; }
+    if (threadIdx.x == 0) { P.cbox[2 * blockIdx.x] = lo; P.cbox[2 * blockIdx.x + 1] = hi; }
 }
 
 // The generic kernel's pair terms for one target in double precision, all
@@ -152,8 +163,11 @@ __device__ __noinline__ void fx_fallback(const KArgs<double> *ap, const Consts<d
 constexpr int kFxFarOct = 6;                     // 1 + 8^2 > 2^6
 template <int OP, bool FAR> constexpr int fx_ntab() { return FAR && OP == OP_SSL ? 1 : FxOp<OP>::ntab; }
 
-template <int OP, bool FAR>
-__global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ FxArgs a) {
+// GROUPS > 1: the threads form groups that share the CTA's 256 / GROUPS targets
+// and take sources grp, grp + GROUPS, .. of each staged tile; their sums are
+// added in order at the end.
+template <int OP, bool FAR, int GROUPS>
+__global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
     typedef FxOp<OP> T;
     constexpr int kOct0 = FAR ? kFxFarOct : 0;
     const int tstride = (a.noct - kOct0) * kFxSeg * kFxEntry;
@@ -166,6 +180,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
     __shared__ int4 s_uh[VU ? kTile : 1], s_ul[VU ? kTile : 1];
     __shared__ int4 s_fh[VF ? kTile : 1], s_fl[VF ? kTile : 1];
     __shared__ unsigned long long s_max[2][kFxTPB / 32];
+    __shared__ double s_sum[GROUPS > 1 ? NC : 1][GROUPS > 1 ? kFxTPB : 1];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t tbase, s_beg, s_end, part_base, pstride, b0 = 0, b1 = a.nblk;
@@ -186,7 +201,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
         part_base = blockIdx.y * a.k.part_stride + NC * sf.pbase + (int64_t)it.split * NC * sf.n_pad - sf.poff;
         pstride = sf.n_pad;
     } else {
-        tbase = (blockIdx.x + a.k.tile0) * kFxTPB;
+        tbase = (blockIdx.x + a.k.tile0) * (kFxTPB / GROUPS);
         s_beg = blockIdx.y * a.k.chunk;
         s_end = s_beg + a.k.chunk;
         const int64_t top = (a.n + kChunk - 1) / kChunk * kChunk;
@@ -194,7 +209,20 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
         part_base = blockIdx.y * NC * a.k.n_pad;
         pstride = a.k.n_pad;
     }
-    const int64_t i = tbase + threadIdx.x;
+    constexpr int nt = kFxTPB / GROUPS;
+    const int grp = threadIdx.x / nt;
+    const int64_t i = tbase + threadIdx.x % nt;
+    // the tables arrive while the densities' scale is found
+    for (int k = 0; k < fx_ntab<OP, FAR>(); ++k) {
+        const int4 *src = reinterpret_cast<const int4 *>(a.tab) +
+                          ((int64_t)T::tab(k) * kFxMaxOct + kOct0) * kFxSeg * kFxEntry;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_tab) + (uint32_t)(k * tstride) * 16u;
+        for (int q = threadIdx.x; q < tstride; q += kFxTPB)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q * 16u), "l"(src + q));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    pdl_wait();
+    pdl_release();
     // largest densities of this surface and right-hand side
     {
         unsigned long long m0 = 0, m1 = 0;
@@ -205,12 +233,6 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
             m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
         }
         if (lane == 0) { s_max[0][warp] = m0; s_max[1][warp] = m1; }
-    }
-    for (int k = 0; k < fx_ntab<OP, FAR>(); ++k) {
-        const int4 *src = reinterpret_cast<const int4 *>(a.tab) +
-                          ((int64_t)T::tab(k) * kFxMaxOct + kOct0) * kFxSeg * kFxEntry;
-        int4 *dst = reinterpret_cast<int4 *>(s_tab) + (int64_t)k * tstride;
-        for (int q = threadIdx.x; q < tstride; q += kFxTPB) dst[q] = src[q];
     }
     __syncthreads();
     int ee[2];
@@ -226,7 +248,8 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
     }
     double sum[3] = {0.0, 0.0, 0.0}, low[3] = {0.0, 0.0, 0.0};
     if (bad) {
-        fx_fallback<OP>(&a.k, cp, d0, d1, i, s_beg, s_end, sum);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (grp == 0) fx_fallback<OP>(&a.k, cp, d0, d1, i, s_beg, s_end, sum);
     } else {
         const FxGeo &g = *gp;
         const FxScale sc = fx_scale<OP>(ee[0], ee[1], g.em, g.dq, g.ed);
@@ -249,7 +272,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
         }
         int tlo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, thi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
 #pragma unroll
-        for (int k = 0; k < kFxTPB / kChunk; ++k) {
+        for (int k = 0; k < nt / kChunk; ++k) {
             const int4 l = a.cbox[2 * (tbase / kChunk + k)], h = a.cbox[2 * (tbase / kChunk + k) + 1];
             tlo[0] = min(tlo[0], l.x); tlo[1] = min(tlo[1], l.y); tlo[2] = min(tlo[2], l.z);
             thi[0] = max(thi[0], h.x); thi[1] = max(thi[1], h.y); thi[2] = max(thi[2], h.z);
@@ -329,6 +352,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
                     s_fl[threadIdx.x] = l;
                 }
             }
+            asm volatile("cp.async.wait_all;" ::: "memory");   // the tables, before the first tile
             __syncthreads();
             fx_split(grid(Y.x), y.x.h[0], y.x.l[0]);
             fx_split(grid(Y.y), y.x.h[1], y.x.l[1]);
@@ -339,7 +363,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
             // Stokes layer has no registers left beyond 2)
             constexpr int kUnroll = OP == OP_SDLT ? 2 : 4;
 #pragma unroll kUnroll
-            for (int j = 0; j < cnt; ++j) {
+            for (int j = grp; j < cnt; j += GROUPS) {
                 FxPoint<OP> x;
                 auto vec = [](FxV &v, const int4 &h, const int4 &l) {
                     v.h[0] = h.x; v.h[1] = h.y; v.h[2] = h.z;
@@ -373,6 +397,15 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const __grid_constant__ F
         }
 #pragma unroll
         for (int c = 0; c < NC; ++c) sum[c] += low[c];
+    }
+    if constexpr (GROUPS > 1) {   // the groups' sums, in order
+#pragma unroll
+        for (int q = 0; q < NC; ++q) s_sum[q][threadIdx.x] = sum[q];
+        __syncthreads();
+        if (grp) return;
+        for (int g = 1; g < GROUPS; ++g)
+#pragma unroll
+            for (int q = 0; q < NC; ++q) sum[q] += s_sum[q][threadIdx.x + g * nt];
     }
     if (a.k.acc) {
 #pragma unroll
@@ -423,27 +456,34 @@ template <int OP, bool FAR> size_t fx_smem(int noct) {
     return (size_t)fx_ntab<OP, FAR>() * (noct - (FAR ? kFxFarOct : 0)) * kFxSeg * kFxEntry * sizeof(FxI4);
 }
 
-template <int OP, bool FAR = false> cudaError_t launch_fx1(dim3 grid, const FxArgs &a, cudaStream_t s) {
-    fx_kernel<OP, FAR><<<grid, kFxTPB, fx_smem<OP, FAR>(a.noct), s>>>(a);
-    return cudaGetLastError();
+template <int OP, bool FAR = false, int GROUPS = 1>
+cudaError_t launch_fx1(dim3 grid, const FxArgs &a, cudaStream_t s) {
+    return launch_pdl(fx_kernel<OP, FAR, GROUPS>, grid, dim3(kFxTPB), fx_smem<OP, FAR>(a.noct), s, a);
+}
+template <int OP> cudaError_t launch_fx1(dim3 grid, const FxArgs &a, int groups, cudaStream_t s) {
+    return groups == 1 ? launch_fx1<OP, false, 1>(grid, a, s) : launch_fx1<OP, false, kFxGroups>(grid, a, s);
 }
 
-cudaError_t launch_fx(int op, dim3 grid, const FxArgs &a, cudaStream_t s) {
+cudaError_t launch_fx(int op, dim3 grid, const FxArgs &a, int groups, cudaStream_t s) {
     switch (op) {
-        case OP_LSL: return launch_fx1<OP_LSL>(grid, a, s);
-        case OP_LDL: return launch_fx1<OP_LDL>(grid, a, s);
-        case OP_SSL: return launch_fx1<OP_SSL>(grid, a, s);
-        case OP_SDL: return launch_fx1<OP_SDL>(grid, a, s);
-        case OP_SSLDL: return launch_fx1<OP_SSLDL>(grid, a, s);
-        case OP_LSLDL: return launch_fx1<OP_LSLDL>(grid, a, s);
-        case OP_LDLT: return launch_fx1<OP_LDLT>(grid, a, s);
-        default: return launch_fx1<OP_SDLT>(grid, a, s);
+        case OP_LSL: return launch_fx1<OP_LSL>(grid, a, groups, s);
+        case OP_LDL: return launch_fx1<OP_LDL>(grid, a, groups, s);
+        case OP_SSL: return launch_fx1<OP_SSL>(grid, a, groups, s);
+        case OP_SDL: return launch_fx1<OP_SDL>(grid, a, groups, s);
+        case OP_SSLDL: return launch_fx1<OP_SSLDL>(grid, a, groups, s);
+        case OP_LSLDL: return launch_fx1<OP_LSLDL>(grid, a, groups, s);
+        case OP_LDLT: return launch_fx1<OP_LDLT>(grid, a, groups, s);
+        default: return launch_fx1<OP_SDLT>(grid, a, groups, s);
     }
 }
 
 template <int OP, bool FAR = false> cudaError_t fx_attr1() {
-    return cudaFuncSetAttribute(fx_kernel<OP, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)fx_smem<OP, FAR>(kFxMaxOct));
+    const int bytes = (int)fx_smem<OP, FAR>(kFxMaxOct);
+    cudaError_t e = cudaFuncSetAttribute(fx_kernel<OP, FAR, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if constexpr (!FAR)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fx_kernel<OP, false, kFxGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
 }
 
 // Uploads the kernel tables of a context and lets the kernels use them.

@@ -72,6 +72,8 @@ struct Layout {
     float4 *cbox = nullptr;    // per 32-point chunk: [2 * c] = (lo x, y, z, 0), [2 * c + 1] = (hi ...)
     double wsum = 0.0;         // sum of weights (host copy)
     Extent ext{};              // box and largest weighted normal (host copy)
+    void *fx_block = nullptr;  // grid positions and chunk boxes of the fixed-point kernel (pool memory)
+    double fx_delta = 0.0;     // smoothing radius they were made for
     void *block = nullptr;     // single allocation backing the arrays
     // launch order of the FP32C pair grid (prepared layouts only), cached for
     // the last (grid, rho_far delta) it was built for
@@ -104,7 +106,7 @@ struct ssd_ctx {
     int waves32 = 12;          // FP32C grid: about this many waves of resident CTAs (tuned)
     int lpt = 1;               // pair grids in near-first order on prepared layouts
     int sym = 1;               // layer operators (both precisions): far block pairs once for both directions
-    int waves_fx = 4;          // FP64 fixed-point grid: about this many waves of resident CTAs
+    int waves_fx = 10;         // FP64 fixed-point grid of large sets: rounds of two CTAs per SM
     int waves64 = 8;           // FP64 grid: about this many waves of resident CTAs (tuned)
     void *fx_tab = nullptr;    // kernel tables of the fixed-point FP64 kernels (built with the context)
     void *noalloc_scratch = nullptr;   // device address of the no-alloc scratch array (first no-alloc call)
@@ -202,6 +204,7 @@ struct BatchLayout {
     std::vector<double> delta, wsum;
     std::vector<Extent> ext;
     void *fx_geo = nullptr;   // per-surface constants of the fixed-point kernel (in block)
+    void *fx_pos = nullptr;   // grid positions and chunk boxes
     int fx_noct = 0;          // octaves of the kernel tables the surfaces need; 0: some surface is out of range
     Layout L;                 // concatenated padded arrays; L.perm maps to caller indices
     int32_t *elem_surf = nullptr;   // [n_total] surface of each caller index
@@ -248,6 +251,36 @@ int quadrature_jacobian(ssd_ctx *ctx, const ssd_surface *surf, double h, double 
 
 // Small vector kernels (solve.cu)
 int dot(ssd_ctx *ctx, const double *a, const double *b, int64_t n, double *dev_out, cudaStream_t s);
+
+}  // namespace ssd
+
+namespace ssd {
+
+// Programmatic dependent launch: a kernel launched this way may start while
+// its predecessor in the stream still runs, so that launch latency and set-up
+// overlap; it calls pdl_wait() before it reads anything the predecessor wrote
+// or writes anything the predecessor may still read.  pdl_release() lets the
+// next kernel start and comes after pdl_wait(), so that whatever lies further
+// back in the stream is complete for it.  Both are no-ops in a plain launch.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename Arg>
+inline cudaError_t launch_pdl(void (*kernel)(Arg), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Arg &arg) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, arg);
+}
+#endif
 
 }  // namespace ssd
 

@@ -20,7 +20,6 @@
 #include <math.h>
 #include <string.h>
 
-
 #include "internal.h"
 #include "erfcx_coef.h"
 #include "fx_pair.h"
@@ -530,6 +529,8 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
         part_base = bs * NC * a.nslot * a.n_pad;
         pstride = a.n_pad;
     }
+    pdl_wait();
+    pdl_release();
     // target t = 2k + j (pair k, lane j) is index tbase + threadIdx.x + t * kTPB32
     float2 y[NP][3], dt[NP][3];
     float blo[3] = {1e30f, 1e30f, 1e30f}, bhi[3] = {-1e30f, -1e30f, -1e30f};
@@ -1009,6 +1010,8 @@ struct PackArgs {
 template <typename V4, typename R>
 __global__ void pack_kernel(const PackArgs a) {
     __shared__ double red[256];
+    pdl_wait();
+    pdl_release();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double wd = 0.0;
     V4 r0 = {R(0), R(0), R(0), R(0)}, r1 = {R(0), R(0), R(0), R(0)};
@@ -1056,7 +1059,7 @@ __global__ void pack_kernel(const PackArgs a) {
         if (a.out1) reinterpret_cast<V4 *>(a.out1)[i] = r1;
     }
     if constexpr (sizeof(R) == 8) {   // n_pad is a multiple of 512: whole blocks
-        if (a.fx.X) fx_pack(a.fx, i, a.n - 1, a.pos64, a.perm, r0, r1, 0, gridDim.x);
+        if (a.fx.bmax) fx_pack(a.fx, r0, r1, 0, gridDim.x);
     }
     if (a.wdot_part) {
         red[threadIdx.x] = wd;
@@ -1097,17 +1100,19 @@ __global__ void epilogue_kernel(const EpiArgs a) {
     // one thread per (point, component): partial sums are summed over the
     // splits in a fixed order in FP64
     __shared__ double extra, rank1;
-    if (threadIdx.x == 0) {
-        double e = a.add_dev ? *a.add_dev : 0.0;
-        double r1 = 0.0;
-        if (a.wdot_part) {
-            double s = 0.0;
-            for (int k = 0; k < a.nwdot; ++k) s += a.wdot_part[k];
-            if (a.rank1_nrm) r1 = s * a.wdot_scale;
-            else e += s * a.wdot_scale;
+    pdl_wait();
+    pdl_release();
+    if (threadIdx.x < 32) {
+        double s = 0.0;
+        if (a.wdot_part) {   // one warp, fixed order (a serial sum of N / 256 parts took longer than the rest)
+            for (int k = threadIdx.x; k < a.nwdot; k += 32) s += a.wdot_part[k];
+            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            s *= a.wdot_scale;
         }
-        extra = e;
-        rank1 = r1;
+        if (threadIdx.x == 0) {
+            extra = (a.add_dev ? *a.add_dev : 0.0) + (a.rank1_nrm ? 0.0 : s);
+            rank1 = a.rank1_nrm ? s : 0.0;
+        }
     }
     __syncthreads();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1196,8 +1201,7 @@ cudaError_t launch_transpose(int op, dim3 grid, const KArgs<R> &ka, cudaStream_t
 
 template <int OP>
 cudaError_t launch32(dim3 grid, const K32Args &ka, cudaStream_t s) {
-    pair32_kernel<OP><<<grid, kTPB32, 0, s>>>(ka);
-    return cudaGetLastError();
+    return launch_pdl(pair32_kernel<OP>, grid, dim3(kTPB32), 0, s, ka);
 }
 
 cudaError_t launch_pair_op32(int op, dim3 grid, const K32Args &ka, cudaStream_t s) {
@@ -1291,7 +1295,7 @@ __global__ void bpack_kernel(const BPackArgs a) {
         if (a.out1) reinterpret_cast<V4 *>(a.out1)[(int64_t)r * a.n_pad + i] = r1;
     }
     if constexpr (sizeof(R) == 8) {
-        if (a.fx.X) fx_pack(a.fx, i, 0, a.pos64, a.perm, r0, r1, r, gridDim.x);
+        if (a.fx.bmax) fx_pack(a.fx, r0, r1, r, gridDim.x);
     }
     if (a.want_wdot) {
         red[threadIdx.x] = wd;
@@ -1654,17 +1658,58 @@ int pair_occupancy(ssd_ctx *ctx) {
 
 size_t fx_geo_bytes(int nsurf) { return sizeof(FxGeo) * nsurf; }
 
-// Source split of the fixed-point grid: every tile costs the same, so the
-// grid only has to fill the GPU evenly; splits are multiples of 32 sources.
-static int64_t fx_chunk(const ssd_ctx *ctx, int64_t n, int64_t ntiles_t, int64_t *nsplit) {
+// Grid of the fixed-point kernel.  Every pair costs the same, so it only has to
+// fill the SMs evenly.  Small sets: at most one round of two CTAs per SM, the
+// grouped form where its finer items leave less to the fullest CTA (N = 1062:
+// 289 CTAs of 64 targets, against 170 of 256: Stokes double layer 44 us instead
+// of 55 with its packing and epilogue; N = 1742: 280 against 196).  From 6000
+// points on about 5 rounds, which the scheduler levels.
+struct FxSplit {
+    int groups = 1;
+    int64_t chunk = 0, nsplit = 1;
+};
+
+static FxSplit fx_split_grid(const ssd_ctx *ctx, int64_t n) {
     const int64_t units = (n + kChunk - 1) / kChunk;
-    const int64_t want = (int64_t)ctx->num_sms * 2 * ctx->waves_fx;
-    int64_t ns = (want + ntiles_t - 1) / ntiles_t;
-    if (ns < 1) ns = 1;
-    if (ns > units) ns = units;
-    const int64_t cu = (units + ns - 1) / ns;
-    *nsplit = (units + cu - 1) / cu;
-    return cu * kChunk;
+    const int64_t want = (int64_t)ctx->num_sms * 2 * (n < 6000 ? 1 : ctx->waves_fx);
+    FxSplit best;
+    int64_t cost = 0;
+    for (int g = 1; g <= kFxGroups; g *= kFxGroups) {
+        const int64_t span = kFxTPB / g, nt = (n + span - 1) / span;
+        int64_t ns = want / nt;
+        ns = ns < 1 ? 1 : (ns > units ? units : ns);
+        int64_t cu = (units + ns - 1) / ns;
+        if (cu > 8) cu = (cu + 3) / 4 * 4;   // whole staged tiles
+        if (g > 1 && (n >= 6000 || span * cu >= cost)) continue;   // pairs of the fullest CTA
+        cost = span * cu;
+        best.groups = g;
+        best.chunk = cu * kChunk;
+        best.nsplit = (units + cu - 1) / cu;
+    }
+    return best;
+}
+
+// Grid positions of a layout at a smoothing radius, kept with a prepared
+// layout for the last radius it was used with.
+static int fx_positions(ssd_ctx *ctx, const Layout &L, double delta, const FxGeo &geo, const l4 **X, const int4 **cbox,
+                        cudaStream_t s) {
+    Layout &M = const_cast<Layout &>(L);
+    if (!M.fx_block) {
+        SSD_TRY(dev_alloc(ctx, sizeof(l4) * L.n_pad + sizeof(int4) * 2 * (L.n_pad / kChunk), &M.fx_block));
+        M.fx_delta = 0.0;
+    }
+    l4 *x = static_cast<l4 *>(M.fx_block);
+    int4 *cb = reinterpret_cast<int4 *>(x + L.n_pad);
+    if (M.fx_delta != delta) {
+        FxGrid g{L.pos64, L.n_pad, L.n - 1, geo, nullptr, nullptr, 1, x, cb};
+        fx_grid_kernel<<<(unsigned)(L.n_pad / kChunk), kChunk, 0, s>>>(g);
+        ctx->launches++;
+        SSD_TRY(launch_check(ctx, "grid positions"));
+        M.fx_delta = delta;
+    }
+    *X = x;
+    *cbox = cb;
+    return SSD_OK;
 }
 
 int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s) {
@@ -1678,7 +1723,8 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     FxGeo geo;
     int noct = 0;
     const bool use_fx = !f32 && fx_geo(L.ext, pc.delta, &geo, &noct);
-    const int tspan = packed32 ? kTPB32 * kTPT32 : (f32 ? kTPB64 * kTPT64 : kFxTPB);
+    const FxSplit fs = use_fx ? fx_split_grid(ctx, n) : FxSplit();
+    const int tspan = packed32 ? kTPB32 * kTPT32 : (f32 ? kTPB64 * kTPT64 : kFxTPB / fs.groups);
     const int64_t ntiles_t = use_fx ? (n + tspan - 1) / tspan : n_pad / tspan;
     const int64_t ntiles_s = n_pad / kTile;
     // splits: enough CTAs for several waves of resident CTAs, so that the
@@ -1692,7 +1738,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     const int64_t chunk_tiles = (ntiles_s + nsplit - 1) / nsplit;
     nsplit = (ntiles_s + chunk_tiles - 1) / chunk_tiles;
     int64_t chunk = chunk_tiles * kTile;
-    if (use_fx) chunk = fx_chunk(ctx, n, ntiles_t, &nsplit);
+    if (use_fx) { chunk = fs.chunk; nsplit = fs.nsplit; }
 
     const size_t rec = f32 ? sizeof(float4) : sizeof(d4);
     // FP32C keeps a (hi, lo) pair per target and split; one slot suffices when
@@ -1724,8 +1770,6 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         use_sym = L.sym[f32 ? 0 : 1].use;
     }
     const size_t o_acc = use_sym ? carve(sizeof(double) * nc * n_pad) : 0;
-    const size_t o_fx = use_fx ? carve(sizeof(l4) * n_pad) : 0;
-    const size_t o_fxb = use_fx ? carve(sizeof(int4) * 2 * (n_pad / kChunk)) : 0;
     const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks) : 0;
     void *ws = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &ws));
@@ -1766,20 +1810,17 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     pa.wdot_part = rank1 ? reinterpret_cast<double *>(base + o_wdot) : nullptr;
     FxArgs fa{};
     if (use_fx) {
-        pa.fx.X = reinterpret_cast<l4 *>(base + o_fx);
-        pa.fx.cbox = reinterpret_cast<int4 *>(base + o_fxb);
+        SSD_TRY(fx_positions(ctx, L, pc.delta, geo, &fa.X, &fa.cbox, s));
         pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
-        pa.fx.geo = geo;
         pa.fx.two = op == OP_LSLDL ? 1 : 0;
-        fa.X = pa.fx.X; fa.cbox = pa.fx.cbox; fa.bmax = pa.fx.bmax;
+        fa.bmax = pa.fx.bmax;
         fa.nblk = pack_blocks; fa.tab = static_cast<const FxI4 *>(ctx->fx_tab); fa.noct = noct;
         fa.geo = geo; fa.geos = nullptr; fa.n = n;
         self_src = nullptr;    // the self pair is part of the sum
     }
-    if (f32) pack_kernel<float4, float><<<pack_blocks, 256, 0, s>>>(pa);
-    else pack_kernel<d4, double><<<pack_blocks, 256, 0, s>>>(pa);
+    SSD_TRY(cuda_check(ctx, launch_pdl(f32 ? pack_kernel<float4, float> : pack_kernel<d4, double>, dim3(pack_blocks),
+                                       dim3(256), 0, s, pa), "pack kernel"));
     ctx->launches++;
-    SSD_TRY(launch_check(ctx, "pack kernel"));
 
     const int cls = kernel_class(op);
     // a row block (layout rows [row_begin, row_end)) launches only the target
@@ -1858,7 +1899,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         ka.tile0 = tile0;
         if (use_fx) {
             fa.k = ka;
-            e = launch_fx(op, grid, fa, s);
+            e = launch_fx(op, grid, fa, fs.groups, s);
         } else {
             e = transposed ? launch_transpose<double>(op, grid, ka, s) : launch_pair_op64(op, grid, ka, s);
         }
@@ -1882,9 +1923,9 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     ea.weight_out = tsl ? 1 : 0;
     ea.out = pc.out;
     if (rows) { ea.row0 = pc.row_begin; ea.row1 = pc.row_end; }
-    epilogue_kernel<<<(unsigned)((n_pad * nc + 127) / 128), 128, 0, s>>>(ea);
     ctx->launches++;
-    return launch_check(ctx, "epilogue kernel");
+    return cuda_check(ctx, launch_pdl(epilogue_kernel, dim3((unsigned)((n_pad * nc + 127) / 128)), dim3(128), 0, s, ea),
+                      "epilogue kernel");
 }
 
 
@@ -1999,6 +2040,16 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
                                                 cudaMemcpyHostToDevice, s), "surfs copy"));
         SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(bp + o_c, cbuf.data(), csz * ns, cudaMemcpyHostToDevice, s),
                            "consts copy"));
+        if (fx) {
+            SSD_TRY(dev_alloc(ctx, sizeof(l4) * B->n_pad_total + sizeof(int4) * 2 * (B->n_pad_total / kChunk),
+                              &B->fx_pos));
+            l4 *x = static_cast<l4 *>(B->fx_pos);
+            FxGrid g{B->L.pos64, B->n_pad_total, 0, FxGeo(), static_cast<const FxGeo *>(B->fx_geo),
+                     reinterpret_cast<const BSurf *>(bp + o_sf), ns, x, reinterpret_cast<int4 *>(x + B->n_pad_total)};
+            fx_grid_kernel<<<(unsigned)(B->n_pad_total / kChunk), kChunk, 0, s>>>(g);
+            ctx->launches++;
+            SSD_TRY(launch_check(ctx, "grid positions"));
+        }
         // the host vectors go out of scope: wait for the copies
         SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "items sync"));
         if (pr == 0 && ctx->lpt && !items.empty()) {
@@ -2054,8 +2105,6 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
     const size_t o_wdot = carve(sizeof(double) * pack_blocks * nrhs);
     const size_t o_r1 = carve(sizeof(double) * B.nsurf * nrhs);
     const bool use_fx = !f32 && B.fx_noct > 0;
-    const size_t o_fx = use_fx ? carve(sizeof(l4) * n_pad) : 0;
-    const size_t o_fxb = use_fx ? carve(sizeof(int4) * 2 * (n_pad / kChunk)) : 0;
     const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks * nrhs) : 0;
     void *ws = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &ws));
@@ -2092,16 +2141,13 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
     pa.want_wdot = rank1 ? 1 : 0;
     FxArgs fa{};
     if (use_fx) {
-        pa.fx.X = reinterpret_cast<l4 *>(base + o_fx);
-        pa.fx.cbox = reinterpret_cast<int4 *>(base + o_fxb);
         pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
-        pa.fx.geos = static_cast<const FxGeo *>(B.fx_geo);
-        pa.fx.surfs = reinterpret_cast<const BSurf *>(B.surfs[pr]);
-        pa.fx.nsurf = B.nsurf;
         pa.fx.two = op == OP_LSLDL ? 1 : 0;
-        fa.X = pa.fx.X; fa.cbox = pa.fx.cbox; fa.bmax = pa.fx.bmax;
+        fa.X = static_cast<const l4 *>(B.fx_pos);
+        fa.cbox = reinterpret_cast<const int4 *>(fa.X + n_pad);
+        fa.bmax = pa.fx.bmax;
         fa.nblk = pack_blocks; fa.tab = static_cast<const FxI4 *>(ctx->fx_tab); fa.noct = B.fx_noct;
-        fa.geos = pa.fx.geos; fa.n = n_pad;
+        fa.geos = static_cast<const FxGeo *>(B.fx_geo); fa.n = n_pad;
         self_src = nullptr;    // the self pair is part of the sum
     }
     const dim3 pg((unsigned)pack_blocks, (unsigned)nrhs);
@@ -2148,7 +2194,7 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
         ka.rec_stride = n_pad; ka.part_stride = part_stride;
         if (use_fx) {
             fa.k = ka;
-            e = launch_fx(op, grid, fa, s);
+            e = launch_fx(op, grid, fa, 1, s);
         } else {
             e = launch_pair_op64(op, grid, ka, s);
         }

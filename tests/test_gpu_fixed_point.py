@@ -143,3 +143,16 @@ def test_batch_mixes_sizes_and_scales(gpu_ctx, cloud):
             ref = ALPHA * oracle.stokes_sl(p, deltas[k], MU, y) + BETA * oracle.stokes_dl(p, deltas[k], x)
             assert np.linalg.norm(out[r][:, sl] - ref) <= TOL * np.linalg.norm(ref), (r, k)
     B.release()
+
+
+def test_one_layout_serves_several_radii(gpu_ctx, cloud):
+    # grid positions are kept per layout and radius
+    import paper_2110_10749_gb300 as ssd
+    n = 300
+    p = subset(cloud, n)
+    rng = np.random.default_rng(12)
+    dens = rng.normal(size=n), rng.normal(size=(3, n)), rng.normal(size=n), rng.normal(size=(3, n))
+    P = ssd.Points.from_numpy(p).prepare(gpu_ctx)
+    for d in (0.4, 0.1, 0.1, 0.4):
+        close(device(ssd, gpu_ctx, P, d, *dens), dense(p, d, *dens))
+    P.release()
