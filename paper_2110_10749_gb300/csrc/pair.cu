@@ -500,14 +500,13 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
     __shared__ float4 sm_d0[kTile];
     __shared__ float4 sm_d1[OpInfo<OP>::D1 ? kTile : 1];
 
-    int64_t tbase, s_beg, s_end, part_base, pstride, nreal_end;
+    int64_t tbase, s_beg, s_end, part_base, pstride;
     const float4 *d0 = a.d0, *d1 = a.d1;
     Consts<float> c;
     if (a.items) {
         const BItem it = a.items[blockIdx.x];
         const BSurf sf = a.surfs[it.surf];
         tbase = it.tbase; s_beg = it.s_beg; s_end = it.s_end;
-        nreal_end = sf.poff + sf.n_real;
         c = a.consts[it.surf];
         d0 += blockIdx.y * a.rec_stride;
         d1 += blockIdx.y * a.rec_stride;
@@ -524,7 +523,6 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
         s_beg = bs * a.chunk;
         s_end = s_beg + a.chunk;
         if (s_end > a.n_pad) s_end = a.n_pad;
-        nreal_end = a.n;
         c = a.c;
         part_base = bs * NC * a.nslot * a.n_pad;
         pstride = a.n_pad;
@@ -533,7 +531,6 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
     pdl_release();
     // target t = 2k + j (pair k, lane j) is index tbase + threadIdx.x + t * kTPB32
     float2 y[NP][3], dt[NP][3];
-    float blo[3] = {1e30f, 1e30f, 1e30f}, bhi[3] = {-1e30f, -1e30f, -1e30f};
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         const int64_t i0 = tbase + threadIdx.x + (2 * k) * kTPB32, i1 = i0 + kTPB32;
@@ -541,24 +538,14 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
         const float4 e0 = d0[i0], e1 = d0[i1];
         y[k][0] = make_float2(p0.x, p1.x); y[k][1] = make_float2(p0.y, p1.y); y[k][2] = make_float2(p0.z, p1.z);
         dt[k][0] = make_float2(e0.x, e1.x); dt[k][1] = make_float2(e0.y, e1.y); dt[k][2] = make_float2(e0.z, e1.z);
-        if (i0 < nreal_end) {
-            blo[0] = fminf(blo[0], p0.x); blo[1] = fminf(blo[1], p0.y); blo[2] = fminf(blo[2], p0.z);
-            bhi[0] = fmaxf(bhi[0], p0.x); bhi[1] = fmaxf(bhi[1], p0.y); bhi[2] = fmaxf(bhi[2], p0.z);
-        }
-        if (i1 < nreal_end) {
-            blo[0] = fminf(blo[0], p1.x); blo[1] = fminf(blo[1], p1.y); blo[2] = fminf(blo[2], p1.z);
-            bhi[0] = fmaxf(bhi[0], p1.x); bhi[1] = fmaxf(bhi[1], p1.y); bhi[2] = fmaxf(bhi[2], p1.z);
-        }
     }
-    // warp bounding box of its real targets
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            blo[q] = fminf(blo[q], __shfl_xor_sync(0xffffffffu, blo[q], off));
-            bhi[q] = fmaxf(bhi[q], __shfl_xor_sync(0xffffffffu, bhi[q], off));
-        }
-    const bool warp_empty = blo[0] > bhi[0];
+    // near test of a tile: lane (chunk, patch) compares the box of one 32-source
+    // chunk with that of one of the warp's kTPT32 patches of 32 consecutive targets
+    const int lane = threadIdx.x & 31;
+    constexpr int kChunks = kTile / kChunk;
+    static_assert(kChunks * kTPT32 <= 32, "one lane per (chunk, patch)");
+    const int64_t patch = (tbase + (threadIdx.x & ~31) + (lane % kTPT32) * kTPB32) / kChunk;
+    const float4 tlo = a.cbox[2 * patch], thi = a.cbox[2 * patch + 1];
     float hi[kTPT32][NC], lo[kTPT32][NC];
 #pragma unroll
     for (int t = 0; t < kTPT32; ++t)
@@ -577,15 +564,19 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
         float2 part[NP][3];
 #pragma unroll
         for (int k = 0; k < NP; ++k) part[k][0] = part[k][1] = part[k][2] = make_float2(0.f, 0.f);
-        for (int ch = 0; ch < kTile / kChunk; ++ch) {
-            const int64_t cidx = (tile + ch * kChunk) / kChunk;
+        uint32_t nearmask;
+        {
+            const int64_t cidx = tile / kChunk + (lane / kTPT32) % kChunks;
             const float4 clo = a.cbox[2 * cidx], chi = a.cbox[2 * cidx + 1];
-            const float gx = fmaxf(0.f, fmaxf(clo.x - bhi[0], blo[0] - chi.x));
-            const float gy = fmaxf(0.f, fmaxf(clo.y - bhi[1], blo[1] - chi.y));
-            const float gz = fmaxf(0.f, fmaxf(clo.z - bhi[2], blo[2] - chi.z));
-            const bool far_chunk = warp_empty || (gx * gx + gy * gy + gz * gz >= c.rfar2);
+            const float gx = fmaxf(0.f, fmaxf(clo.x - thi.x, tlo.x - chi.x));
+            const float gy = fmaxf(0.f, fmaxf(clo.y - thi.y, tlo.y - chi.y));
+            const float gz = fmaxf(0.f, fmaxf(clo.z - thi.z, tlo.z - chi.z));
+            nearmask = __ballot_sync(0xffffffffu, !(gx * gx + gy * gy + gz * gz >= c.rfar2));
+        }
+        for (int ch = 0; ch < kChunks; ++ch) {
+            const uint32_t bits = (nearmask >> (ch * kTPT32)) & ((1u << kTPT32) - 1u);   // near patches
             const int j0 = ch * kChunk;
-            if (far_chunk) {
+            if (bits == 0) {
 #pragma unroll 4
                 for (int j = j0; j < j0 + kChunk; ++j) {
                     const float4 sp = sm_pos[j];
@@ -606,17 +597,24 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
                     const float4 sw = OpInfo<OP>::WN ? sm_wn[j] : sp;
                     const float4 s0 = sm_d0[j];
                     const float4 s1 = OpInfo<OP>::D1 ? sm_d1[j] : s0;
-                    bool nearv = false, serv = false;
                     float2 DX[NP], DY[NP], DZ[NP], R2[NP];
+                    float m[NP], mall = 1e30f;   // smallest squared distances
 #pragma unroll
                     for (int k = 0; k < NP; ++k) {
                         DX[k] = sub2(y[k][0], bc2(sp.x));
                         DY[k] = sub2(y[k][1], bc2(sp.y));
                         DZ[k] = sub2(y[k][2], bc2(sp.z));
                         R2[k] = fma2(DZ[k], DZ[k], fma2(DY[k], DY[k], mul2(DX[k], DX[k])));
-                        nearv |= (R2[k].x < c.rfar2) | (R2[k].y < c.rfar2);
-                        serv |= (R2[k].x * c.inv_d2 < c.tser) | (R2[k].y * c.inv_d2 < c.tser);
+                        m[k] = fminf(R2[k].x, R2[k].y);
+                        mall = fminf(mall, m[k]);
                     }
+                    if (!__any_sync(0xffffffffu, mall < c.rfar2)) {
+#pragma unroll
+                        for (int k = 0; k < NP; ++k)
+                            pair2<OP, false>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
+                        continue;
+                    }
+                    const bool serv = mall * c.inv_d2 < c.tser;
                     if (__any_sync(0xffffffffu, serv)) {
                         // a target of the warp is within 0.5 delta of this source
                         // (the self pair or a close neighbour): scalar path with
@@ -644,14 +642,16 @@ __global__ void __launch_bounds__(kTPB32, kMinCTA32) pair32_kernel(const K32Args
                                 }
                             }
                         }
-                    } else if (__any_sync(0xffffffffu, nearv)) {
-#pragma unroll
-                        for (int k = 0; k < NP; ++k)
-                            pair2<OP, true>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
                     } else {
+                        // smoothed terms only for the target pairs that need them (they
+                        // equal the bare ones bit for bit beyond rho_far)
 #pragma unroll
-                        for (int k = 0; k < NP; ++k)
-                            pair2<OP, false>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
+                        for (int k = 0; k < NP; ++k) {
+                            if (((bits >> (2 * k)) & 3u) && __any_sync(0xffffffffu, m[k] < c.rfar2))
+                                pair2<OP, true>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
+                            else
+                                pair2<OP, false>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
+                        }
                     }
                 }
             }
