@@ -412,7 +412,21 @@ __device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 rsq2(float2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+// The hardware approximations without the library's handling of subnormals (two
+// multiplications and a comparison each): the same bits for normal arguments
+// and results.  r^2 of a packed pair is normal (closer pairs take the scalar
+// path; padding against padding is 0 with zero weight) and 2^x has x > -58.
+__device__ __forceinline__ float rsq1(float a) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float ex2(float a) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float2 rsq2(float2 a) { return make_float2(rsq1(a.x), rsq1(a.y)); }
 
 // Packed pair terms for the target pair (dt = target densities) with the
 // displacement (dx, dy, dz) = y - x and r2 = |y - x|^2 already formed.
@@ -438,7 +452,7 @@ __device__ __forceinline__ void pair2(const float2 dx, const float2 dy, const fl
         const float2 rr = mul2(mul2(r2, ri), bc2(c.inv_d));
         const float2 rho = make_float2(fminf(rr.x, 6.32455532f), fminf(rr.y, 6.32455532f));
         const float2 et = mul2(t, bc2(-1.4426950408889634f));
-        const float2 e = make_float2(exp2f(et.x), exp2f(et.y));
+        const float2 e = make_float2(ex2(et.x), ex2(et.y));
         const float2 w = fma2(make_float2(__fdividef(1.f, 1.f + rho.x), __fdividef(1.f, 1.f + rho.y)),
                               bc2(kErfcxA), bc2(-kErfcxB));
         const float2 P = erfcx_fit2(w);
