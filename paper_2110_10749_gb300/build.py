@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libssd.so")
 SOURCES = ["ctx.cu", "pair.cu", "quad.cu", "solve.cu", "batch.cu", "geom.cu", "field.cu", "fx_table.cu"]
-HEADERS = ["internal.h", "series_coef.h", "erfcx_coef.h", "fx.h", "fx_pair.h", "fx_kernel.h", os.path.join("..", "..", "include", "ssd.h")]
+HEADERS = ["internal.h", "series_coef.h", "erfcx_coef.h", "fx.h", "fx_geo.h", "fx_pair.h", "fx_kernel.h", os.path.join("..", "..", "include", "ssd.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS_EXTRA = []
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",

@@ -35,6 +35,8 @@ constexpr int kFxSegBits = 6;                   // segments per octave of v: 64
 constexpr int kFxSeg = 1 << kFxSegBits;
 constexpr int kFxMaxOct = 20;                   // octaves of v = 1 + t
 constexpr int kFxEntry = 3;                     // 16-byte words of a table entry
+constexpr int kFxBareEntries = 2 * kFxSeg;      // t^(-1/2) over two octaves of t
+constexpr int kFxTabEntries = 4 * kFxMaxOct * kFxSeg + kFxBareEntries;
 constexpr int kFxEBias = 8;                     // bias of the stored exponent
 // extent / delta served: beyond 256 the position grid is coarser than 2^-54
 // delta; below 1/16 all terms are small against the bounds that fix the units
@@ -227,8 +229,9 @@ FX_HD double fx_value(const FxMac &a) {
     return (double)a.h * 16777216.0 + (double)m;
 }
 
-// Kernel tables of sigma_1 .. sigma_4 on v in [1, 2^kFxMaxOct): host array of
-// 4 * kFxMaxOct * kFxSeg entries, built once per process (fx_table.cu).
+// Kernel tables of sigma_1 .. sigma_4 on v in [1, 2^kFxMaxOct), then t^(-1/2) on
+// t in [1, 4): host array of kFxTabEntries entries, built once per process
+// (fx_table.cu).
 const FxI4 *fx_table_host();
 
 }  // namespace ssd

@@ -30,19 +30,7 @@
 // whose extent is over 256 or under 1/16 delta, or that are not finite, keep the
 // generic kernel (fx_geo).
 
-constexpr int kFxExpMax = 400;
 constexpr int kFxGroups = 4;   // source groups of a CTA on small sets
-
-struct FxGeo {
-    double c[3];          // grid origin
-    double inv, inv_lo;   // 1 / delta to twice double precision
-    double grid;          // 2^ps
-    int ps;               // positions: (x - c) / delta in units of 2^-ps
-    int em;               // |w n| < 2^em
-    int ed, pad;
-    int64_t dq;           // 1 / delta = dq 2^(ed - 62)
-    double f_sl, f_dl;    // 1 / delta, 1 / delta^2
-};
 
 struct FxArgs {
     const l4 *X;
@@ -62,15 +50,6 @@ struct FxPack {
     unsigned long long *bmax = nullptr;   // NULL: not wanted
     int two = 0;                          // LSLDL: .y of the first record is the second density
 };
-
-__device__ __forceinline__ int64_t fx_grid(double x, double c, const FxGeo &g) {
-    const double hi = x - c, bb = hi - x, lo = (x - (hi - bb)) - (c + bb);   // x - c = hi + lo exactly
-    const double q = hi * g.inv;
-    const double e = fma(hi, g.inv, -q) + (hi * g.inv_lo + lo * g.inv);
-    const double r = q * g.grid;
-    const long long a = __double2ll_rn(r);
-    return a + __double2ll_rn((r - (double)a) + e * g.grid);
-}
 
 // block maxima (every thread of a 256-thread block calls this)
 __device__ __forceinline__ void fx_pack(const FxPack &P, const d4 &r0, const d4 &r1, int rhs, int64_t nblk) {
@@ -381,7 +360,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
                 }
                 if constexpr (VU) vec(x.u, s_uh[j], s_ul[j]);
                 if constexpr (VF) vec(x.f, s_fh[j], s_fl[j]);
-                fx_pair<OP, FAR>(y, x, tl, sc, idx_max, tab, acc);
+                fx_pair<OP, FAR ? kFxFar : kFxFull>(y, x, tl, sc, idx_max, tab, acc);
             }
             const double f = __longlong_as_double((long long)(1023 + tl.ex) << 52) *
                              (T::fused || !T::dl ? g.f_sl : g.f_dl);
@@ -414,42 +393,6 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
     }
 #pragma unroll
     for (int q = 0; q < NC; ++q) a.k.part[part_base + (int64_t)q * pstride + i] = sum[q];
-}
-
-// Constants of a point set and smoothing radius; false when the fixed-point
-// kernel does not serve it (extent outside kFxMinExt .. kFxMaxExt delta, values
-// that are not finite or far from unit scale).  noct: octaves of 1 + rho^2 that occur.
-bool fx_geo(const Extent &e, double delta, FxGeo *g, int *noct) {
-    if (!(e.fin > 0.0)) return false;
-    double ext = 0.0, r2 = 0.0;
-    for (int c = 0; c < 3; ++c) {
-        const double d = e.hi[c] - e.lo[c];
-        g->c[c] = 0.5 * (e.lo[c] + e.hi[c]);
-        ext = fmax(ext, d / delta);
-        r2 += d / delta * (d / delta);
-    }
-    g->em = 0;
-    if (e.mmax > 0.0) frexp(e.mmax, &g->em);
-    int xd;
-    frexp(delta, &xd);
-    double cm = 0.0;
-    for (int c = 0; c < 3; ++c) cm = fmax(cm, fabs(g->c[c]));
-    if (!(ext >= kFxMinExt && ext <= kFxMaxExt) || g->em > kFxExpMax || g->em < -kFxExpMax || xd > 60 || xd < -60 || !(cm < 1e100))
-        return false;
-    int xe;
-    frexp(ext, &xe);
-    g->ps = 62 - xe < 58 ? 62 - xe : 58;       // |x - c| / delta <= 2^(xe - 1): the grid value stays below 2^62
-    g->grid = ldexp(1.0, g->ps);
-    g->inv = 1.0 / delta;
-    g->inv_lo = fma(-g->inv, delta, 1.0) / delta;
-    const double m = frexp(g->inv, &g->ed);    // 1 / delta = (m + lo) 2^ed, 62 bits
-    g->dq = (int64_t)ldexp(m, 53) * 512 + llrint(ldexp(g->inv_lo, 62 - g->ed));
-    g->f_sl = 1.0 / delta;
-    g->f_dl = 1.0 / (delta * delta);
-    g->pad = 0;
-    const int k = (int)floor(log2(1.0 + r2 * (1.0 + 1e-12))) + 1;
-    *noct = k < kFxMaxOct ? k : kFxMaxOct;
-    return true;
 }
 
 template <int OP, bool FAR> size_t fx_smem(int noct) {
@@ -488,7 +431,7 @@ template <int OP, bool FAR = false> cudaError_t fx_attr1() {
 
 // Uploads the kernel tables of a context and lets the kernels use them.
 int fx_init(ssd_ctx *ctx) {
-    const size_t bytes = (size_t)4 * kFxMaxOct * kFxSeg * kFxEntry * sizeof(FxI4);
+    const size_t bytes = (size_t)kFxTabEntries * kFxEntry * sizeof(FxI4);
     SSD_TRY(dev_alloc(ctx, bytes, &ctx->fx_tab));
     SSD_TRY(cuda_check(ctx, cudaMemcpy(ctx->fx_tab, fx_table_host(), bytes, cudaMemcpyHostToDevice), "kernel tables"));
     cudaError_t e = fx_attr1<OP_LSL>();

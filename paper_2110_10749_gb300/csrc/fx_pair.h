@@ -76,10 +76,21 @@ template <int OP> FX_HD FxTile fx_tile(const FxScale &s, int L, int r) {
 
 template <int OP> struct FxSum { FxMac v[FxOp<OP>::vec ? 3 : 1]; FxF f; };
 
-// FAR: every pair of the tile has rho >= 8, where sigma_3 = sigma_1^3 (bare
-// kernels): the Stokes single layer then needs one table instead of two.
+// Modes.  kFxFar: every pair of the tile has rho >= 8, where sigma_3 = sigma_1^3
+// (bare kernels): the Stokes single layer then needs one table instead of two.
+// kFxBare: bare kernels at any rho >= 1, all from one table of t^(-1/2) over
+// 1 <= t < 4 (kFxBareEntries segments; t scales by powers of 4), with t.one = 0.
+enum FxMode { kFxFull = 0, kFxFar = 1, kFxBare = 2 };
+
+FX_HD FxQ fx_cube(const FxQ &a, int64_t sq) {   // (m 2^-(61+e))^3, sq = m^2 2^-62
+    FxQ r;
+    r.m = fx_mul(sq, a.m);
+    r.e = 3 * a.e - 2;
+    return r;
+}
+
 // tab(k, idx, w): word w of entry idx of staged table k
-template <int OP, bool FAR, typename Tab>
+template <int OP, FxMode MODE, typename Tab>
 FX_HD void fx_pair(const FxPoint<OP> &y, const FxPoint<OP> &x, const FxTile &t, const FxScale &s, uint32_t idx_max,
                    const Tab &tab, FxSum<OP> &acc) {
     typedef FxOp<OP> T;
@@ -88,15 +99,24 @@ FX_HD void fx_pair(const FxPoint<OP> &y, const FxPoint<OP> &x, const FxTile &t, 
     const FxArgSeg a = fx_index(d, t.one, t.oct0);
     const uint32_t idx = a.idx < idx_max ? a.idx : idx_max;
     FxQ K1, K3, KD;
-    if constexpr (T::k1 >= 0) K1 = fx_poly<fx_unit(0)>(tab(T::k1, idx, 0), tab(T::k1, idx, 1), tab(T::k1, idx, 2), a.sh, a.sl);
-    if constexpr (T::k3 >= 0 && FAR) {
-        K3.m = fx_mul(fx_mul(K1.m, K1.m), K1.m);   // (m 2^-(61+e))^3 in units of 2^-(61 + e3)
-        K3.e = 3 * K1.e - 2;
-    } else if constexpr (T::k3 >= 0) {
-        K3 = fx_poly<fx_unit(2)>(tab(T::k3, idx, 0), tab(T::k3, idx, 1), tab(T::k3, idx, 2), a.sh, a.sl);
+    if constexpr (MODE == kFxBare) {
+        const uint32_t i = a.idx & (kFxBareEntries - 1);
+        K1 = fx_poly<fx_unit(0)>(tab(0, i, 0), tab(0, i, 1), tab(0, i, 2), a.sh, a.sl);
+        K1.e += (int)(a.idx / kFxBareEntries);
+        const int64_t sq = fx_mul(K1.m, K1.m);
+        K3 = fx_cube(K1, sq);
+        KD = K3;
+        if constexpr (T::vec) { KD.m = fx_mul(K3.m, sq); KD.e = K3.e + 2 * K1.e - 2; }
+    } else {
+        if constexpr (T::k1 >= 0)
+            K1 = fx_poly<fx_unit(0)>(tab(T::k1, idx, 0), tab(T::k1, idx, 1), tab(T::k1, idx, 2), a.sh, a.sl);
+        if constexpr (T::k3 >= 0 && MODE == kFxFar)
+            K3 = fx_cube(K1, fx_mul(K1.m, K1.m));
+        else if constexpr (T::k3 >= 0)
+            K3 = fx_poly<fx_unit(2)>(tab(T::k3, idx, 0), tab(T::k3, idx, 1), tab(T::k3, idx, 2), a.sh, a.sl);
+        if constexpr (T::kd >= 0)
+            KD = fx_poly<fx_unit(T::vec ? 3 : 1)>(tab(T::kd, idx, 0), tab(T::kd, idx, 1), tab(T::kd, idx, 2), a.sh, a.sl);
     }
-    if constexpr (T::kd >= 0)
-        KD = fx_poly<fx_unit(T::vec ? 3 : 1)>(tab(T::kd, idx, 0), tab(T::kd, idx, 1), tab(T::kd, idx, 2), a.sh, a.sl);
     if constexpr (!T::vec) {
         if constexpr (OP == OP_LDL || OP == OP_LSLDL) {
             const FxQ B = fx_dot(d, x.m);

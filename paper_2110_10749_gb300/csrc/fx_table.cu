@@ -73,7 +73,7 @@ int64_t round_ll(ld x) { return (int64_t)llrintl(x); }
 
 std::vector<FxI4> build() {
     static const Sigma sig;
-    std::vector<FxI4> tab((size_t)4 * kFxMaxOct * kFxSeg * kFxEntry);
+    std::vector<FxI4> tab((size_t)kFxTabEntries * kFxEntry);
     ld node[kNodes], cheb[kNodes][kNodes];   // nodes, T_k(node_j)
     for (int j = 0; j < kNodes; ++j) {
         node[j] = cosl(kPiL * (j + 0.5L) / kNodes);
@@ -84,39 +84,44 @@ std::vector<FxI4> build() {
     mono[1][1] = 1;
     for (int k = 2; k <= kDeg; ++k)
         for (int p = 0; p <= k; ++p) mono[k][p] = (p ? 2 * mono[k - 1][p - 1] : 0) - mono[k - 2][p];
+    // entry of the polynomial through val (at the nodes), coefficient units 2^unit ..
+    auto entry = [&](const ld *val, int unit, FxI4 *t) {
+        ld c[kDeg + 1] = {}, top = 0;
+        for (int j = 0; j < kNodes; ++j) top = fmaxl(top, fabsl(val[j]));
+        for (int k = 0; k <= kDeg; ++k) {
+            ld a = 0;
+            for (int j = 0; j < kNodes; ++j) a += val[j] * cheb[k][j];
+            a *= (k ? 2.0L : 1.0L) / kNodes;
+            for (int p = 0; p <= k; ++p) c[p] += a * mono[k][p];
+        }
+        int ex;
+        frexpl(top * 1.002L, &ex);          // top < 2^ex: mantissa below 2^62 over the whole segment
+        const int e = 1 - ex;
+        const ld u = ldexpl(1, 61 + e);
+        int64_t q[kDeg + 1];
+        for (int p = 0; p <= 3; ++p) q[p] = round_ll(c[p] * u);
+        for (int p = 4; p <= kDeg; ++p) q[p] = round_ll(ldexpl(c[p] * u, p - 4 - unit));
+        auto lo = [](int64_t x) { return (int)(uint32_t)x; };
+        auto hi = [](int64_t x) { return (int)(x >> 32); };
+        t[0] = FxI4{lo(q[0]), hi(q[0]), lo(q[1]), hi(q[1])};
+        t[1] = FxI4{lo(q[2]), hi(q[2]), lo(q[3]), hi(q[3])};
+        t[2] = FxI4{(int)q[4], (int)q[5], (int)q[6], (int)((uint32_t)(int)q[7] << 8 | (uint32_t)(e + kFxEBias))};
+    };
     for (int o = 0; o < kFxMaxOct; ++o)
         for (int g = 0; g < kFxSeg; ++g) {
             const ld base = ldexpl(1, o), hw = base / (2 * kFxSeg);
             const ld vc = base + (2 * g + 1) * hw;
-            ld val[4][kNodes];
+            ld val[4][kNodes], bare[kNodes];
             for (int j = 0; j < kNodes; ++j) {
                 ld v4[4];
                 sig.at(vc - 1 + hw * node[j], v4);
                 for (int i = 0; i < 4; ++i) val[i][j] = v4[i];
+                bare[j] = 1 / sqrtl(vc + hw * node[j]);
             }
-            for (int i = 0; i < 4; ++i) {
-                ld c[kDeg + 1] = {}, top = 0;
-                for (int j = 0; j < kNodes; ++j) top = fmaxl(top, fabsl(val[i][j]));
-                for (int k = 0; k <= kDeg; ++k) {
-                    ld a = 0;
-                    for (int j = 0; j < kNodes; ++j) a += val[i][j] * cheb[k][j];
-                    a *= (k ? 2.0L : 1.0L) / kNodes;
-                    for (int p = 0; p <= k; ++p) c[p] += a * mono[k][p];
-                }
-                int ex;
-                frexpl(top * 1.002L, &ex);          // top < 2^ex: mantissa below 2^62 over the whole segment
-                const int e = 1 - ex;
-                const ld u = ldexpl(1, 61 + e);
-                int64_t q[kDeg + 1];
-                for (int p = 0; p <= 3; ++p) q[p] = round_ll(c[p] * u);
-                for (int p = 4; p <= kDeg; ++p) q[p] = round_ll(ldexpl(c[p] * u, p - 4 - fx_unit(i)));
-                FxI4 *t = &tab[((size_t)i * kFxMaxOct * kFxSeg + (size_t)o * kFxSeg + g) * kFxEntry];
-                auto lo = [](int64_t x) { return (int)(uint32_t)x; };
-                auto hi = [](int64_t x) { return (int)(x >> 32); };
-                t[0] = FxI4{lo(q[0]), hi(q[0]), lo(q[1]), hi(q[1])};
-                t[1] = FxI4{lo(q[2]), hi(q[2]), lo(q[3]), hi(q[3])};
-                t[2] = FxI4{(int)q[4], (int)q[5], (int)q[6], (int)((uint32_t)(int)q[7] << 8 | (uint32_t)(e + kFxEBias))};
-            }
+            for (int i = 0; i < 4; ++i)
+                entry(val[i], fx_unit(i), &tab[((size_t)i * kFxMaxOct * kFxSeg + (size_t)o * kFxSeg + g) * kFxEntry]);
+            if (o < 2)
+                entry(bare, fx_unit(0), &tab[((size_t)4 * kFxMaxOct * kFxSeg + (size_t)o * kFxSeg + g) * kFxEntry]);
         }
     return tab;
 }

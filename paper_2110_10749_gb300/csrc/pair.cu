@@ -22,6 +22,7 @@
 
 #include "internal.h"
 #include "erfcx_coef.h"
+#include "fx_geo.h"
 #include "fx_pair.h"
 #include "series_coef.h"
 

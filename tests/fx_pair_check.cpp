@@ -89,7 +89,7 @@ template <int OP> double check(const std::vector<Pt> &src, const std::vector<Pt>
         std::memset(&acc, 0, sizeof(acc));
         ld ref[3] = {0, 0, 0}, mag[3] = {0, 0, 0};
         for (const Pt &x : src) {
-            fx_pair<OP, false>(Y, conv(x), tl, sc, kFxMaxOct * kFxSeg - 1, entry, acc);
+            fx_pair<OP, kFxFull>(Y, conv(x), tl, sc, kFxMaxOct * kFxSeg - 1, entry, acc);
             ld d[3], r2 = 0, s[4], v[3] = {0, 0, 0}, av[3] = {0, 0, 0};
             for (int c = 0; c < 3; ++c) { d[c] = (ld)y.x[c] - x.x[c]; r2 += d[c] * d[c]; }
             const ld de = delta;
