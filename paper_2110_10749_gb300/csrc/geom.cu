@@ -150,51 +150,52 @@ __device__ __forceinline__ void geo_pair(const double d[3], double r2, double de
     }
 }
 
+// One CTA per point k, its threads taking every kGeoTPB-th partner.  The
+// double-precision pipe bounds it (49, 67, 90 and 101 clocks a pair and SM for
+// LSL, LDL, SSL and SDL on 9847 points, against 1.6 operations a clock; the
+// 9-13 loads of a pair come from L1), so what counts is that every SM has the
+// same share down to small sets.  With a thread per point instead, 1099 points
+// kept 9 of the 152 SMs busy: 5.3, 6.4, 9.1 and 9.2 ms, now 0.36, 0.44, 0.58
+// and 0.61; 9847 points 39-74 ms, now 17-34.
 template <int OP>
 __global__ void __launch_bounds__(kGeoTPB) geo_kernel(const GeoArgs A) {
     constexpr int NC = (OP == OP_LSL || OP == OP_LDL) ? 1 : 3;
-    __shared__ double sx[3][kGeoTPB], sn[3][kGeoTPB], sw[kGeoTPB], sa[NC][kGeoTPB], sb[NC][kGeoTPB];
+    constexpr int kWarps = kGeoTPB / 32;
+    __shared__ double part[kWarps][7];
     const int64_t n = A.n;
-    const int64_t k = (int64_t)blockIdx.x * kGeoTPB + threadIdx.x;
-    const bool act = k < n;
-    double xk[3] = {0, 0, 0}, nk[3] = {0, 0, 0}, ak[3] = {0, 0, 0}, bk[3] = {0, 0, 0}, wk = 0.0;
-    if (act) {
-        for (int e = 0; e < 3; ++e) { xk[e] = A.xyz[e * n + k]; nk[e] = A.nrm[e * n + k]; }
-        wk = A.w[k];
-        for (int e = 0; e < NC; ++e) { ak[e] = A.a[e * n + k]; bk[e] = A.b[e * n + k]; }
-    }
+    const int64_t k = blockIdx.x;
+    double xk[3], nk[3], ak[3] = {0, 0, 0}, bk[3] = {0, 0, 0};
+    for (int e = 0; e < 3; ++e) { xk[e] = A.xyz[e * n + k]; nk[e] = A.nrm[e * n + k]; }
+    const double wk = A.w[k];
+    for (int e = 0; e < NC; ++e) { ak[e] = A.a[e * n + k]; bk[e] = A.b[e * n + k]; }
     double gx[3] = {0, 0, 0}, gn[3] = {0, 0, 0}, gw = 0.0;
-    for (int64_t base = 0; base < n; base += kGeoTPB) {
-        const int64_t m = base + threadIdx.x;
-        __syncthreads();
-        if (m < n) {
-            for (int e = 0; e < 3; ++e) { sx[e][threadIdx.x] = A.xyz[e * n + m]; sn[e][threadIdx.x] = A.nrm[e * n + m]; }
-            sw[threadIdx.x] = A.w[m];
-            for (int e = 0; e < NC; ++e) { sa[e][threadIdx.x] = A.a[e * n + m]; sb[e][threadIdx.x] = A.b[e * n + m]; }
-        }
-        __syncthreads();
-        const int cnt = (int)((n - base) < kGeoTPB ? (n - base) : kGeoTPB);
-        if (!act) continue;
-        for (int j = 0; j < cnt; ++j) {
-            if (base + j == k) continue;
-            const double d[3] = {xk[0] - sx[0][j], xk[1] - sx[1][j], xk[2] - sx[2][j]};
-            const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-            const double nm[3] = {sn[0][j], sn[1][j], sn[2][j]};
-            double am[3] = {0, 0, 0}, bm[3] = {0, 0, 0};
-            for (int e = 0; e < NC; ++e) { am[e] = sa[e][j]; bm[e] = sb[e][j]; }
-            geo_pair<OP>(d, r2, A.delta, nk, wk, ak, bk, nm, sw[j], am, bm, gx, gn, gw);
-        }
+    for (int64_t m = threadIdx.x; m < n; m += kGeoTPB) {
+        if (m == k) continue;
+        double d[3], nm[3], am[3] = {0, 0, 0}, bm[3] = {0, 0, 0};
+        for (int e = 0; e < 3; ++e) { d[e] = xk[e] - A.xyz[e * n + m]; nm[e] = A.nrm[e * n + m]; }
+        for (int e = 0; e < NC; ++e) { am[e] = A.a[e * n + m]; bm[e] = A.b[e * n + m]; }
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        geo_pair<OP>(d, r2, A.delta, nk, wk, ak, bk, nm, A.w[m], am, bm, gx, gn, gw);
     }
-    if (!act) return;
-    // single-layer self term selfc * w_k (a_k . b_k)
-    double self = 0.0;
-    if (OP == OP_LSL || OP == OP_SSL)
-        for (int e = 0; e < NC; ++e) self += ak[e] * bk[e];
-    for (int e = 0; e < 3; ++e) {
-        A.gx[e * n + k] += A.scale * gx[e];
-        A.gn[e * n + k] += A.scale * gn[e];
+    double v[7] = {gx[0], gx[1], gx[2], gn[0], gn[1], gn[2], gw};
+    for (int e = 0; e < 7; ++e)
+        for (int o = 16; o; o >>= 1) v[e] += __shfl_xor_sync(0xffffffffu, v[e], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int e = 0; e < 7; ++e) part[threadIdx.x >> 5][e] = v[e];
+    __syncthreads();
+    if (threadIdx.x >= 7) return;
+    const int e = threadIdx.x;
+    double g = 0.0;
+    for (int i = 0; i < kWarps; ++i) g += part[i][e];
+    if (e < 3) A.gx[e * n + k] += A.scale * g;
+    else if (e < 6) A.gn[(e - 3) * n + k] += A.scale * g;
+    else {
+        // single-layer self term selfc * w_k (a_k . b_k)
+        double self = 0.0;
+        if (OP == OP_LSL || OP == OP_SSL)
+            for (int c = 0; c < NC; ++c) self += ak[c] * bk[c];
+        A.gw[k] += A.scale * g + A.selfc * self;
     }
-    A.gw[k] += A.scale * gw + A.selfc * self;
 }
 
 }  // namespace
@@ -218,7 +219,7 @@ int geometry_gradient(ssd_ctx *ctx, const ssd_points *pts, int op, double delta,
     }
     A.scale *= alpha;
     A.selfc *= alpha;
-    const unsigned grid = (unsigned)((A.n + kGeoTPB - 1) / kGeoTPB);
+    const unsigned grid = (unsigned)A.n;
     switch (op) {
         case OP_LSL: geo_kernel<OP_LSL><<<grid, kGeoTPB, 0, s>>>(A); break;
         case OP_LDL: geo_kernel<OP_LDL><<<grid, kGeoTPB, 0, s>>>(A); break;
