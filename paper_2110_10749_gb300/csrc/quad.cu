@@ -2,8 +2,8 @@
 // the four-atom molecule (eq. Molecule) and star-shaped surfaces
 // r(xi) = 1 + sum_{l<=4} c_lm Y_lm(xi).
 //
-// One thread per grid line.  A first pass counts the kept intersections per
-// line, an exclusive scan turns counts into output offsets, and a second pass
+// A first pass counts the kept intersections per grid line (one thread a line
+// on spheres and ellipsoids, quad_sample_kernel on the others), an exclusive scan turns counts into output offsets, and a second pass
 // writes points, normals, weights and (axis, j1, j2, root ordinal).  Points
 // and normals use correctly rounded +, -, *, /, sqrt only, in the order
 // stated next to each line (this file is compiled without FMA contraction),
@@ -53,8 +53,8 @@ __device__ __forceinline__ double bump(double r) {
 }
 
 // Evaluates the line; returns the number of kept roots and fills them.
-__device__ int eval_line(const QuadGeo &g, int ax, int64_t ja, int64_t jb, double P[kMaxRoots][3],
-                         double N[kMaxRoots][3], int br[kMaxRoots]) {
+__device__ int eval_line(const QuadGeo &g, int ax, int64_t ja, int64_t jb, double P[2][3],
+                         double N[2][3], int br[2]) {
     const int a = ax == 0 ? 1 : 0;
     const int b = ax == 2 ? 1 : 2;
     const double xa = __dmul_rn((double)ja, g.h);
@@ -230,57 +230,6 @@ __device__ void star_normal(const T *a, const QuadGeo &g, const T X[3], T nv[3])
     for (int k = 0; k < 3; ++k) nv[k] = G[k] / gn;
 }
 
-// Crossings of one grid line with the star surface (sampling + bisection).
-__device__ int eval_line_star(const QuadGeo &g, int ax, int64_t ja, int64_t jb, double P[kMaxRoots][3],
-                              double N[kMaxRoots][3], int br[kMaxRoots]) {
-    const int a = ax == 0 ? 1 : 0;
-    const int b = ax == 2 ? 1 : 2;
-    const double xa = (double)ja * g.h;
-    const double xb = (double)jb * g.h;
-    const double da = xa - g.c[a], db = xb - g.c[b];
-    if (!(da * da + db * db < g.rb * g.rb)) return 0;
-    double X[3];
-    X[a] = xa;
-    X[b] = xb;
-    X[ax] = g.tlo[ax];
-    double fprev = star_phi(g, X);
-    double tprev = g.tlo[ax];
-    int kept = 0, ordinal = 0;
-    for (int k = 1; k <= g.nk; ++k) {
-        const double t = g.tlo[ax] + (double)k * g.dt[ax];
-        X[ax] = t;
-        const double f = star_phi(g, X);
-        if ((fprev > 0.0) != (f > 0.0)) {
-            double lo = tprev, hi = t, flo = fprev, fhi = f;
-            const bool slo = flo > 0.0;
-            for (int it = 0; it < 200; ++it) {
-                const double mid = 0.5 * (lo + hi);
-                if (mid == lo || mid == hi) break;
-                X[ax] = mid;
-                const double fm = star_phi(g, X);
-                if ((fm > 0.0) == slo) { lo = mid; flo = fm; }
-                else { hi = mid; fhi = fm; }
-            }
-            X[ax] = fabs(flo) <= fabs(fhi) ? lo : hi;
-            double nv[3];
-            star_normal<double>(g.a, g, X, nv);
-            if (fabs(nv[ax]) >= g.ct) {
-                if (kept == kMaxRoots) {
-                    atomicExch(g.overflow, 1);
-                } else {
-                    for (int q = 0; q < 3; ++q) { P[kept][q] = X[q]; N[kept][q] = nv[q]; }
-                    br[kept] = ordinal;
-                    ++kept;
-                }
-            }
-            ++ordinal;
-        }
-        fprev = f;
-        tprev = t;
-    }
-    return kept;
-}
-
 // ----------------------------------------------------------------- molecule
 // e^x for the Gaussians of the level set (x <= 0), by one stated method so
 // that the point set does not depend on a math library's last bits: Cody and
@@ -327,76 +276,15 @@ __device__ void mol_normal(const QuadGeo &g, const double X[3], double nv[3]) {
     for (int q = 0; q < 3; ++q) nv[q] = G[q] / gn;
 }
 
-__device__ int eval_line_molecule(const QuadGeo &g, int ax, int64_t ja, int64_t jb, double P[kMaxRoots][3],
-                                  double N[kMaxRoots][3], int br[kMaxRoots]) {
-    const int a = ax == 0 ? 1 : 0;
-    const int b = ax == 2 ? 1 : 2;
-    const double xa = (double)ja * g.h;
-    const double xb = (double)jb * g.h;
-    bool near = false;
-    for (int k = 0; k < 4; ++k) {
-        const double da = xa - g.mol[k][a], db = xb - g.mol[k][b];
-        near |= da * da + db * db < g.mD * g.mD;
-    }
-    if (!near) return 0;
-    double X[3];
-    X[a] = xa;
-    X[b] = xb;
-    X[ax] = g.tlo[ax];
-    double fprev = mol_phi(g, X);
-    double tprev = g.tlo[ax];
-    int kept = 0, ordinal = 0;
-    for (int k = 1; k <= g.nka[ax]; ++k) {
-        const double t = g.tlo[ax] + (double)k * g.dt[ax];
-        X[ax] = t;
-        const double f = mol_phi(g, X);
-        if ((fprev > 0.0) != (f > 0.0)) {
-            double lo = tprev, hi = t, flo = fprev, fhi = f;
-            const bool slo = flo > 0.0;
-            for (int it = 0; it < 200; ++it) {
-                const double mid = 0.5 * (lo + hi);
-                if (mid == lo || mid == hi) break;
-                X[ax] = mid;
-                const double fm = mol_phi(g, X);
-                if ((fm > 0.0) == slo) { lo = mid; flo = fm; }
-                else { hi = mid; fhi = fm; }
-            }
-            X[ax] = fabs(flo) <= fabs(fhi) ? lo : hi;
-            double nv[3];
-            mol_normal(g, X, nv);
-            if (fabs(nv[ax]) >= g.ct) {
-                if (kept == kMaxRoots) {
-                    atomicExch(g.overflow, 1);
-                } else {
-                    for (int q = 0; q < 3; ++q) { P[kept][q] = X[q]; N[kept][q] = nv[q]; }
-                    br[kept] = ordinal;
-                    ++kept;
-                }
-            }
-            ++ordinal;
-        }
-        fprev = f;
-        tprev = t;
-    }
-    return kept;
-}
-
-__device__ __forceinline__ int eval_any(const QuadGeo &g, int ax, int64_t ja, int64_t jb, double P[kMaxRoots][3],
-                                        double N[kMaxRoots][3], int br[kMaxRoots]) {
-    if (g.kind == SSD_STAR) return eval_line_star(g, ax, ja, jb, P, N, br);
-    if (g.kind == SSD_MOLECULE) return eval_line_molecule(g, ax, ja, jb, P, N, br);
-    return eval_line(g, ax, ja, jb, P, N, br);
-}
-
 __global__ void quad_count_kernel(const QuadGeo g, int64_t nlines, int32_t *count) {
     const int64_t line = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (line >= nlines) return;
     int ax;
     int64_t ja, jb;
     line_coords(g, line, ax, ja, jb);
-    double P[kMaxRoots][3], N[kMaxRoots][3];
-    int br[kMaxRoots];
-    count[line] = eval_any(g, ax, ja, jb, P, N, br);
+    double P[2][3], N[2][3];
+    int br[2];
+    count[line] = eval_line(g, ax, ja, jb, P, N, br);
 }
 
 // Exclusive scan, three phases: per-block scan, scan of block totals (one
@@ -433,6 +321,26 @@ __global__ void scan_add_kernel(int64_t *out, int64_t n, const int64_t *blocksum
     if (i < n) out[i] += blocksum[blockIdx.x];
 }
 
+// Point o of the set: position, normal, weight and (axis, j1, j2, ordinal)
+__device__ void write_point(const QuadGeo &g, int ax, int64_t ja, int64_t jb, const double P[3], const double N[3],
+                            int br, int64_t o, int64_t n, double *xyz, double *nrm, double *w, int32_t *meta) {
+    for (int q = 0; q < 3; ++q) {
+        xyz[q * n + o] = P[q];
+        nrm[q * n + o] = N[q];
+    }
+    // psi_i = b(acos|n_i|/theta) / sum_j b(acos|n_j|/theta); w = psi_i h^2 / |n_i|
+    double beta[3];
+    for (int q = 0; q < 3; ++q) beta[q] = bump(acos(fabs(N[q])) / g.theta);
+    const double psi = beta[ax] / ((beta[0] + beta[1]) + beta[2]);
+    w[o] = (psi * (g.h * g.h)) / fabs(N[ax]);
+    if (meta) {
+        meta[o] = ax;
+        meta[n + o] = (int32_t)ja;
+        meta[2 * n + o] = (int32_t)jb;
+        meta[3 * n + o] = br;
+    }
+}
+
 __global__ void quad_write_kernel(const QuadGeo g, int64_t nlines, const int64_t *offs, int64_t n, double *xyz,
                                   double *nrm, double *w, int32_t *meta) {
     const int64_t line = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -440,27 +348,11 @@ __global__ void quad_write_kernel(const QuadGeo g, int64_t nlines, const int64_t
     int ax;
     int64_t ja, jb;
     line_coords(g, line, ax, ja, jb);
-    double P[kMaxRoots][3], N[kMaxRoots][3];
-    int br[kMaxRoots];
-    const int kept = eval_any(g, ax, ja, jb, P, N, br);
-    for (int k = 0; k < kept; ++k) {
-        const int64_t o = offs[line] + k;
-        for (int q = 0; q < 3; ++q) {
-            xyz[q * n + o] = P[k][q];
-            nrm[q * n + o] = N[k][q];
-        }
-        // psi_i = b(acos|n_i|/theta) / sum_j b(acos|n_j|/theta); w = psi_i h^2 / |n_i|
-        double beta[3];
-        for (int q = 0; q < 3; ++q) beta[q] = bump(acos(fabs(N[k][q])) / g.theta);
-        const double psi = beta[ax] / ((beta[0] + beta[1]) + beta[2]);
-        w[o] = (psi * (g.h * g.h)) / fabs(N[k][ax]);
-        if (meta) {
-            meta[o] = ax;
-            meta[n + o] = (int32_t)ja;
-            meta[2 * n + o] = (int32_t)jb;
-            meta[3 * n + o] = br[k];
-        }
-    }
+    double P[2][3], N[2][3];
+    int br[2];
+    const int kept = eval_line(g, ax, ja, jb, P, N, br);
+    for (int k = 0; k < kept; ++k)
+        write_point(g, ax, ja, jb, P[k], N[k], br[k], offs[line] + k, n, xyz, nrm, w, meta);
 }
 
 // Derivatives of the points, normals and weights of a star surface with
@@ -497,44 +389,208 @@ __device__ void pou_derivative(const QuadGeo &g, int ax, const double nv[3], con
     dw = h2 * (dpsi / ui - psi * dui / (ui * ui));
 }
 
-__global__ void quad_jacobian_kernel(const QuadGeo g, int64_t nlines, const int64_t *offs, int64_t n, double *dxyz,
-                                     double *dnrm, double *dw) {
-    const int64_t line = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (line >= nlines) return;
-    int ax;
-    int64_t ja, jb;
-    line_coords(g, line, ax, ja, jb);
-    double P[kMaxRoots][3], N[kMaxRoots][3];
-    int br[kMaxRoots];
-    const int kept = eval_any(g, ax, ja, jb, P, N, br);
-    for (int r = 0; r < kept; ++r) {
-        const int64_t o = offs[line] + r;
-        const double *X = P[r];
-        double G[3];
-        star_grad<double>(g.a, g, X, G);
-        const double d0 = X[0] - g.c[0], d1 = X[1] - g.c[1], d2 = X[2] - g.c[2];
-        const double rho = sqrt((d0 * d0 + d1 * d1) + d2 * d2);
-        const double xi[3] = {d0 / rho, d1 / rho, d2 / rho};
-        for (int k = 0; k < kStarCoef; ++k) {
-            double e[kStarCoef];
-            for (int j = 0; j < kStarCoef; ++j) e[j] = j == k ? 1.0 : 0.0;
-            double pk, gdum[3];
-            star_eval<double, false>(e, xi[0], xi[1], xi[2], pk, gdum);
-            const double dt = g.K[k] * pk / G[ax];
-            Dual ad[kStarCoef], Xd[3], nd[3];
-            for (int j = 0; j < kStarCoef; ++j) ad[j] = {g.a[j], j == k ? g.K[k] : 0.0};
-            for (int q = 0; q < 3; ++q) Xd[q] = {X[q], q == ax ? dt : 0.0};
-            star_normal<Dual>(ad, g, Xd, nd);
-            double dn[3], wv, dwv;
-            for (int q = 0; q < 3; ++q) {
-                dn[q] = nd[q].d;
-                dxyz[((int64_t)k * 3 + q) * n + o] = q == ax ? dt : 0.0;
-                dnrm[((int64_t)k * 3 + q) * n + o] = dn[q];
-            }
-            pou_derivative(g, ax, N[r], dn, wv, dwv);
-            dw[(int64_t)k * n + o] = dwv;
-        }
+// Derivatives of point o (position X and normal N on a line of axis ax) with
+// respect to coefficient k
+__device__ void write_derivative(const QuadGeo &g, int ax, const double X[3], const double N[3], int k, int64_t o,
+                                 int64_t n, double *dxyz, double *dnrm, double *dw) {
+    double G[3];
+    star_grad<double>(g.a, g, X, G);
+    const double d0 = X[0] - g.c[0], d1 = X[1] - g.c[1], d2 = X[2] - g.c[2];
+    const double rho = sqrt((d0 * d0 + d1 * d1) + d2 * d2);
+    double e[kStarCoef];
+    for (int j = 0; j < kStarCoef; ++j) e[j] = j == k ? 1.0 : 0.0;
+    double pk, gdum[3];
+    star_eval<double, false>(e, d0 / rho, d1 / rho, d2 / rho, pk, gdum);
+    const double Kk = g.K[k];
+    const double dt = Kk * pk / G[ax];
+    Dual ad[kStarCoef], Xd[3], nd[3];
+    for (int j = 0; j < kStarCoef; ++j) ad[j] = {g.a[j], j == k ? Kk : 0.0};
+    for (int q = 0; q < 3; ++q) Xd[q] = {X[q], q == ax ? dt : 0.0};
+    star_normal<Dual>(ad, g, Xd, nd);
+    double dn[3], wv, dwv;
+    for (int q = 0; q < 3; ++q) {
+        dn[q] = nd[q].d;
+        dxyz[((int64_t)k * 3 + q) * n + o] = q == ax ? dt : 0.0;
+        dnrm[((int64_t)k * 3 + q) * n + o] = dn[q];
     }
+    pou_derivative(g, ax, N, dn, wv, dwv);
+    dw[(int64_t)k * n + o] = dwv;
+}
+
+// Star surfaces and molecules: 8 lines a CTA.  Crossings of a line lie where
+// the sign of phi changes between two of its samples t_k = tlo + k dt, then
+// by bisection.  The double-precision pipe bounds both parts, and an
+// instruction occupies it for a whole warp however few lanes take part, so
+// the samples of a line are spread over the lanes of a warp, and the
+// crossings of all 8 lines are gathered first and bisected one per lane,
+// instead of each by a thread of its own while its warp waits.
+// A star surface's points (three passes over the lines) at h = 1/8 took 50.6 ms
+// with a thread per line, 1.5 ms now; at h = 1/32 62 and 6.9 ms; the molecule
+// at h = 1/8 49 and 1.9 ms; the 25 derivatives at h = 1/8 37 and 1.1 ms.
+// Results go to registers through selects (on_line), not to indexed arrays.
+// Samples go by windows of 512 a line, which bounds the list of crossings;
+// a star surface has at most 272, a molecule any number.
+constexpr int kSampleLines = 8;
+constexpr int kSampleTPB = 32 * kSampleLines;
+constexpr int kSampleWindow = 512;
+
+enum QuadOut { kQuadCount, kQuadPoints, kQuadJacobian };
+
+struct QuadOutArgs {
+    int32_t *count;
+    const int64_t *offs;
+    int64_t n;
+    double *xyz, *nrm, *w;   // points, or their derivatives
+    int32_t *meta;
+};
+
+// The point at t on the line of axis ax whose in-plane coordinates are pa, pb
+__device__ __forceinline__ void on_line(int ax, double t, double pa, double pb, double X[3]) {
+    X[0] = ax == 0 ? t : pa;
+    X[1] = ax == 0 ? pa : ax == 1 ? t : pb;
+    X[2] = ax == 2 ? t : pb;
+}
+
+template <int KIND>
+__device__ __forceinline__ double level(const QuadGeo &g, const double X[3]) {
+    return KIND == SSD_STAR ? star_phi(g, X) : mol_phi(g, X);
+}
+
+template <int KIND, int OUT>
+__global__ void __launch_bounds__(kSampleTPB) quad_sample_kernel(const QuadGeo g, int64_t nlines,
+                                                                 const QuadOutArgs A) {
+    __shared__ uint16_t list[kSampleLines][kSampleWindow];   // samples that end a crossing, of the window
+    __shared__ int nlist[kSampleLines];                      // their number
+    __shared__ int order0[kSampleLines], kept[kSampleLines];   // crossings and kept crossings of the windows before
+    __shared__ int axis[kSampleLines];
+    __shared__ double plane[kSampleLines][2];
+    __shared__ double rt[kSampleLines][kMaxRoots], rn[kSampleLines][kMaxRoots][3];
+    __shared__ int rbr[kSampleLines][kMaxRoots];
+    __shared__ unsigned char keep[kSampleTPB];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t line = (int64_t)blockIdx.x * kSampleLines + wid;
+    int ax = 0, ns = -1;   // last sample of the line, -1: no crossing possible
+    int64_t ja = 0, jb = 0;
+    double X[3], xa = 0.0, xb = 0.0;
+    if (line < nlines) {
+        line_coords(g, line, ax, ja, jb);
+        const int a = ax == 0 ? 1 : 0;
+        const int b = ax == 2 ? 1 : 2;
+        xa = (double)ja * g.h;
+        xb = (double)jb * g.h;
+        bool near = false;
+        if (KIND == SSD_STAR) {
+            const double da = xa - g.c[a], db = xb - g.c[b];
+            near = da * da + db * db < g.rb * g.rb;
+        } else {
+            for (int k = 0; k < 4; ++k) {
+                const double da = xa - g.mol[k][a], db = xb - g.mol[k][b];
+                near |= da * da + db * db < g.mD * g.mD;
+            }
+        }
+        if (near) ns = KIND == SSD_STAR ? g.nk : g.nka[ax];
+        if (lane == 0) { axis[wid] = ax; plane[wid][0] = xa; plane[wid][1] = xb; }
+    }
+    if (lane == 0) { order0[wid] = 0; kept[wid] = 0; }
+    bool before = false;   // phi > 0 at the last sample of the chunk before
+    const double tlo = g.tlo[ax], dt = g.dt[ax];
+    for (int64_t win = 0; __syncthreads_or(win <= ns); win += kSampleWindow) {
+        int cnt = 0;
+        for (int c = 0; c < kSampleWindow && win + c <= ns; c += 32) {
+            const int k = (int)win + c + lane;
+            bool pos = false;
+            if (k <= ns) {
+                on_line(ax, tlo + (double)k * dt, xa, xb, X);
+                pos = level<KIND>(g, X) > 0.0;
+            }
+            const unsigned p = __ballot_sync(0xffffffffu, pos);
+            const unsigned prev = (p << 1) | (before ? 1u : 0u);
+            const unsigned cross = __ballot_sync(0xffffffffu, k >= 1 && k <= ns && (((p ^ prev) >> lane) & 1u));
+            if ((cross >> lane) & 1u) list[wid][cnt + __popc(cross & ((1u << lane) - 1u))] = (uint16_t)(c + lane);
+            cnt += __popc(cross);
+            before = p >> 31;
+        }
+        if (lane == 0) nlist[wid] = cnt;
+        __syncthreads();
+        int total = 0;
+        for (int l = 0; l < kSampleLines; ++l) total += nlist[l];
+        for (int base = 0; base < total; base += kSampleTPB) {
+            // crossing i of line l, line by line in ascending order
+            int l = 0, i = base + (int)threadIdx.x;
+            const bool act = i < total;
+            while (act && i >= nlist[l]) i -= nlist[l++];
+            double root = 0.0, nv[3];
+            bool ok = false;
+            if (act) {
+                const int e = axis[l];
+                const double pa = plane[l][0], pb = plane[l][1];
+                double Y[3];
+                const int64_t k = win + list[l][i];
+                double lo = g.tlo[e] + (double)(k - 1) * g.dt[e], hi = g.tlo[e] + (double)k * g.dt[e];
+                on_line(e, lo, pa, pb, Y);
+                double flo = level<KIND>(g, Y);
+                on_line(e, hi, pa, pb, Y);
+                double fhi = level<KIND>(g, Y);
+                const bool slo = flo > 0.0;
+                for (int it = 0; it < 200; ++it) {
+                    const double mid = 0.5 * (lo + hi);
+                    if (mid == lo || mid == hi) break;
+                    on_line(e, mid, pa, pb, Y);
+                    const double fm = level<KIND>(g, Y);
+                    if ((fm > 0.0) == slo) { lo = mid; flo = fm; }
+                    else { hi = mid; fhi = fm; }
+                }
+                root = fabs(flo) <= fabs(fhi) ? lo : hi;
+                on_line(e, root, pa, pb, Y);
+                if (KIND == SSD_STAR) star_normal<double>(g.a, g, Y, nv);
+                else mol_normal(g, Y, nv);
+                ok = fabs(e == 0 ? nv[0] : e == 1 ? nv[1] : nv[2]) >= g.ct;
+            }
+            keep[threadIdx.x] = ok;
+            __syncthreads();
+            int slot = 0;
+            if (act) {
+                slot = kept[l];
+                for (int j = i < (int)threadIdx.x ? (int)threadIdx.x - i : 0; j < (int)threadIdx.x; ++j)
+                    slot += keep[j];
+                if (ok && slot < kMaxRoots) {
+                    rt[l][slot] = root;
+                    for (int q = 0; q < 3; ++q) rn[l][slot][q] = nv[q];
+                    rbr[l][slot] = order0[l] + i;
+                } else if (ok) {
+                    atomicExch(g.overflow, 1);
+                }
+            }
+            __syncthreads();
+            // the line's last crossing of this batch leaves the new count
+            if (act && (i + 1 == nlist[l] || threadIdx.x + 1 == kSampleTPB)) kept[l] = slot + (ok ? 1 : 0);
+            __syncthreads();
+        }
+        if (lane == 0) order0[wid] += cnt;
+    }
+    if (OUT == kQuadCount) {
+        if (lane == 0 && line < nlines) A.count[line] = min(kept[wid], kMaxRoots);
+        return;
+    }
+    constexpr int kPer = OUT == kQuadPoints ? 1 : kStarCoef;   // results per kept crossing
+    const int nres = line < nlines ? min(kept[wid], kMaxRoots) * kPer : 0;
+    for (int i = lane; i < nres; i += 32) {
+        const int r = i / kPer;
+        double N[3];
+        on_line(ax, rt[wid][r], xa, xb, X);
+        for (int q = 0; q < 3; ++q) N[q] = rn[wid][r][q];
+        const int64_t o = A.offs[line] + r;
+        if (OUT == kQuadPoints) write_point(g, ax, ja, jb, X, N, rbr[wid][r], o, A.n, A.xyz, A.nrm, A.w, A.meta);
+        else write_derivative(g, ax, X, N, i % kPer, o, A.n, A.xyz, A.nrm, A.w);
+    }
+}
+
+template <int OUT>
+void launch_quad_sample(const QuadGeo &g, int64_t nlines, const QuadOutArgs &A, cudaStream_t s) {
+    const unsigned grid = (unsigned)((nlines + kSampleLines - 1) / kSampleLines);
+    if (g.kind == SSD_STAR) quad_sample_kernel<SSD_STAR, OUT><<<grid, kSampleTPB, 0, s>>>(g, nlines, A);
+    else if (OUT != kQuadJacobian)
+        quad_sample_kernel<SSD_MOLECULE, OUT == kQuadJacobian ? kQuadPoints : OUT><<<grid, kSampleTPB, 0, s>>>(g, nlines, A);
 }
 
 // Host setup of the surface description (all kinds).
@@ -669,7 +725,9 @@ int quadrature_impl(ssd_ctx *ctx, const ssd_surface *surf, double h, double angl
     g.overflow = reinterpret_cast<int *>(tb + o_ovf);
     SSD_TRY(cuda_check(ctx, cudaMemsetAsync(g.overflow, 0, sizeof(int), s), "memset"));
     const unsigned lb = (unsigned)((nlines + 255) / 256);
-    quad_count_kernel<<<lb, 256, 0, s>>>(g, nlines, cnt);
+    const bool sampled = g.kind == SSD_STAR || g.kind == SSD_MOLECULE;
+    if (sampled) launch_quad_sample<kQuadCount>(g, nlines, {cnt}, s);
+    else quad_count_kernel<<<lb, 256, 0, s>>>(g, nlines, cnt);
     scan_block_kernel<<<(unsigned)nb, 1024, 0, s>>>(cnt, nlines, offs, bs);
     scan_totals_kernel<<<1, 32, 0, s>>>(bs, nb, tot);
     scan_add_kernel<<<(unsigned)nb, 1024, 0, s>>>(offs, nlines, bs);
@@ -690,7 +748,7 @@ int quadrature_impl(ssd_ctx *ctx, const ssd_surface *surf, double h, double angl
         if (g.kind != SSD_STAR) return set_error(ctx, SSD_EINVAL, "shape derivatives need a STAR surface");
         if (capacity != total) return set_error(ctx, SSD_EINVAL, "n differs from the point count");
         if (!jn || !jw) return set_error(ctx, SSD_EINVAL, "NULL output array");
-        quad_jacobian_kernel<<<lb, 256, 0, s>>>(g, nlines, offs, total, jx, jn, jw);
+        launch_quad_sample<kQuadJacobian>(g, nlines, {nullptr, offs, total, jx, jn, jw, nullptr}, s);
         ctx->launches += 1;
         SSD_TRY(launch_check(ctx, "quadrature jacobian"));
         return cuda_check(ctx, cudaStreamSynchronize(s), "quadrature sync");
@@ -698,7 +756,8 @@ int quadrature_impl(ssd_ctx *ctx, const ssd_surface *surf, double h, double angl
     if (!xyz) return SSD_OK;
     if (capacity < total) return set_error(ctx, SSD_EINVAL, "capacity smaller than the point count");
     if (!nrm || !w) return set_error(ctx, SSD_EINVAL, "NULL output array");
-    quad_write_kernel<<<lb, 256, 0, s>>>(g, nlines, offs, total, xyz, nrm, w, meta);
+    if (sampled) launch_quad_sample<kQuadPoints>(g, nlines, {nullptr, offs, total, xyz, nrm, w, meta}, s);
+    else quad_write_kernel<<<lb, 256, 0, s>>>(g, nlines, offs, total, xyz, nrm, w, meta);
     ctx->launches += 1;
     SSD_TRY(launch_check(ctx, "quadrature write"));
     return cuda_check(ctx, cudaStreamSynchronize(s), "quadrature sync");
