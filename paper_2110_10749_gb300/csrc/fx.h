@@ -222,12 +222,12 @@ FX_HD void fx_mac(FxMac &a, const FxB &b, int gh, int gl) {
     a.l1 = fx_mw(b.b0, gh, a.l1);
     a.l2 = fx_mw(b.b1, gl, a.l2);
 }
-// the sum in units of 2^55 of f's and g's last places
-FX_HD double fx_value(const FxMac &a) {
+// the sum is h 2^24 + fx_low in units of 2^55 of f's and g's last places
+FX_HD int64_t fx_low(const FxMac &a) {
     const int64_t l = a.l1 + (a.l2 >> 7);
-    const int64_t m = a.m1 + (a.m2 >> 7) + (l >> 24);
-    return (double)a.h * 16777216.0 + (double)m;
+    return a.m1 + (a.m2 >> 7) + (l >> 24);
 }
+FX_HD double fx_value(const FxMac &a) { return (double)a.h * 16777216.0 + (double)fx_low(a); }
 
 // Kernel tables of sigma_1 .. sigma_4 on v in [1, 2^kFxMaxOct), then t^(-1/2) on
 // t in [1, 4): host array of kFxTabEntries entries, built once per process

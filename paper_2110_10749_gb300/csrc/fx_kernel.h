@@ -143,8 +143,8 @@ constexpr int kFxFarOct = 6;                     // 1 + 8^2 > 2^6
 template <int OP, bool FAR> constexpr int fx_ntab() { return FAR && OP == OP_SSL ? 1 : FxOp<OP>::ntab; }
 
 // GROUPS > 1: the threads form groups that share the CTA's 256 / GROUPS targets
-// and take sources grp, grp + GROUPS, .. of each staged tile; their sums are
-// added in order at the end.
+// and take sources grp, grp + GROUPS, .. of each staged tile; their integer
+// sums are added before they become a double.
 template <int OP, bool FAR, int GROUPS>
 __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
     typedef FxOp<OP> T;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
     __shared__ int4 s_uh[VU ? kTile : 1], s_ul[VU ? kTile : 1];
     __shared__ int4 s_fh[VF ? kTile : 1], s_fl[VF ? kTile : 1];
     __shared__ unsigned long long s_max[2][kFxTPB / 32];
-    __shared__ double s_sum[GROUPS > 1 ? NC : 1][GROUPS > 1 ? kFxTPB : 1];
+    __shared__ int64_t s_acc[GROUPS > 1 ? 2 * NC : 1][GROUPS > 1 ? kFxTPB : 1];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t tbase, s_beg, s_end, part_base, pstride, b0 = 0, b1 = a.nblk;
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             tl.oct0 -= kOct0 * kFxSeg;
             const int ks = 61 - L - g.ps;
             auto grid = [&](int64_t v) { return ks >= 0 ? (int64_t)((uint64_t)v << ks) : v >> -ks; };
-            __syncthreads();
+            if constexpr (GROUPS == 1) __syncthreads();   // (with groups the one before their sums)
             if (threadIdx.x < cnt) {
                 const int64_t j = tile + threadIdx.x;
                 const l4 p = a.X[j];
@@ -364,27 +364,57 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             }
             const double f = __longlong_as_double((long long)(1023 + tl.ex) << 52) *
                              (T::fused || !T::dl ? g.f_sl : g.f_dl);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {   // TwoSum: the tiles add no rounding of their own
-                double v;
-                if constexpr (T::vec) v = fx_value(acc.v[c]) * f;
-                else v = ((double)acc.f.h + (double)acc.f.l * 2.3283064365386963e-10) * f;
+            auto value = [&](int64_t h, int64_t l) {   // of a component's two integers
+                return T::vec ? ((double)h * 16777216.0 + (double)l) * f
+                              : ((double)h + (double)l * 2.3283064365386963e-10) * f;
+            };
+            auto add = [&](int c, double v) {   // TwoSum: the tiles add no rounding of their own
                 const double t = sum[c] + v, b = t - sum[c];
                 low[c] += (sum[c] - (t - b)) + (v - b);
                 sum[c] = t;
+            };
+            if constexpr (GROUPS == 1) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    if constexpr (T::vec) add(c, value(acc.v[c].h, fx_low(acc.v[c])));
+                    else add(c, value(acc.f.h, acc.f.l));
+                }
+            } else {
+                // The groups' integers are added first, exactly: together they hold the
+                // tile's 128 terms.  A thread then takes one component of one target.
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    if constexpr (T::vec) {
+                        s_acc[c][threadIdx.x] = acc.v[c].h;
+                        s_acc[NC + c][threadIdx.x] = fx_low(acc.v[c]);
+                    } else {
+                        s_acc[0][threadIdx.x] = acc.f.h;
+                        s_acc[1][threadIdx.x] = acc.f.l;
+                    }
+                }
+                __syncthreads();
+                if (grp < NC) {
+                    int64_t h = 0, l = 0;
+#pragma unroll
+                    for (int q = 0; q < GROUPS; ++q) {
+                        h += s_acc[grp][q * nt + threadIdx.x % nt];
+                        l += s_acc[NC + grp][q * nt + threadIdx.x % nt];
+                    }
+                    add(0, value(h, l));
+                }
             }
         }
 #pragma unroll
         for (int c = 0; c < NC; ++c) sum[c] += low[c];
     }
-    if constexpr (GROUPS > 1) {   // the groups' sums, in order
-#pragma unroll
-        for (int q = 0; q < NC; ++q) s_sum[q][threadIdx.x] = sum[q];
-        __syncthreads();
-        if (grp) return;
-        for (int g = 1; g < GROUPS; ++g)
-#pragma unroll
-            for (int q = 0; q < NC; ++q) sum[q] += s_sum[q][threadIdx.x + g * nt];
+    if constexpr (GROUPS > 1) {
+        if (grp >= (bad ? 1 : NC)) return;
+        if (!bad) {   // component grp of target i
+            const int64_t q = grp;
+            if (a.k.acc) atomicAdd(a.k.acc + q * a.k.n_pad + i, sum[0]);
+            else a.k.part[part_base + q * pstride + i] = sum[0];
+            return;
+        }
     }
     if (a.k.acc) {
 #pragma unroll
