@@ -200,8 +200,29 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q * 16u), "l"(src + q));
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    // and, where it pays, the target's grid position and its block's box, which are
+    // kept with the layout: Stokes double layer at N = 17070 3.37 ms, 3.48 with these
+    // loads after the scale and the tile's boxes one by one; transposed at N = 4302
+    // 339 and 350 us; the Laplace layers and the Stokes single layer of large sets
+    // lose 0.5%.
+    constexpr bool kEarly = GROUPS > 1 || (T::vec && T::dl);
+    l4 Y;
+    d4 Yd;
+    int tlo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, thi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
+    auto grow = [&](int (&lo)[3], int (&hi)[3], int64_t box) {
+        const int4 l = a.cbox[2 * box], h = a.cbox[2 * box + 1];
+        lo[0] = min(lo[0], l.x); lo[1] = min(lo[1], l.y); lo[2] = min(lo[2], l.z);
+        hi[0] = max(hi[0], h.x); hi[1] = max(hi[1], h.y); hi[2] = max(hi[2], h.z);
+    };
+    auto load_target = [&] {
+        Y = a.X[i];
+#pragma unroll
+        for (int k = 0; k < nt / kChunk; ++k) grow(tlo, thi, tbase / kChunk + k);
+    };
+    if constexpr (kEarly) load_target();
     pdl_wait();
     pdl_release();
+    if constexpr (kEarly) Yd = d0[i];
     // largest densities of this surface and right-hand side
     {
         unsigned long long m0 = 0, m1 = 0;
@@ -233,28 +254,21 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
         const FxGeo &g = *gp;
         const FxScale sc = fx_scale<OP>(ee[0], ee[1], g.em, g.dq, g.ed);
         FxPoint<OP> y;
-        const l4 Y = a.X[i];
-        {
-            const d4 d = d0[i];
-            if constexpr (VU) {
-                fx_split(fx_fix(d.x, sc.eu, 58), y.u.h[0], y.u.l[0]);
-                fx_split(fx_fix(d.y, sc.eu, 58), y.u.h[1], y.u.l[1]);
-                fx_split(fx_fix(d.z, sc.eu, 58), y.u.h[2], y.u.l[2]);
-            }
-            if constexpr (!T::vec && T::dl) y.p = fx_fix(d.x, sc.eu, 60);
-            if constexpr (T::tr) {
-                const d4 m = a.k.wn[i];
-                fx_split(fx_fix(m.x, sc.em, 59), y.m.h[0], y.m.l[0]);
-                fx_split(fx_fix(m.y, sc.em, 59), y.m.h[1], y.m.l[1]);
-                fx_split(fx_fix(m.z, sc.em, 59), y.m.h[2], y.m.l[2]);
-            }
+        if constexpr (!kEarly) {
+            load_target();
+            Yd = d0[i];
         }
-        int tlo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, thi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
-#pragma unroll
-        for (int k = 0; k < nt / kChunk; ++k) {
-            const int4 l = a.cbox[2 * (tbase / kChunk + k)], h = a.cbox[2 * (tbase / kChunk + k) + 1];
-            tlo[0] = min(tlo[0], l.x); tlo[1] = min(tlo[1], l.y); tlo[2] = min(tlo[2], l.z);
-            thi[0] = max(thi[0], h.x); thi[1] = max(thi[1], h.y); thi[2] = max(thi[2], h.z);
+        if constexpr (VU) {
+            fx_split(fx_fix(Yd.x, sc.eu, 58), y.u.h[0], y.u.l[0]);
+            fx_split(fx_fix(Yd.y, sc.eu, 58), y.u.h[1], y.u.l[1]);
+            fx_split(fx_fix(Yd.z, sc.eu, 58), y.u.h[2], y.u.l[2]);
+        }
+        if constexpr (!T::vec && T::dl) y.p = fx_fix(Yd.x, sc.eu, 60);
+        if constexpr (T::tr) {
+            const d4 m = a.k.wn[i];
+            fx_split(fx_fix(m.x, sc.em, 59), y.m.h[0], y.m.l[0]);
+            fx_split(fx_fix(m.y, sc.em, 59), y.m.h[1], y.m.l[1]);
+            fx_split(fx_fix(m.z, sc.em, 59), y.m.h[2], y.m.l[2]);
         }
         const uint32_t idx_max = (uint32_t)((a.noct - kOct0) * kFxSeg - 1);
         const int4 *tab4 = reinterpret_cast<const int4 *>(s_tab);
@@ -268,10 +282,12 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             int dmax = 0, gap = 0;
             {
                 int slo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, shi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
-                for (int k = 0; k < cnt / kChunk; ++k) {
-                    const int4 l = a.cbox[2 * (tile / kChunk + k)], h = a.cbox[2 * (tile / kChunk + k) + 1];
-                    slo[0] = min(slo[0], l.x); slo[1] = min(slo[1], l.y); slo[2] = min(slo[2], l.z);
-                    shi[0] = max(shi[0], h.x); shi[1] = max(shi[1], h.y); shi[2] = max(shi[2], h.z);
+                if constexpr (kEarly) {   // overlapping loads (a short tile's last box again)
+                    const int top = cnt / kChunk - 1;
+#pragma unroll
+                    for (int k = 0; k < kTile / kChunk; ++k) grow(slo, shi, tile / kChunk + (k < top ? k : top));
+                } else {
+                    for (int k = 0; k < cnt / kChunk; ++k) grow(slo, shi, tile / kChunk + k);
                 }
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -339,7 +355,8 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             FxSum<OP> acc{};
             // 4 pairs in flight fill the wide multiplier's latency (Stokes double layer
             // 3.10 clocks per pair and SM against 3.50 unrolled once; the transposed
-            // Stokes layer has no registers left beyond 2)
+            // Stokes layer has no registers left beyond 2).  3 resident CTAs of the Laplace
+            // layers with 2 pairs in flight are slower: 2.29 ms against 2.20 at N = 17070.
             constexpr int kUnroll = OP == OP_SDLT ? 2 : 4;
 #pragma unroll kUnroll
             for (int j = grp; j < cnt; j += GROUPS) {
