@@ -31,6 +31,7 @@
 // generic kernel (fx_geo).
 
 constexpr int kFxGroups = 4;   // source groups of a CTA on small sets
+constexpr int kFxUnit = 8;     // and the granularity of their chunks of sources
 
 struct FxArgs {
     const l4 *X;
@@ -277,15 +278,18 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             return FxI4{v.x, v.y, v.z, v.w};
         };
         for (int64_t tile = s_beg; tile < s_end; tile += kTile) {
-            const int cnt = (int)(s_end - tile < kTile ? s_end - tile : kTile);   // a multiple of kChunk
+            const int cnt = (int)(s_end - tile < kTile ? s_end - tile : kTile);   // a multiple of kChunk, or of kFxUnit
             // the tile's largest distance exponent L and a lower bound 2^r of its distances
             int dmax = 0, gap = 0;
             {
                 int slo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, shi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
                 if constexpr (kEarly) {   // overlapping loads (a short tile's last box again)
-                    const int top = cnt / kChunk - 1;
+                    // (tiles of small sets start and end at multiples of kFxUnit)
+                    constexpr int kBoxes = kTile / kChunk + (GROUPS > 1 ? 1 : 0);
+                    const int64_t b = tile / kChunk;
+                    const int top = (int)((tile + cnt - 1) / kChunk - b);
 #pragma unroll
-                    for (int k = 0; k < kTile / kChunk; ++k) grow(slo, shi, tile / kChunk + (k < top ? k : top));
+                    for (int k = 0; k < kBoxes; ++k) grow(slo, shi, b + (k < top ? k : top));
                 } else {
                     for (int k = 0; k < cnt / kChunk; ++k) grow(slo, shi, tile / kChunk + k);
                 }

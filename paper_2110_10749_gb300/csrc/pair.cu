@@ -1683,8 +1683,11 @@ size_t fx_geo_bytes(int nsurf) { return sizeof(FxGeo) * nsurf; }
 // fill the SMs evenly.  Small sets: at most one round of two CTAs per SM, the
 // grouped form where its finer items leave less to the fullest CTA (N = 1062:
 // 289 CTAs of 64 targets, against 170 of 256: Stokes double layer 44 us instead
-// of 55 with its packing and epilogue; N = 1742: 280 against 196).  From 6000
-// points on about 5 rounds, which the scheduler levels.
+// of 55 with its packing and epilogue; N = 1742: 280 against 196).  Their chunks
+// go by 8 sources, not 32: at N = 1099 the fullest thread has 18 pairs instead of
+// 24 (value and gradients on a star surface 128.9 ms against 140.5), at N = 1742
+// 44 instead of 48 (fused Stokes layers 96.4 us against 103.4).  From 6000 points
+// on about 5 rounds, which the scheduler levels.
 struct FxSplit {
     int groups = 1;
     int64_t chunk = 0, nsplit = 1;
@@ -1699,13 +1702,14 @@ static FxSplit fx_split_grid(const ssd_ctx *ctx, int64_t n) {
         const int64_t span = kFxTPB / g, nt = (n + span - 1) / span;
         int64_t ns = want / nt;
         ns = ns < 1 ? 1 : (ns > units ? units : ns);
-        int64_t cu = (units + ns - 1) / ns;
-        if (cu > 8) cu = (cu + 3) / 4 * 4;   // whole staged tiles
-        if (g > 1 && (n >= 6000 || span * cu >= cost)) continue;   // pairs of the fullest CTA
-        cost = span * cu;
+        const int64_t per = (units * kChunk + ns - 1) / ns;
+        int64_t chunk = g > 1 ? (per + kFxUnit - 1) / kFxUnit * kFxUnit : (per + kChunk - 1) / kChunk * kChunk;
+        if (chunk > 256) chunk = (chunk + kTile - 1) / kTile * kTile;   // whole staged tiles
+        if (g > 1 && (n >= 6000 || span * chunk >= cost)) continue;   // pairs of the fullest CTA
+        cost = span * chunk;
         best.groups = g;
-        best.chunk = cu * kChunk;
-        best.nsplit = (units + cu - 1) / cu;
+        best.chunk = chunk;
+        best.nsplit = (units * kChunk + chunk - 1) / chunk;
     }
     return best;
 }
