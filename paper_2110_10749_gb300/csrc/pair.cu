@@ -1085,11 +1085,12 @@ __global__ void pack_kernel(const PackArgs a) {
     if (a.wdot_part) {
         red[threadIdx.x] = wd;
         __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) a.wdot_part[blockIdx.x] = red[0];
+        if (threadIdx.x >= 32) return;
+        const int t = threadIdx.x;   // a tree over the 256 threads: halves of 128, 64, 32, then across the warp
+        double v = ((red[t] + red[t + 128]) + (red[t + 64] + red[t + 192])) +
+                   ((red[t + 32] + red[t + 160]) + (red[t + 96] + red[t + 224]));
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+        if (t == 0) a.wdot_part[blockIdx.x] = v;
     }
 }
 
@@ -1117,80 +1118,109 @@ struct EpiArgs {
     int64_t row0 = 0, row1 = -1;   // only layout rows [row0, row1) are written (row1 < 0: all)
 };
 
-__global__ void epilogue_kernel(const EpiArgs a) {
-    // one thread per (point, component): partial sums are summed over the
-    // splits in a fixed order in FP64
+// One thread per (point, component) sums the splits' partials in a fixed order;
+// a fifth warp reduces the rank-one term meanwhile.  Latency bounds it (N = 1062:
+// 51 KB of partials), so whatever the packing and the pair kernel do not write is
+// read before the wait for the latter, and 16 splits are in flight at a time.
+// With its packing at N = 1062 (Stokes double layer, three launches) 28.5 us a
+// call, 30.0 when every load followed the wait and each four splits the last.
+constexpr int kEpiTPB = 128;
+
+__global__ void __launch_bounds__(kEpiTPB + 32) epilogue_kernel(const EpiArgs a) {
     __shared__ double extra, rank1;
+    const int64_t g = (int64_t)blockIdx.x * kEpiTPB + threadIdx.x;
+    const int q = (int)(g / a.n_pad);
+    const int64_t i = g - (int64_t)q * a.n_pad;
+    int32_t o = -1;
+    if (threadIdx.x < kEpiTPB && g < a.n_pad * a.nc && (a.row1 < 0 || (i >= a.row0 && i < a.row1))) o = a.perm[i];
+    double weight = 1.0, selfv = 0.0, nrm = 0.0, x = 0.0;
+    if (o >= 0) {
+        if (a.weight_out || a.self_src) weight = a.pos64[i].w;
+        if (a.self_src) selfv = a.self_src[(int64_t)q * a.n + o];
+        if (a.rank1_nrm) nrm = a.rank1_nrm[(int64_t)q * a.n + o];
+        if (a.xin) x = a.xin[(int64_t)q * a.n + o];
+    }
     pdl_wait();
     pdl_release();
-    if (threadIdx.x < 32) {
+    if (threadIdx.x >= kEpiTPB) {
+        const int lane = threadIdx.x - kEpiTPB;
         double s = 0.0;
         if (a.wdot_part) {   // one warp, fixed order (a serial sum of N / 256 parts took longer than the rest)
-            for (int k = threadIdx.x; k < a.nwdot; k += 32) s += a.wdot_part[k];
+            for (int k = lane; k < a.nwdot; k += 32) s += a.wdot_part[k];
             for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
             s *= a.wdot_scale;
         }
-        if (threadIdx.x == 0) {
+        if (lane == 0) {
             extra = (a.add_dev ? *a.add_dev : 0.0) + (a.rank1_nrm ? 0.0 : s);
             rank1 = a.rank1_nrm ? s : 0.0;
         }
     }
-    __syncthreads();
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= a.n_pad * a.nc) return;
-    const int q = (int)(g / a.n_pad);
-    const int64_t i = g - (int64_t)q * a.n_pad;
-    if (a.row1 >= 0 && (i < a.row0 || i >= a.row1)) return;
-    const int32_t o = a.perm[i];
-    if (o < 0) return;
-    // four interleaved partial sums over the splits (loads stay in flight),
-    // combined in a fixed order
+    // four interleaved partial sums over the splits, combined in a fixed order
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    const int64_t sstride = (int64_t)a.nc * a.nslot * a.n_pad;
-    const int64_t base0 = ((int64_t)q * a.nslot) * a.n_pad + i;
-    if (a.part_is_float) {
-        // FP32 partials summed with an error-free transformation (TwoSum) into
-        // a (hi, lo) pair: FP32 arithmetic, no rounding error beyond lo's
-        // loads are issued eight splits ahead of the sums
-        const float *pf = reinterpret_cast<const float *>(a.part);
-        float hi = 0.f, lo = 0.f;
-        auto two_sum = [&](float p) {
-            const float t = hi + p;
-            const float bp = t - hi;
-            lo += (hi - (t - bp)) + (p - bp);
-            hi = t;
-        };
-        int sp = 0;
-        if (a.nslot == 1) {
-            for (; sp + 7 < a.nsplit; sp += 8) {
-                float p[8];
+    if (o >= 0) {
+        const int64_t sstride = (int64_t)a.nc * a.nslot * a.n_pad;
+        const int64_t base0 = ((int64_t)q * a.nslot) * a.n_pad + i;
+        if (a.part_is_float) {
+            // FP32 partials summed with an error-free transformation (TwoSum) into
+            // a (hi, lo) pair: FP32 arithmetic, no rounding error beyond lo's
+            // loads are issued eight ahead of the sums
+            const float *pf = reinterpret_cast<const float *>(a.part);
+            float hi = 0.f, lo = 0.f;
+            auto two_sum = [&](float p) {
+                const float t = hi + p;
+                const float bp = t - hi;
+                lo += (hi - (t - bp)) + (p - bp);
+                hi = t;
+            };
+            int sp = 0;
+            if (a.nslot == 1) {
+                for (; sp + 7 < a.nsplit; sp += 8) {
+                    float p[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) p[u] = pf[base0 + (sp + u) * sstride];
+                    for (int u = 0; u < 8; ++u) p[u] = pf[base0 + (sp + u) * sstride];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) two_sum(p[u]);
+                    for (int u = 0; u < 8; ++u) two_sum(p[u]);
+                }
+            } else {
+                for (; sp + 3 < a.nsplit; sp += 4) {
+                    float p[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) p[u] = pf[base0 + (sp + u / 2) * sstride + (u & 1) * a.n_pad];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) two_sum(p[u]);
+                }
             }
+            for (; sp < a.nsplit; ++sp)
+                for (int l = 0; l < a.nslot; ++l) two_sum(pf[base0 + sp * sstride + l * a.n_pad]);
+            s0 = (double)hi + (double)lo;
+        } else {
+            const double *pd = reinterpret_cast<const double *>(a.part);
+            int sp = 0;
+            for (; sp + 15 < a.nsplit; sp += 16) {
+                double p[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) p[u] = pd[base0 + (sp + u) * sstride];
+#pragma unroll
+                for (int u = 0; u < 16; u += 4) { s0 += p[u]; s1 += p[u + 1]; s2 += p[u + 2]; s3 += p[u + 3]; }
+            }
+            for (; sp + 3 < a.nsplit; sp += 4) {
+                const int64_t b = base0 + sp * sstride;
+                s0 += pd[b];
+                s1 += pd[b + sstride];
+                s2 += pd[b + 2 * sstride];
+                s3 += pd[b + 3 * sstride];
+            }
+            for (; sp < a.nsplit; ++sp) s0 += pd[base0 + sp * sstride];
         }
-        for (; sp < a.nsplit; ++sp)
-            for (int l = 0; l < a.nslot; ++l) two_sum(pf[base0 + sp * sstride + l * a.n_pad]);
-        s0 = (double)hi + (double)lo;
-    } else {
-        const double *pd = reinterpret_cast<const double *>(a.part);
-        int sp = 0;
-        for (; sp + 3 < a.nsplit; sp += 4) {
-            const int64_t b = base0 + sp * sstride;
-            s0 += pd[b];
-            s1 += pd[b + sstride];
-            s2 += pd[b + 2 * sstride];
-            s3 += pd[b + 3 * sstride];
-        }
-        for (; sp < a.nsplit; ++sp) s0 += pd[base0 + sp * sstride];
     }
+    __syncthreads();
+    if (o < 0) return;
     const double s = (s0 + s1) + (s2 + s3);
-    double v = a.scale * s * (a.weight_out ? a.pos64[i].w : 1.0);
-    if (a.self_src) v += a.self_coef * a.pos64[i].w * a.self_src[(int64_t)q * a.n + o];
+    double v = a.scale * s * (a.weight_out ? weight : 1.0);
+    if (a.self_src) v += a.self_coef * weight * selfv;
     double r = a.a_op * v + extra + (q == 0 ? a.add0 : (q == 1 ? a.add1 : a.add2));
-    if (a.rank1_nrm) r += rank1 * a.rank1_nrm[(int64_t)q * a.n + o];
-    if (a.xin) r += a.a_id * a.xin[(int64_t)q * a.n + o];
+    if (a.rank1_nrm) r += rank1 * nrm;
+    if (a.xin) r += a.a_id * x;
     a.out[(int64_t)q * a.n + o] = r;
 }
 
@@ -1949,7 +1979,8 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     ea.out = pc.out;
     if (rows) { ea.row0 = pc.row_begin; ea.row1 = pc.row_end; }
     ctx->launches++;
-    return cuda_check(ctx, launch_pdl(epilogue_kernel, dim3((unsigned)((n_pad * nc + 127) / 128)), dim3(128), 0, s, ea),
+    return cuda_check(ctx, launch_pdl(epilogue_kernel, dim3((unsigned)((n_pad * nc + kEpiTPB - 1) / kEpiTPB)), dim3(kEpiTPB + 32),
+                                      0, s, ea),
                       "epilogue kernel");
 }
 
@@ -2400,7 +2431,7 @@ extern "C" int ssd_stokes_DL_noalloc(ssd_ctx *ctx, const ssd_points *pts, double
     ea.add0 = ea.add1 = ea.add2 = 0.0; ea.add_dev = nullptr;
     ea.wdot_part = nullptr; ea.nwdot = 0; ea.wdot_scale = 0.0; ea.rank1_nrm = nullptr;
     ea.out = out;
-    epilogue_kernel<<<(unsigned)((n_pad * 3 + 127) / 128), 128, 0, s>>>(ea);   // one thread per point and component
+    epilogue_kernel<<<(unsigned)((n_pad * 3 + kEpiTPB - 1) / kEpiTPB), kEpiTPB + 32, 0, s>>>(ea);
     ctx->launches++;
     return launch_check(ctx, "no-alloc epilogue");
 }
