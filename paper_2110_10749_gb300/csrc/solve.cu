@@ -196,7 +196,9 @@ __global__ void givens_kernel(double *H, int ldh, double *cs, double *sn, double
 // row share the vectors of an update; a warp takes whole vectors of a dot.
 // Time of an FP32C GMRES step outside its pair kernel: 49 us against 94 with
 // separate kernels at n = 6500, 57 against 100 at 26000, 73 against 118 at
-// 104000; longer vectors keep the separate kernels (kArnMaxN).
+// 104000; longer vectors keep the separate kernels (kArnMaxN).  The norm after a
+// second pass comes from that pass's own sums: two meetings instead of three, a
+// coupled solve at N = 1062 6.82 ms against 7.12.
 constexpr int kArnTPB = 256;
 constexpr int kArnRows = 64;       // rows per block step: few, for FP64 adds are slow (1.6 per clock and SM)
 constexpr int kArnMaxRows = 1024;  // rows of a block
@@ -299,32 +301,32 @@ __global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
     ok = grid_barrier(a.bar) && ok;
     gather(p0, j + 2, h1);
     update(h1);
-    // DGKS test, the same in every block: more than half of ||w||^2 removed?
-    {
+    // DGKS test, the same in every warp: more than half of ||w||^2 removed?
+    auto squares = [&](const double *h) {
         double s = 0.0;
-        for (int i = tid; i <= j; i += kArnTPB) s = fma(h1[i], h1[i], s);
+        for (int i = lane; i <= j; i += 32) s = fma(h[i], h[i], s);
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) s_red[warp] = s;
-        __syncthreads();
-        s = 0.0;
-#pragma unroll
-        for (int k = 0; k < kArnTPB / 32; ++k) s += s_red[k];
-        __syncthreads();
-        if (ok && s > 0.5 * h1[j + 1]) {
-            dots(p1, j + 1);
-            ok = grid_barrier(a.bar + 1) && ok;
-            gather(p1, j + 1, h2);
-            update(h2);
-        } else {
-            for (int i = tid; i <= j; i += kArnTPB) h2[i] = 0.0;
-        }
+        return s;
+    };
+    double t = -1.0;   // ||w||^2 once known
+    if (ok && squares(h1) > 0.5 * h1[j + 1]) {
+        dots(p1, j + 2);
+        ok = grid_barrier(a.bar + 1) && ok;
+        gather(p1, j + 2, h2);
+        update(h2);
+        // the second pass removes next to nothing: ||w - V h2||^2 = ||w||^2 - |h2|^2
+        // loses no digits then, and saves the third meeting of the blocks
+        const double s2 = squares(h2);
+        if (s2 < 1e-3 * h2[j + 1]) t = h2[j + 1] - s2;
+    } else {
+        for (int i = tid; i <= j; i += kArnTPB) h2[i] = 0.0;
     }
     if (!ok) {   // a barrier's wait ran out: report it as a residual that is not finite
         if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
-    {
-        double t = 0.0;
+    if (t < 0.0) {
+        t = 0.0;
         for (int r = tid; r < nr; r += kArnTPB) t = fma(w[r], w[r], t);
         for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
         if (lane == 0) s_red[warp] = t;
@@ -334,15 +336,15 @@ __global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
             for (int k = 0; k < kArnTPB / 32; ++k) t += s_red[k];
             p2[blockIdx.x] = t;
         }
-    }
-    if (!grid_barrier(a.bar + 2)) {
-        if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
-        return;
-    }
-    {
-        double t = 0.0;
+        if (!grid_barrier(a.bar + 2)) {
+            if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
+            return;
+        }
+        t = 0.0;
         for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(p2 + b);
         for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    }
+    {
         const double hn = sqrt(fmax(t, 0.0));
         const double f = hn != 0.0 ? 1.0 / hn : 1.0;
         for (int r = tid; r < nr; r += kArnTPB) wg[r] = w[r] * f;
