@@ -1163,7 +1163,8 @@ __global__ void __launch_bounds__(kEpiTPB + 32) epilogue_kernel(const EpiArgs a)
         if (a.part_is_float) {
             // FP32 partials summed with an error-free transformation (TwoSum) into
             // a (hi, lo) pair: FP32 arithmetic, no rounding error beyond lo's
-            // loads are issued eight ahead of the sums
+            // loads are issued 32 or eight ahead of the sums (N = 17070, 134 splits: 279.3 us
+            // the Stokes double layer, 282.2 with eight)
             const float *pf = reinterpret_cast<const float *>(a.part);
             float hi = 0.f, lo = 0.f;
             auto two_sum = [&](float p) {
@@ -1174,6 +1175,13 @@ __global__ void __launch_bounds__(kEpiTPB + 32) epilogue_kernel(const EpiArgs a)
             };
             int sp = 0;
             if (a.nslot == 1) {
+                for (; sp + 31 < a.nsplit; sp += 32) {
+                    float p[32];
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) p[u] = pf[base0 + (sp + u) * sstride];
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) two_sum(p[u]);
+                }
                 for (; sp + 7 < a.nsplit; sp += 8) {
                     float p[8];
 #pragma unroll
