@@ -20,8 +20,10 @@
  *   asynchronous on the given stream.  Quadrature, solver and layout calls
  *   synchronise the stream before they return, because they report counts
  *   or iteration results to the host.
- * - prec selects the arithmetic of the pair sums: SSD_FP64 (plain double) or
- *   SSD_FP32C (single precision pair terms, compensated two-float
+ * - prec selects the arithmetic of the pair sums: SSD_FP64 (double precision:
+ *   the pair terms in 62-bit fixed point where the extent of the points is
+ *   between 1/16 and 256 delta, in double elsewhere; errors at or below plain
+ *   double's) or SSD_FP32C (single precision pair terms, compensated two-float
  *   accumulation per target, FP64 epilogue).  Krylov and interface
  *   arithmetic is always FP64.
  * - Non-finite scalar arguments, n <= 0, delta <= 0, mu <= 0, kappa <= 0,
@@ -68,10 +70,11 @@ enum ssd_precision { SSD_FP64 = 0, SSD_FP32C = 1 };
  *                       prepared layout runs the direct kernels, whose split
  *                       sums are added in a fixed order (results reproducible
  *                       bit for bit); with the plans (default) the far block
- *                       pairs of the four layer operators are evaluated once
- *                       for both directions and summed by FP64 atomic adds,
- *                       so results vary in the last bits of an FP64 sum
- *   SSD_PAIR_LPT=0      direct FP32C/FP64 grids in plain (tile, split) order
+ *                       pairs of the four layer operators run on kernels of
+ *                       their own (FP32C: once for both directions) and end
+ *                       in FP64 atomic adds, so results vary in the last bits
+ *                       of an FP64 sum
+ *   SSD_PAIR_LPT=0      direct FP32C grids in plain (tile, split) order
  *                       instead of near-first order
  *   SSD_PAIR_WAVES=k    FP32C direct grid sized for k (1..64) waves of resident CTAs
  *   SSD_PAIR_WAVES64=k  the same for the FP64 direct grid */
@@ -473,7 +476,9 @@ int ssd_hessenberg_eigenvalues(int n, const double *h /* host */, int ldh, doubl
  * Field values away from the surface from the boundary data of a D-N solve
  * (FP64, bare kernels; accurate for field points a few grid spacings from
  * the surface: the paper gives no near-surface correction).  Field points
- * targets[3][nt] and outputs are device arrays; nt may be 0.
+ * targets[3][nt] and outputs are device arrays; nt may be 0.  On prepared
+ * points the velocity and the Darcy pressure run in fixed point as the
+ * operators do; the Stokes pressure, and unprepared points, in double.
  *
  * Darcy pressure inside the body, Green's representation (eq. Greens) with
  * dp/dn = -(mu/kappa) q (Darcy's law, the interface flux q = u . n):

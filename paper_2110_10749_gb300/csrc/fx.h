@@ -1,6 +1,6 @@
 // Fixed-point arithmetic of the FP64 pair sums.
 //
-// This device issues 64 32x32+64-bit integer multiply-adds per clock and SM
+// This device issues 32 32x32+64-bit integer multiply-adds per clock and SM
 // against 1.6 double-precision FMAs (measured), so the FP64 operators run
 // their pair terms in 59 to 62-bit fixed point on the integer pipes: more
 // significant bits than a double carries, at a fraction of the cost.  The

@@ -16,11 +16,13 @@
 // their order does not matter); they enter a double accumulator once per tile.
 // Tables are read by lane-dependent index, sources by broadcast.
 // Measured on the h = 1/32 sphere (N = 17070), against the double-precision
-// kernel: Laplace double layer 2.1 ms (18.9), and on small sets, where every
-// pair is smoothed, Stokes double layer 0.053 ms (0.62) at N = 1062, fused
-// Stokes layers 0.113 ms (1.44) at N = 1742, transposed Stokes double layer
-// 0.34 ms (3.7) at N = 4302; errors against long double at or below the double
-// kernel's.  The wide multiplier is 80% busy (32 a clock and SM).
+// kernel: Laplace double layer 2.20 ms (18.9), and on small sets, where every
+// pair is smoothed, with packing and epilogue: Stokes double layer 0.028 ms
+// (0.62) at N = 1062, fused Stokes layers 0.095 ms (1.44) at N = 1742, transposed
+// Stokes double layer 0.334 ms (3.7) at N = 4302; errors against long double at
+// or below the double kernel's.  The wide multiplier is 80% busy (32 a clock and
+// SM) on large sets; clocks per pair and SM: LSL 1.6, LDL 2.2, SDL 3.3, SSL 4.0,
+// SDLT 4.4, SSLDL 6.
 //
 // Densities are scaled by their largest magnitude, which the packing kernel
 // leaves per block; the kernel reduces those at its start.  When that scale
@@ -137,9 +139,9 @@ __device__ __noinline__ void fx_fallback(const KArgs<double> *ap, const Consts<d
 // layer takes sigma_3 from sigma_1: one table of noct - 6 octaves instead of two
 // of noct.  Stokes single layer at N = 68166: 58.9 ms with the plan against 64.9
 // with every tile on the general kernel; the other layers gain 1-2%.  (The
-// double-precision symmetric kernel that ran the far pairs before took 154 of
-// the 164 ms of this operator at N = 78106; both directions in fixed point take
-// it to 76 ms.)
+// double-precision symmetric kernel that ran the far pairs before left this
+// operator at 164 ms at N = 78106, nearly all of it in that kernel; both directions
+// in fixed point take it to 76 ms.)
 constexpr int kFxFarOct = 6;                     // 1 + 8^2 > 2^6
 template <int OP, bool FAR> constexpr int fx_ntab() { return FAR && OP == OP_SSL ? 1 : FxOp<OP>::ntab; }
 

@@ -11,7 +11,9 @@
 // Each split writes its per-target partial sums; the epilogue kernel adds the
 // splits in a fixed order in FP64, applies the physical constants, the FP64
 // self term of the single layers and the identity/right-hand-side terms, and
-// scatters to the caller's order.
+// scatters to the caller's order.  (FP64 sums run in fixed point instead,
+// fx_kernel.h, without a near/far split; the double-precision kernels here serve
+// the point sets that it does not.)
 //
 // FP32C: pair terms in FP32; each thread adds a tile's terms in FP32 and folds
 // the tile sum into a two-float (hi, lo) accumulator with an error-free
@@ -879,7 +881,8 @@ __global__ void __launch_bounds__(kSymTPB32, sym_min_cta(OP)) sym32_kernel(const
     }
 }
 
-// FP64 counterpart of sym32_kernel on the same block plan: a CTA of 128
+// FP64 counterpart of sym32_kernel on the same block plan, for the point sets
+// that the fixed-point kernels do not serve (fx_geo): a CTA of 128
 // threads holds the 512 targets of one block, 4 per thread (threadIdx.x +
 // 128 t), and walks the source tiles of its item with the same lane-rotated
 // source order and per-warp reverse sums.  Sources are staged as separate

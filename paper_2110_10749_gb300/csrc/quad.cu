@@ -437,11 +437,11 @@ constexpr int kSampleWindow = 512;
 enum QuadOut { kQuadCount, kQuadPoints, kQuadJacobian };
 
 struct QuadOutArgs {
-    int32_t *count;
-    const int64_t *offs;
-    int64_t n;
-    double *xyz, *nrm, *w;   // points, or their derivatives
-    int32_t *meta;
+    int32_t *count = nullptr;
+    const int64_t *offs = nullptr;
+    int64_t n = 0;
+    double *xyz = nullptr, *nrm = nullptr, *w = nullptr;   // points, or their derivatives
+    int32_t *meta = nullptr;
 };
 
 // The point at t on the line of axis ax whose in-plane coordinates are pa, pb
