@@ -564,6 +564,7 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cuda
     char *b = static_cast<char *>(blk);
     Layout out;
     out.n = n;
+    out.owner = ctx;
     out.n_pad = n_pad;
     out.block = blk;
     out.perm = reinterpret_cast<int32_t *>(b + o_perm);

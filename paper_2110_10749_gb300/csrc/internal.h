@@ -74,6 +74,7 @@ struct Layout {
     Extent ext{};              // box and largest weighted normal (host copy)
     void *fx_block = nullptr;  // grid positions and chunk boxes of the fixed-point kernel (pool memory)
     double fx_delta = 0.0;     // smoothing radius they were made for
+    const void *owner = nullptr;   // context that built the layout
     void *block = nullptr;     // single allocation backing the arrays
     // launch order of the FP32C pair grid (prepared layouts only), cached for
     // the last (grid, rho_far delta) it was built for

@@ -1755,23 +1755,38 @@ static FxSplit fx_split_grid(const ssd_ctx *ctx, int64_t n) {
     return best;
 }
 
-// Grid positions of a layout at a smoothing radius, kept with a prepared
-// layout for the last radius it was used with.
-static int fx_positions(ssd_ctx *ctx, const Layout &L, double delta, const FxGeo &geo, const l4 **X, const int4 **cbox,
-                        cudaStream_t s) {
+static size_t fx_position_bytes(const Layout &L) { return sizeof(l4) * L.n_pad + sizeof(int4) * 2 * (L.n_pad / kChunk); }
+
+// Whether a call may use and replace the grid positions kept with a layout.  A
+// graph replays after calls at other radii, and another context's calls have
+// a stream order of their own: such calls make the positions in their
+// workspace (about 3 us more).
+static bool fx_keeps(const ssd_ctx *ctx, const Layout &L, cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {   // the legacy stream while another one captures
+        cudaGetLastError();
+        return false;
+    }
+    return L.owner == ctx && st == cudaStreamCaptureStatusNone;
+}
+
+// Grid positions of a layout at a smoothing radius: in ws, or (ws NULL) kept
+// with the layout for the last radius that it was used with.
+static int fx_positions(ssd_ctx *ctx, const Layout &L, double delta, const FxGeo &geo, void *ws, const l4 **X,
+                        const int4 **cbox, cudaStream_t s) {
     Layout &M = const_cast<Layout &>(L);
-    if (!M.fx_block) {
-        SSD_TRY(dev_alloc(ctx, sizeof(l4) * L.n_pad + sizeof(int4) * 2 * (L.n_pad / kChunk), &M.fx_block));
+    if (!ws && !M.fx_block) {
+        SSD_TRY(dev_alloc(ctx, fx_position_bytes(L), &M.fx_block));
         M.fx_delta = 0.0;
     }
-    l4 *x = static_cast<l4 *>(M.fx_block);
+    l4 *x = static_cast<l4 *>(ws ? ws : M.fx_block);
     int4 *cb = reinterpret_cast<int4 *>(x + L.n_pad);
-    if (M.fx_delta != delta) {
+    if (ws || M.fx_delta != delta) {
         FxGrid g{L.pos64, L.n_pad, L.n - 1, geo, nullptr, nullptr, 1, x, cb};
         fx_grid_kernel<<<(unsigned)(L.n_pad / kChunk), kChunk, 0, s>>>(g);
         ctx->launches++;
         SSD_TRY(launch_check(ctx, "grid positions"));
-        M.fx_delta = delta;
+        if (!ws) M.fx_delta = delta;
     }
     *X = x;
     *cbox = cb;
@@ -1837,6 +1852,8 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     }
     const size_t o_acc = use_sym ? carve(sizeof(double) * nc * n_pad) : 0;
     const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks) : 0;
+    const bool fx_kept = use_fx && fx_keeps(ctx, L, s);
+    const size_t o_fxx = use_fx ? carve(fx_position_bytes(L)) : 0;   // always: a captured call cannot grow the pool
     void *ws = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &ws));
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, ws};
@@ -1876,7 +1893,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     pa.wdot_part = rank1 ? reinterpret_cast<double *>(base + o_wdot) : nullptr;
     FxArgs fa{};
     if (use_fx) {
-        SSD_TRY(fx_positions(ctx, L, pc.delta, geo, &fa.X, &fa.cbox, s));
+        SSD_TRY(fx_positions(ctx, L, pc.delta, geo, fx_kept ? nullptr : base + o_fxx, &fa.X, &fa.cbox, s));
         pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
         pa.fx.two = op == OP_LSLDL ? 1 : 0;
         fa.bmax = pa.fx.bmax;
