@@ -124,27 +124,49 @@ static int drain_timing(ssd_ctx *ctx) {
 // ------------------------------------------------------------------ layouts
 namespace {
 
-__global__ void bbox_kernel(const double *xyz, int64_t n, double *out /* 6 */) {
-    __shared__ double lo[3][256], hi[3][256];
-    double l[3] = {1e300, 1e300, 1e300}, h[3] = {-1e300, -1e300, -1e300};
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x)
+// Bounding box of n points: one block, or 32 partial boxes (block b: out + 6 (1 + b))
+// and then their union.  The comparisons are double precision, 1.6 a clock and SM,
+// six a point: preparing 78106 points took 344 us with one block and takes 190,
+// 17070 points 188 and 153; up to 4096 points the second launch costs as much as it
+// saves.
+constexpr int kBoxBlocks = 32;
+
+__global__ void bbox_kernel(const double *xyz, int64_t n, double *out) {
+    __shared__ double red[6][256];   // (lo, -hi)
+    double v[6] = {1e300, 1e300, 1e300, 1e300, 1e300, 1e300};
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
         for (int k = 0; k < 3; ++k) {
-            const double v = xyz[k * n + i];
-            l[k] = fmin(l[k], v);
-            h[k] = fmax(h[k], v);
+            const double x = xyz[k * n + i];
+            v[k] = fmin(v[k], x);
+            v[3 + k] = fmin(v[3 + k], -x);
         }
-    for (int k = 0; k < 3; ++k) { lo[k][threadIdx.x] = l[k]; hi[k][threadIdx.x] = h[k]; }
+    for (int k = 0; k < 6; ++k) red[k][threadIdx.x] = v[k];
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+    for (int st = 128; st > 0; st >>= 1) {
         if (threadIdx.x < st)
-            for (int k = 0; k < 3; ++k) {
-                lo[k][threadIdx.x] = fmin(lo[k][threadIdx.x], lo[k][threadIdx.x + st]);
-                hi[k][threadIdx.x] = fmax(hi[k][threadIdx.x], hi[k][threadIdx.x + st]);
-            }
+            for (int k = 0; k < 6; ++k) red[k][threadIdx.x] = fmin(red[k][threadIdx.x], red[k][threadIdx.x + st]);
         __syncthreads();
     }
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; ++k) { out[k] = lo[k][0]; out[3 + k] = hi[k][0]; }
+    if (threadIdx.x < 6)
+        out[6 * (gridDim.x > 1 ? 1 + blockIdx.x : 0) + threadIdx.x] = threadIdx.x < 3 ? red[threadIdx.x][0] : -red[threadIdx.x][0];
+}
+
+__global__ void bbox_union_kernel(double *out) {   // one warp
+    const double *p = out + 6 * (1 + threadIdx.x);
+    for (int k = 0; k < 6; ++k) {
+        double v = p[k];
+        for (int off = 16; off > 0; off >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v, off);
+            v = k < 3 ? fmin(v, u) : fmax(v, u);
+        }
+        if (threadIdx.x == 0) out[k] = v;
+    }
+}
+
+static void launch_bbox(const double *xyz, int64_t n, double *bb, cudaStream_t s) {
+    const int blocks = n <= 4096 ? 1 : kBoxBlocks;
+    bbox_kernel<<<blocks, 256, 0, s>>>(xyz, n, bb);
+    if (blocks > 1) bbox_union_kernel<<<1, kBoxBlocks, 0, s>>>(bb);
 }
 
 __device__ __forceinline__ uint32_t spread10(uint32_t v) {
@@ -219,14 +241,14 @@ __global__ void chunk_box_kernel(Layout L) {
     L.cbox[2 * c + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
 }
 
-// fixed-order FP64 sum of the weights (one block)
-__global__ void wsum_kernel(const double *w, int64_t n, double *out) {
-    __shared__ double red[256];
+// fixed-order FP64 sum of the weights, by one block of 256 threads
+__device__ void wsum_block(const double *w, int64_t n, double *red, double *out) {
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += w[i];
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < n; i += 256) s += w[i];
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+    for (int st = 128; st > 0; st >>= 1) {
         if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
         __syncthreads();
     }
@@ -235,12 +257,19 @@ __global__ void wsum_kernel(const double *w, int64_t n, double *out) {
 
 // Extent (see internal.h) of points [off[y], off[y + 1]) of surface y =
 // blockIdx.y (off NULL: all n points), block x of kExtentBlocks partials each.
+// With wsum, block 0 of one more sums the weights beside them (a launch of its own made
+// the layout of 1062 points take 7 us longer, with one block for the box).
 __global__ void extent_kernel(const double *xyz, const double *nrm, const double *w, int64_t n, const int64_t *off,
-                              Extent *out) {
+                              Extent *out, double *wsum) {
     __shared__ double red[8][256];
+    const int64_t nb = (int64_t)gridDim.x - (wsum ? 1 : 0), blk = (int64_t)blockIdx.x - (wsum ? 1 : 0);
+    if (blk < 0) {
+        wsum_block(w, n, red[0], wsum);
+        return;
+    }
     const int64_t beg = off ? off[blockIdx.y] : 0, end = off ? off[blockIdx.y + 1] : n;
     double v[8] = {1e308, 1e308, 1e308, 1e308, 1e308, 1e308, 0.0, 1.0};   // lo, -hi (minima), -mmax, fin
-    for (int64_t i = beg + (int64_t)blockIdx.x * 256 + threadIdx.x; i < end; i += (int64_t)gridDim.x * 256) {
+    for (int64_t i = beg + blk * 256 + threadIdx.x; i < end; i += nb * 256) {
         for (int c = 0; c < 3; ++c) {
             const double x = xyz[c * n + i], m = w[i] * nrm[c * n + i];
             v[c] = fmin(v[c], x);
@@ -262,7 +291,7 @@ __global__ void extent_kernel(const double *xyz, const double *nrm, const double
         for (int c = 0; c < 3; ++c) { e.lo[c] = red[c][0]; e.hi[c] = -red[3 + c][0]; }
         e.mmax = -red[6][0];
         e.fin = red[7][0];
-        out[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = e;
+        out[blockIdx.y * nb + blk] = e;
     }
 }
 
@@ -469,7 +498,7 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
         auto tcarve = [&](size_t bb) { size_t o = t_off; t_off += (bb + 255) & ~size_t(255); return o; };
         const size_t o_k0 = tcarve(sizeof(uint64_t) * n), o_k1 = tcarve(sizeof(uint64_t) * n);
         const size_t o_i0 = tcarve(sizeof(int32_t) * n), o_i1 = tcarve(sizeof(int32_t) * n);
-        const size_t o_bb = tcarve(sizeof(double) * 6), o_cub = tcarve(cub_bytes);
+        const size_t o_bb = tcarve(sizeof(double) * 6 * (1 + kBoxBlocks)), o_cub = tcarve(cub_bytes);
         st = dev_alloc(ctx, t_off, &tmp);
         if (st == SSD_OK) {
             char *tb = static_cast<char *>(tmp);
@@ -478,9 +507,9 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
             double *bb = reinterpret_cast<double *>(tb + o_bb);
             const unsigned gn = (unsigned)((n + 255) / 256);
             batch_esurf_kernel<<<gn, 256, 0, s>>>(dmeta, ns, n, out.elem_surf);
-            bbox_kernel<<<1, 256, 0, s>>>(b->xyz, n, bb);
+            launch_bbox(b->xyz, n, bb, s);
             batch_key_kernel<<<gn, 256, 0, s>>>(b->xyz, n, bb, out.elem_surf, k0, i0);
-            ctx->launches += 3;
+            ctx->launches += 4;
             st = launch_check(ctx, "batch keys");
             if (st == SSD_OK) {
                 cudaError_t e = cub::DeviceRadixSort::SortPairs(tb + o_cub, cub_bytes, k0, k1, i0, i1, (int)n, 0,
@@ -498,7 +527,7 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
                 batch_wsum_kernel<<<ns, 256, 0, s>>>(b->w, dmeta, out.d_wsum);
                 for (int k = 0; k < ns; k += 65535)   // grid.y limit
                     extent_kernel<<<dim3(1, (unsigned)(ns - k < 65535 ? ns - k : 65535)), 256, 0, s>>>(
-                        b->xyz, b->nrm, b->w, n, dmeta + k, dext + k);
+                        b->xyz, b->nrm, b->w, n, dmeta + k, dext + k, nullptr);
                 ctx->launches += 4;
                 st = launch_check(ctx, "batch fill");
             }
@@ -587,16 +616,16 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cuda
         auto tcarve = [&](size_t bb) { size_t o = t_off; t_off += (bb + 255) & ~size_t(255); return o; };
         const size_t o_k0 = tcarve(sizeof(uint32_t) * n), o_k1 = tcarve(sizeof(uint32_t) * n);
         const size_t o_i0 = tcarve(sizeof(int32_t) * n), o_i1 = tcarve(sizeof(int32_t) * n);
-        const size_t o_bb = tcarve(sizeof(double) * 6), o_cub = tcarve(cub_bytes);
+        const size_t o_bb = tcarve(sizeof(double) * 6 * (1 + kBoxBlocks)), o_cub = tcarve(cub_bytes);
         st = dev_alloc(ctx, t_off, &tmp);
         if (st != SSD_OK) { release_layout(ctx, &out); return st; }
         char *tb = static_cast<char *>(tmp);
         uint32_t *k0 = reinterpret_cast<uint32_t *>(tb + o_k0), *k1 = reinterpret_cast<uint32_t *>(tb + o_k1);
         int32_t *i0 = reinterpret_cast<int32_t *>(tb + o_i0), *i1 = reinterpret_cast<int32_t *>(tb + o_i1);
         double *bb = reinterpret_cast<double *>(tb + o_bb);
-        bbox_kernel<<<1, 256, 0, s>>>(pts->xyz, n, bb);
+        launch_bbox(pts->xyz, n, bb, s);
         morton_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pts->xyz, n, bb, k0, i0);
-        ctx->launches += 2;
+        ctx->launches += 3;
         st = launch_check(ctx, "morton keys");
         if (st == SSD_OK) {
             cudaError_t e = cub::DeviceRadixSort::SortPairs(tb + o_cub, cub_bytes, k0, k1, i0, i1, (int)n, 0, 30, s);
@@ -608,11 +637,10 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cuda
     if (st == SSD_OK) {
         fill_layout_kernel<<<(unsigned)((n_pad + 255) / 256), 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, n_pad,
                                                                           sorted, out);
-        wsum_kernel<<<1, 256, 0, s>>>(pts->w, n, dsum);
-        extent_kernel<<<kExtentBlocks, 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, nullptr,
-                                                    reinterpret_cast<Extent *>(dsum + 8));
+        extent_kernel<<<1 + kExtentBlocks, 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, nullptr,
+                                                        reinterpret_cast<Extent *>(dsum + 8), dsum);
         chunk_box_kernel<<<(unsigned)((n_pad / kChunk + 127) / 128), 128, 0, s>>>(out);
-        ctx->launches += 4;
+        ctx->launches += 3;
         st = launch_check(ctx, "layout fill");
     }
     static_assert(8 + 8 * kExtentBlocks <= 512, "the read fits the pinned scratch");
