@@ -20,8 +20,8 @@
 // pair is smoothed, with packing and epilogue: Stokes double layer 0.028 ms
 // (0.62) at N = 1062, fused Stokes layers 0.095 ms (1.44) at N = 1742, transposed
 // Stokes double layer 0.334 ms (3.7) at N = 4302; errors against long double at
-// or below the double kernel's.  The wide multiplier is 80% busy (32 a clock and
-// SM) on large sets; clocks per pair and SM: LSL 1.6, LDL 2.2, SDL 3.3, SSL 4.0,
+// or below the double kernel's.  The wide multiplier is 71% busy (32 a clock and
+// SM) on large sets, the ALU that shifts and adds 64%; clocks per pair and SM: LSL 1.6, LDL 2.2, SDL 3.3, SSL 4.0,
 // SDLT 4.4, SSLDL 6.
 //
 // Densities are scaled by their largest magnitude, which the packing kernel
@@ -292,8 +292,15 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
                     const int top = (int)((tile + cnt - 1) / kChunk - b);
 #pragma unroll
                     for (int k = 0; k < kBoxes; ++k) grow(slo, shi, b + (k < top ? k : top));
+                    if (GROUPS == 1 && top >= kBoxes) grow(slo, shi, b + top);
                 } else {
-                    for (int k = 0; k < cnt / kChunk; ++k) grow(slo, shi, tile / kChunk + k);
+                    const int64_t b = tile / kChunk;
+                    for (int k = 0; k < cnt / kChunk; ++k) grow(slo, shi, b + k);
+                    if ((tile | cnt) % kChunk) {   // (a loop over all boxes costs large sets 0.3%)
+                        const int64_t e = (tile + cnt - 1) / kChunk;
+                        grow(slo, shi, min(b + cnt / kChunk, e));
+                        grow(slo, shi, e);
+                    }
                 }
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {

@@ -1727,8 +1727,12 @@ size_t fx_geo_bytes(int nsurf) { return sizeof(FxGeo) * nsurf; }
 // of 55 with its packing and epilogue; N = 1742: 280 against 196).  Their chunks
 // go by 8 sources, not 32: at N = 1099 the fullest thread has 18 pairs instead of
 // 24 (value and gradients on a star surface 128.9 ms against 140.5), at N = 1742
-// 44 instead of 48 (fused Stokes layers 96.4 us against 103.4).  From 6000 points
-// on about 5 rounds, which the scheduler levels.
+// 44 instead of 48 (fused Stokes layers 96.4 us against 103.4), and without groups
+// at N = 3558 168 sources a CTA instead of 192 (Stokes double layer 177 us against
+// 189).  Chunks of more than 256 sources need not be whole staged tiles: at N = 4974
+// 336 instead of 384 (318 us against 357).
+// From 6000 points on about 5 rounds, which the scheduler levels, of whole staged
+// tiles.
 struct FxSplit {
     int groups = 1;
     int64_t chunk = 0, nsplit = 1;
@@ -1744,10 +1748,12 @@ static FxSplit fx_split_grid(const ssd_ctx *ctx, int64_t n) {
         int64_t ns = want / nt;
         ns = ns < 1 ? 1 : (ns > units ? units : ns);
         const int64_t per = (units * kChunk + ns - 1) / ns;
-        int64_t chunk = g > 1 ? (per + kFxUnit - 1) / kFxUnit * kFxUnit : (per + kChunk - 1) / kChunk * kChunk;
-        if (chunk > 256) chunk = (chunk + kTile - 1) / kTile * kTile;   // whole staged tiles
-        if (g > 1 && (n >= 6000 || span * chunk >= cost)) continue;   // pairs of the fullest CTA
-        cost = span * chunk;
+        const int64_t unit = n < 6000 ? kFxUnit : (per > 256 ? kTile : kChunk);
+        const int64_t chunk = (per + unit - 1) / unit * unit;
+        // pairs of the fullest CTA; staging a source counts as 2 of them, a target's sum of a tile as 4
+        const int64_t c = (span + 2) * chunk + 4 * span * ((chunk + kTile - 1) / kTile);
+        if (g > 1 && (n >= 6000 || c >= cost)) continue;
+        cost = c;
         best.groups = g;
         best.chunk = chunk;
         best.nsplit = (units * kChunk + chunk - 1) / chunk;
