@@ -77,7 +77,9 @@ enum ssd_precision { SSD_FP64 = 0, SSD_FP32C = 1 };
  *   SSD_PAIR_LPT=0      direct FP32C grids in plain (tile, split) order
  *                       instead of near-first order
  *   SSD_PAIR_WAVES=k    FP32C direct grid sized for k (1..64) waves of resident CTAs
- *   SSD_PAIR_WAVES64=k  the same for the FP64 direct grid */
+ *   SSD_PAIR_WAVES64=k  the same for the FP64 direct grid
+ *   SSD_GRID_POLLS=k    polls of a grid barrier (0..2^22, the default) after which a
+ *                       solver call gives up with SSD_ECUDA */
 int ssd_ctx_create(ssd_ctx **ctx, int device);
 /* Free the context, its workspace and layouts.  NULL is accepted. */
 int ssd_ctx_destroy(ssd_ctx *ctx);

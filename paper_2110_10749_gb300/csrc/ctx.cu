@@ -95,7 +95,7 @@ int frame_acquire(ssd_ctx *ctx, double **slots, cudaEvent_t ev[2]) {
         SSD_TRY(cuda_check(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event create"));
         ctx->sync_ev.push_back(e);
     }
-    *slots = ctx->hbuf + 512 + 4 * f;
+    *slots = ctx->hbuf + 512 + kFrameLen * f;
     ev[0] = ctx->sync_ev[2 * f];
     ev[1] = ctx->sync_ev[2 * f + 1];
     ctx->hsp++;
@@ -704,7 +704,7 @@ int ssd_ctx_create(ssd_ctx **out, int device) {
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return SSD_ECUDA; }
     ctx->num_sms = prop.multiProcessorCount;
-    if (cudaMallocHost((void **)&ctx->hbuf, 8192) != cudaSuccess) { delete ctx; return SSD_ENOMEM; }
+    if (cudaMallocHost((void **)&ctx->hbuf, sizeof(double) * (512 + kFrameLen * kHostFrames)) != cudaSuccess) { delete ctx; return SSD_ENOMEM; }
     if (pair_occupancy(ctx) != SSD_OK) { cudaFreeHost(ctx->hbuf); delete ctx; return SSD_ECUDA; }
     // tuning knob: waves of resident CTAs in an FP32C pair-kernel grid
     if (const char *w = getenv("SSD_PAIR_WAVES")) {
@@ -717,6 +717,10 @@ int ssd_ctx_create(ssd_ctx **out, int device) {
     if (const char *w = getenv("SSD_PAIR_WAVES64")) {
         const int v = atoi(w);
         if (v >= 1 && v <= 64) ctx->waves64 = ctx->waves_fx = v;
+    }
+    if (const char *w = getenv("SSD_GRID_POLLS")) {
+        const int v = atoi(w);
+        if (v >= 0 && v <= ctx->grid_polls) ctx->grid_polls = v;
     }
     *out = ctx;
     return SSD_OK;

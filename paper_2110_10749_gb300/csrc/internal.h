@@ -108,6 +108,7 @@ struct ssd_ctx {
     int lpt = 1;               // pair grids in near-first order on prepared layouts
     int sym = 1;               // layer operators (both precisions): far block pairs once for both directions
     int waves_fx = 10;         // FP64 fixed-point grid of large sets: rounds of two CTAs per SM
+    int grid_polls = 1 << 22;  // bound of a wait at a grid barrier
     int waves64 = 8;           // FP64 grid: about this many waves of resident CTAs (tuned)
     void *fx_tab = nullptr;    // kernel tables of the fixed-point FP64 kernels (built with the context)
     void *noalloc_scratch = nullptr;   // device address of the no-alloc scratch array (first no-alloc call)
@@ -116,7 +117,7 @@ struct ssd_ctx {
     struct Block { void *p; size_t bytes; bool used; };
     std::vector<Block> pool;
     // pinned host scratch for small device->host reads
-    double *hbuf = nullptr;     // pinned: [0, 512) scalar reads, [512, 1024) GMRES frames
+    double *hbuf = nullptr;     // pinned: [0, 512) scalar reads, then the GMRES frames
     int hsp = 0;                // GMRES frames in use (nested solves take one each)
     std::vector<cudaEvent_t> sync_ev;   // two per frame, created on first use
     // timing
@@ -154,10 +155,11 @@ struct LayoutRef {
 int get_layout(ssd_ctx *ctx, const ssd_points *pts, LayoutRef *ref, cudaStream_t s);
 int check_points(ssd_ctx *ctx, const ssd_points *pts);
 
-// Pinned frame of 4 doubles and two events for one GMRES solve, so that
+// Pinned frame of kFrameLen doubles and two events for one GMRES solve, so that
 // its residual can be read back asynchronously while nested solves use their
 // own frames (LIFO).  (ctx.cu)
 constexpr int kHostFrames = 128;
+constexpr int kFrameLen = 8;   // two steps' residual and norm, then a flag for a grid barrier that gave up
 int frame_acquire(ssd_ctx *ctx, double **slots, cudaEvent_t ev[2]);
 void frame_release(ssd_ctx *ctx);
 

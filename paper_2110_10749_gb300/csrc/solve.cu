@@ -245,24 +245,29 @@ struct ArnoldiArgs {
     double *H, *cs, *sn, *g;
     double *partial;      // [3][(j + 2) * gridDim.x]
     unsigned *bar;        // three counters of this step, zero at launch
+    int polls;            // bound of a wait
     double *out;          // pinned host: residual estimate, norm
+    double *failed;       // pinned host: not 0 once a wait of the solve has run out
 };
 
 // Grid barrier with a bounded wait (every block is resident: cooperative
-// launch).  Returns false when the wait ran out.
-__device__ bool grid_barrier(unsigned *bar) {
+// launch).  Returns false when the wait ran out.  A block that gives up has
+// been counted, so others may still pass: it sets `failed` itself, which the
+// host reads with the step's residual, after the whole grid has ended.
+__device__ bool grid_barrier(unsigned *bar, int polls, double *failed) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(bar, 1u);
         int good = 0;
-        for (int it = 0; it < (1 << 22); ++it) {
+        for (int it = 0; it < polls; ++it) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar));
             if (v >= gridDim.x) { good = 1; break; }
         }
         __threadfence();
+        if (!good) *static_cast<volatile double *>(failed) = 1.0;
         ok = good;
     }
     __syncthreads();
@@ -330,9 +335,8 @@ __global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
         __syncthreads();
     };
     double *p0 = a.partial, *p1 = p0 + (int64_t)(j + 2) * gridDim.x, *p2 = p1 + (int64_t)(j + 2) * gridDim.x;
-    bool ok = true;
     dots(p0, j + 2);
-    ok = grid_barrier(a.bar) && ok;
+    if (!grid_barrier(a.bar, a.polls, a.failed)) return;
     gather(p0, j + 2, h1);
     update(h1);
     // DGKS test, the same in every warp: more than half of ||w||^2 removed?
@@ -343,9 +347,9 @@ __global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
         return s;
     };
     double t = -1.0;   // ||w||^2 once known
-    if (ok && squares(h1) > 0.5 * h1[j + 1]) {
+    if (squares(h1) > 0.5 * h1[j + 1]) {
         dots(p1, j + 2);
-        ok = grid_barrier(a.bar + 1) && ok;
+        if (!grid_barrier(a.bar + 1, a.polls, a.failed)) return;
         gather(p1, j + 2, h2);
         update(h2);
         // the second pass removes next to nothing: ||w - V h2||^2 = ||w||^2 - |h2|^2
@@ -354,10 +358,6 @@ __global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
         if (s2 < 1e-3 * h2[j + 1]) t = h2[j + 1] - s2;
     } else {
         for (int i = tid; i <= j; i += kArnTPB) h2[i] = 0.0;
-    }
-    if (!ok) {   // a barrier's wait ran out: report it as a residual that is not finite
-        if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
-        return;
     }
     if (t < 0.0) {
         t = 0.0;
@@ -370,10 +370,7 @@ __global__ void __launch_bounds__(kArnTPB) arnoldi_kernel(const ArnoldiArgs a) {
             for (int k = 0; k < kArnTPB / 32; ++k) t += s_red[k];
             p2[blockIdx.x] = t;
         }
-        if (!grid_barrier(a.bar + 2)) {
-            if (tid == 0 && blockIdx.x == 0) a.out[0] = a.out[1] = __longlong_as_double(0x7ff8000000000000ll);
-            return;
-        }
+        if (!grid_barrier(a.bar + 2, a.polls, a.failed)) return;
         t = 0.0;
         for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(p2 + b);
         for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
@@ -599,6 +596,8 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
     cudaEvent_t ev[2];
     SSD_TRY(frame_acquire(ctx, &slot, ev));
     struct FrameGuard { ssd_ctx *c; ~FrameGuard() { frame_release(c); } } frame_guard{ctx};
+    volatile double *failed = slot + 4;
+    *failed = 0.0;
     Buf V, small;
     SSD_TRY(V.alloc(ctx, sizeof(double) * (size_t)(m + 1) * n));
     const int ldh = m + 1;
@@ -667,6 +666,11 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
         int pending = -1;      // queued step whose residual has not been read yet
         auto fetch = [&](int step) -> int {
             SSD_TRY(cuda_check(ctx, cudaEventSynchronize(ev[step & 1]), "event sync"));
+            if (*failed != 0.0) {
+                // a step queued ahead still writes to the frame and the buffers
+                SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "gmres sync"));
+                return set_error(ctx, SSD_ECUDA, "a grid barrier of an Arnoldi step ran out of polls");
+            }
             hb[0] = slot[2 * (step & 1)];
             hb[1] = slot[2 * (step & 1) + 1];
             return SSD_OK;
@@ -678,7 +682,7 @@ int gmres(ssd_ctx *ctx, cudaStream_t s, int64_t n, const MatVec &A, const double
             ++total;
             if (fused) {
                 ArnoldiArgs aa{V.d(), n, j, rows, ldh, H, cs, sn, g, dots.partial.d(), bar + 3 * j,
-                               slot + 2 * (j & 1)};
+                               ctx->grid_polls, slot + 2 * (j & 1), slot + 4};
                 void *params[] = {&aa};
                 SSD_TRY(cuda_check(ctx, cudaLaunchCooperativeKernel((const void *)arnoldi_kernel, dim3(arn_grid),
                                                                     dim3(kArnTPB), params, 0, s), "arnoldi step"));
