@@ -74,8 +74,9 @@ enum ssd_precision { SSD_FP64 = 0, SSD_FP32C = 1 };
  *                       their own (FP32C: once for both directions) and end
  *                       in FP64 atomic adds, so results vary in the last bits
  *                       of an FP64 sum
- *   SSD_PAIR_LPT=0      direct FP32C grids in plain (tile, split) order
- *                       instead of near-first order
+ *   SSD_PAIR_LPT=0      direct grids of FP32C, and of FP64 outside the extents
+ *                       above, in plain (tile, split) order instead of near-first
+ *                       order
  *   SSD_PAIR_WAVES=k    FP32C direct grid sized for k (1..64) waves of resident CTAs
  *   SSD_PAIR_WAVES64=k  the same for the FP64 direct grid
  *   SSD_GRID_POLLS=k    polls of a grid barrier (0..2^22, the default) after which a

@@ -568,7 +568,8 @@ int check_points(ssd_ctx *ctx, const ssd_points *pts) {
 
 void release_layout(ssd_ctx *ctx, Layout *L) {
     if (L->block) dev_free(ctx, L->block);
-    if (L->order32) dev_free(ctx, L->order32);
+    for (int k = 0; k < 2; ++k)
+        if (L->order32[k]) dev_free(ctx, L->order32[k]);
     if (L->fx_block) dev_free(ctx, L->fx_block);
     for (auto &pl : L->sym)
         if (pl.block) dev_free(ctx, pl.block);

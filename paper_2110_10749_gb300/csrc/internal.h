@@ -31,9 +31,8 @@ constexpr int kTPT32 = SSD_TPT32;   // targets per thread, FP32C (pairs of packe
 constexpr int kSymTPT = SSD_SYMTPT; // targets per thread of the FP32C symmetric kernel (4 or 8)
 constexpr int kChunk = 32;          // sources per bounding-box chunk (near/far test per warp)
 constexpr int kTPB64 = 128;         // threads per CTA, generic pair kernel
-constexpr int kTPT64 = 1;           // targets per thread, generic pair kernel in FP32 (transposes)
-constexpr int kTPTd = 2;            // targets per thread, generic pair kernel in double
-constexpr int kFxTPB = 256;         // threads and targets per CTA, FP64 fixed-point kernel (= kTPB64 * kTPTd)
+constexpr int kTPT64 = 1;           // targets per thread, generic pair kernel
+constexpr int kFxTPB = 256;         // threads and targets per CTA, FP64 fixed-point kernel
 constexpr int kRowAlign = 512;      // n_pad is a multiple of this (>= every CTA target span)
 
 // Operators of the pair kernels.
@@ -76,12 +75,13 @@ struct Layout {
     double fx_delta = 0.0;     // smoothing radius they were made for
     const void *owner = nullptr;   // context that built the layout
     void *block = nullptr;     // single allocation backing the arrays
-    // launch order of the FP32C pair grid (prepared layouts only), cached for
+    // launch order of the pair grids (prepared layouts only), cached for
     // the last (grid, rho_far delta) it was built for
+    // (slot 0: FP32C packed kernel, slot 1: generic kernel in double)
     bool order_ok = false;
-    int2 *order32 = nullptr;
-    int64_t order_nit = 0, order_chunk = 0;
-    float order_rfar2 = -1.f;
+    int2 *order32[2] = {nullptr, nullptr};
+    int64_t order_nit[2] = {0, 0}, order_chunk[2] = {0, 0};
+    float order_rfar2[2] = {-1.f, -1.f};
     // plans of the layer operators that evaluate far block pairs once for
     // both directions (prepared layouts only), one per precision:
     // [0] FP32C, [1] FP64

@@ -1243,7 +1243,7 @@ __global__ void __launch_bounds__(kEpiTPB + 32) epilogue_kernel(const EpiArgs a)
 
 template <int OP>
 cudaError_t launch64(dim3 grid, const KArgs<double> &ka, cudaStream_t s) {
-    pair_kernel<double, OP, kTPB64, kTPTd><<<grid, kTPB64, 0, s>>>(ka);
+    pair_kernel<double, OP, kTPB64, kTPT64><<<grid, kTPB64, 0, s>>>(ka);
     return cudaGetLastError();
 }
 
@@ -1261,9 +1261,8 @@ cudaError_t launch_pair_op64(int op, dim3 grid, const KArgs<double> &ka, cudaStr
 // transposed double layers run on the generic kernel in both precisions
 template <typename R>
 cudaError_t launch_transpose(int op, dim3 grid, const KArgs<R> &ka, cudaStream_t s) {
-    constexpr int TPT = sizeof(R) == 8 ? kTPTd : kTPT64;
-    if (op == OP_LDLT) pair_kernel<R, OP_LDLT, kTPB64, TPT><<<grid, kTPB64, 0, s>>>(ka);
-    else pair_kernel<R, OP_SDLT, kTPB64, TPT><<<grid, kTPB64, 0, s>>>(ka);
+    if (op == OP_LDLT) pair_kernel<R, OP_LDLT, kTPB64, kTPT64><<<grid, kTPB64, 0, s>>>(ka);
+    else pair_kernel<R, OP_SDLT, kTPB64, kTPT64><<<grid, kTPB64, 0, s>>>(ka);
     return cudaGetLastError();
 }
 
@@ -1448,7 +1447,7 @@ __global__ void bepilogue_kernel(const BEpiArgs a) {
 
 }  // namespace
 
-// Launch order of the single-surface FP32C grid: items (target tile, split)
+// Launch order of a single-surface grid: items (target tile, split)
 // with more near (warp, 32-source chunk) pairs first, so that the cheap far
 // items fill the last wave (longest-processing-time-first).  key = number of
 // near (warp, chunk) pairs of the item.
@@ -1482,17 +1481,16 @@ __global__ void item_cost_kernel(const float4 *cbox, int64_t ntiles_t, int64_t n
     key[it] = cnt;
 }
 
-// Builds (once per layout, delta and grid) the launch order of the FP32C grid.
-int item_order(ssd_ctx *ctx, const Layout &L, int tpb, int tpt, int64_t ntiles_t, int64_t nsplit,
+// Builds (once per layout, delta and grid) the launch order of a grid.
+int item_order(ssd_ctx *ctx, const Layout &L, int slot, int tpb, int tpt, int64_t ntiles_t, int64_t nsplit,
                int64_t chunk, float rfar2, const int2 **order, cudaStream_t s) {
     Layout &M = const_cast<Layout &>(L);
     const int64_t nit = ntiles_t * nsplit;
-    if (M.order32 && M.order_nit == nit && M.order_chunk == chunk &&
-        M.order_rfar2 == rfar2) {
-        *order = M.order32;
+    if (M.order32[slot] && M.order_nit[slot] == nit && M.order_chunk[slot] == chunk && M.order_rfar2[slot] == rfar2) {
+        *order = M.order32[slot];
         return SSD_OK;
     }
-    if (M.order32) { dev_free(ctx, M.order32); M.order32 = nullptr; }
+    if (M.order32[slot]) { dev_free(ctx, M.order32[slot]); M.order32[slot] = nullptr; }
     void *keys = nullptr;
     SSD_TRY(dev_alloc(ctx, sizeof(int32_t) * nit, &keys));
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, keys};
@@ -1514,14 +1512,14 @@ int item_order(ssd_ctx *ctx, const Layout &L, int tpb, int tpt, int64_t ntiles_t
     for (int64_t i = 0; i < nit; ++i) ho[start[kmax - hk[i]]++] = make_int2((int)(i % ntiles_t), (int)(i / ntiles_t));
     void *dev = nullptr;
     SSD_TRY(dev_alloc(ctx, sizeof(int2) * nit, &dev));
-    M.order32 = static_cast<int2 *>(dev);
-    SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(M.order32, ho.data(), sizeof(int2) * nit, cudaMemcpyHostToDevice,
+    M.order32[slot] = static_cast<int2 *>(dev);
+    SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(M.order32[slot], ho.data(), sizeof(int2) * nit, cudaMemcpyHostToDevice,
                                             s), "order copy"));
     SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "order sync"));
-    M.order_nit = nit;
-    M.order_chunk = chunk;
-    M.order_rfar2 = rfar2;
-    *order = M.order32;
+    M.order_nit[slot] = nit;
+    M.order_chunk[slot] = chunk;
+    M.order_rfar2[slot] = rfar2;
+    *order = M.order32[slot];
     return SSD_OK;
 }
 
@@ -1532,8 +1530,8 @@ int item_order(ssd_ctx *ctx, const Layout &L, int tpb, int tpt, int64_t ntiles_t
 // goes to the symmetric kernel, in items of the target block against at most
 // kSymTiles source tiles; the diagonal blocks and the near block pairs (both
 // directions) are items of the pair kernel of the precision (slot 0:
-// pair32_kernel, one item of 512 targets; slot 1: the fixed-point or the
-// generic FP64 kernel, two items of 256 targets).  The plan is used when far pairs are at least
+// pair32_kernel, one item of 512 targets; slot 1: the fixed-point kernel, two
+// items of 256 targets, or the generic one in double, four of 128).  The plan is used when far pairs are at least
 // half of all pairs.  The device block holds the surface descriptor, the
 // kernel constants (`cbytes` bytes at `consts`), the near and the far items.
 // `ordered` (the fixed-point FP64 kernels): the far list holds items of the
@@ -1546,7 +1544,7 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
     if (pl.block) { dev_free(ctx, pl.block); pl.block = nullptr; }
     pl.use = false;
     pl.near = pl.far = 0;
-    const int nsub = slot == 0 ? 1 : kSymBlock / kFxTPB;   // near items per block pair
+    const int nsub = slot == 0 ? 1 : kSymBlock / (ordered ? kFxTPB : kTPB64 * kTPT64);   // near items per block pair
     const int sub = kSymBlock / nsub;
     const int64_t n = L.n, n_pad = L.n_pad, nb = n_pad / kSymBlock, nch = n_pad / kChunk;
     std::vector<float4> cb(2 * nch);
@@ -1716,7 +1714,7 @@ int pair_occupancy(ssd_ctx *ctx) {
     int o32 = 0, o64 = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o32, pair32_kernel<OP_SSLDL>, kTPB32, 0);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o64, pair_kernel<float, OP_SDLT, kTPB64, kTPT64>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o64, pair_kernel<double, OP_SSLDL, kTPB64, kTPT64>,
                                                           kTPB64, 0);
     if (e != cudaSuccess) return cuda_check(ctx, e, "occupancy query");
     ctx->occ32 = o32 > 0 ? o32 : 1;
@@ -1817,7 +1815,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     int noct = 0;
     const bool use_fx = !f32 && fx_geo(L.ext, pc.delta, &geo, &noct);
     const FxSplit fs = use_fx ? fx_split_grid(ctx, n) : FxSplit();
-    const int tspan = packed32 ? kTPB32 * kTPT32 : (f32 ? kTPB64 * kTPT64 : kFxTPB / fs.groups);
+    const int tspan = packed32 ? kTPB32 * kTPT32 : (use_fx ? kFxTPB / fs.groups : kTPB64 * kTPT64);
     const int64_t ntiles_t = use_fx ? (n + tspan - 1) / tspan : n_pad / tspan;
     const int64_t ntiles_s = n_pad / kTile;
     // splits: enough CTAs for several waves of resident CTAs, so that the
@@ -1976,7 +1974,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         dim3 g = grid;
         if (ctx->lpt && L.order_ok && !rows) {
             const int2 *ord = nullptr;
-            const int st = item_order(ctx, L, kTPB32, kTPT32, ntiles_t, nsplit, chunk, ka.c.rfar2, &ord, s);
+            const int st = item_order(ctx, L, 0, kTPB32, kTPT32, ntiles_t, nsplit, chunk, ka.c.rfar2, &ord, s);
             if (st != SSD_OK) return st;
             ka.order = ord;
             g = dim3((unsigned)(ntiles_t * nsplit), 1);
@@ -1996,7 +1994,19 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
             fa.k = ka;
             e = launch_fx(op, grid, fa, fs.groups, s);
         } else {
-            e = transposed ? launch_transpose<double>(op, grid, ka, s) : launch_pair_op64(op, grid, ka, s);
+            // one target a thread and near pairs first: at 300 delta, Laplace single layer
+            // N = 1062 536 us (1073 with two targets a thread, in plain order), Stokes double
+            // layer N = 4302 1.50 ms (2.25), two spheres of 17070 points each 75 ms (84)
+            dim3 g = grid;
+            if (ctx->lpt && L.order_ok && !rows) {
+                const int2 *ord = nullptr;
+                const int st = item_order(ctx, L, 1, kTPB64, kTPT64, ntiles_t, nsplit, chunk, (float)ka.c.rfar2,
+                                          &ord, s);
+                if (st != SSD_OK) return st;
+                ka.order = ord;
+                g = dim3((unsigned)(ntiles_t * nsplit), 1);
+            }
+            e = transposed ? launch_transpose<double>(op, g, ka, s) : launch_pair_op64(op, g, ka, s);
         }
     }
     ctx->launches++;
@@ -2074,7 +2084,7 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
         // fixed point: real targets and sources only
         auto ntt = [&](int k, int span) { return fx ? (B->n[k] + span - 1) / span : B->n_pad[k] / span; };
         auto nss = [&](int k) { return fx ? (B->n[k] + unit - 1) / unit : B->n_pad[k] / unit; };
-        const int span = pr == 0 ? kTPB32 * kTPT32 : kFxTPB;
+        const int span = pr == 0 ? kTPB32 * kTPT32 : (fx ? kFxTPB : kTPB64 * kTPT64);
         const int occ = pr == 0 ? ctx->occ32 : ctx->occ64;
         const int64_t want = fx ? (int64_t)ctx->num_sms * 2 * ctx->waves_fx
                                 : (int64_t)ctx->num_sms * occ * (pr == 0 ? ctx->waves32 : 2);
