@@ -108,6 +108,7 @@ template <typename R> struct Consts {
     R rfar2;      // (rho_far delta)^2
     R tser;       // rho_series^2
     R cg;         // 2/sqrt(pi)
+    R rvec2;      // packed Laplace single layer: nearer pairs take the scalar path
 };
 
 template <typename R> struct KArgs {
@@ -415,10 +416,11 @@ __device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// The hardware approximations without the library's handling of subnormals (two
-// multiplications and a comparison each): the same bits for normal arguments
-// and results.  r^2 of a packed pair is normal (closer pairs take the scalar
-// path; padding against padding is 0 with zero weight) and 2^x has x > -58.
+// Approximate instructions with .ftz: subnormal arguments and results count as 0,
+// others give what rsqrtf and exp2f give (Stokes double layer at N = 17070: 282 us,
+// 310 with those).  r^2 of a packed pair is normal: closer pairs take the scalar
+// path, the Laplace single layer's near ones all of them where delta is tiny
+// (make_consts); padding against padding is 0 with zero weight.  2^x has x > -58.
 __device__ __forceinline__ float rsq1(float a) {
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
@@ -643,7 +645,7 @@ __global__ void __launch_bounds__(kTPB32, pair32_min_cta(OP)) pair32_kernel(cons
                             pair2<OP, false>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
                         continue;
                     }
-                    const bool serv = mall * c.inv_d2 < c.tser;
+                    const bool serv = OP == OP_LSL ? mall < c.rvec2 : mall * c.inv_d2 < c.tser;
                     if (__any_sync(0xffffffffu, serv)) {
                         // a target of the warp is within 0.5 delta of this source
                         // (the self pair or a close neighbour): scalar path with
@@ -1304,6 +1306,11 @@ Consts<R> make_consts(double delta, double rho_far) {
     c.inv_d5 = R(1.0 / (delta * delta * delta * delta * delta));
     c.rfar2 = R(rho_far * rho_far * delta * delta);
     c.tser = R(kRhoSeries * kRhoSeries);
+    // rho_series delta; where r^2 may be subnormal in FP32 beyond it, which rsq1 takes as
+    // 0, every near pair (the other operators' higher powers of 1 / r are out of range
+    // at such lengths)
+    const double s2 = kRhoSeries * kRhoSeries * delta * delta;
+    c.rvec2 = s2 < 1.2e-38 ? c.rfar2 : R(s2);
     c.cg = R(2.0 / sqrt(kPi));
     return c;
 }
