@@ -45,7 +45,8 @@ enum FieldKind { kDarcy, kVelocity, kPressure };
 //   Darcy:    ca w q / r + cb w p (yh . n) / r^3
 //   velocity: ca w [f / r + yh (yh . f) / r^3] + cb w (u . yh)(yh . n) yh / r^5
 //   pressure: ca w (yh . f) / r^3 + cb w [(u . n) / r^3 - 3 (yh . u)(yh . n) / r^5]
-// with yh = y - x_j.
+// with yh = y - x_j, high powers of 1 / r multiplied in parts (r^-5 leaves the
+// range first).
 template <FieldKind KIND>
 __global__ void __launch_bounds__(kFieldTPB) field_kernel(const FieldArgs A) {
     constexpr int NC = KIND == kVelocity ? 3 : 1, NB = KIND == kDarcy ? 1 : 3;
@@ -64,11 +65,11 @@ __global__ void __launch_bounds__(kFieldTPB) field_kernel(const FieldArgs A) {
             const double w = A.w[m], wa = A.ca * w, wb = A.cb * w;
             for (int e = 0; e < 3; ++e) {
                 sx[e][threadIdx.x] = A.xyz[e * A.n + m];
-                sn[e][threadIdx.x] = wb * A.nrm[e * A.n + m];
+                sn[e][threadIdx.x] = (KIND == kDarcy ? 1.0 : wb) * A.nrm[e * A.n + m];
             }
             for (int e = 0; e < NB; ++e) {
                 sa[e][threadIdx.x] = wa * A.a[e * A.n + m];
-                sb[e][threadIdx.x] = A.b[e * A.n + m];
+                sb[e][threadIdx.x] = (KIND == kDarcy ? wb : 1.0) * A.b[e * A.n + m];
             }
         }
         __syncthreads();
@@ -79,16 +80,16 @@ __global__ void __launch_bounds__(kFieldTPB) field_kernel(const FieldArgs A) {
             const double ri2 = ri * ri, ri3 = ri2 * ri;
             const double dn = fma(d[2], sn[2][j], fma(d[1], sn[1][j], d[0] * sn[0][j]));
             if constexpr (KIND == kDarcy) {
-                s[0] = fma(sa[0][j], ri, fma(sb[0][j] * dn, ri3, s[0]));
+                s[0] = fma(fma(sb[0][j], dn * ri2, sa[0][j]), ri, s[0]);
             } else {
                 const double df = fma(d[2], sa[2][j], fma(d[1], sa[1][j], d[0] * sa[0][j]));
                 const double du = fma(d[2], sb[2][j], fma(d[1], sb[1][j], d[0] * sb[0][j]));
                 if constexpr (KIND == kVelocity) {
-                    const double b = fma(df, ri3, du * dn * (ri3 * ri2));
+                    const double b = fma(df, ri3, (du * ri2) * (dn * ri3));
                     for (int e = 0; e < 3; ++e) s[e] = fma(sa[e][j], ri, fma(d[e], b, s[e]));
                 } else {
                     const double un = fma(sb[2][j], sn[2][j], fma(sb[1][j], sn[1][j], sb[0][j] * sn[0][j]));
-                    s[0] = fma(ri3, df + (un - 3.0 * du * dn * ri2), s[0]);   // n_S = -n flips both terms
+                    s[0] = fma(ri3, df + (un - 3.0 * du * (dn * ri2)), s[0]);   // n_S = -n flips both terms
                 }
             }
         }
@@ -363,12 +364,12 @@ __global__ void __launch_bounds__(kFieldTPB, 2) field_fx_kernel(const FieldFx A)
                     const d4 e1 = A.d1[tile + j];
                     const double df = fma(d[2], e1.z, fma(d[1], e1.y, d[0] * e1.x));
                     const double du = fma(d[2], e0.z, fma(d[1], e0.y, d[0] * e0.x));
-                    const double b = fma(df, ri3, du * dn * (ri3 * ri2));
+                    const double b = fma(df, ri3, (du * ri2) * (dn * ri3));
                     v[0] = fma(e1.x, ri, fma(d[0], b, v[0]));
                     v[1] = fma(e1.y, ri, fma(d[1], b, v[1]));
                     v[2] = fma(e1.z, ri, fma(d[2], b, v[2]));
                 } else {
-                    v[0] = fma(e0.y, ri, fma(e0.x * dn, ri3, v[0]));
+                    v[0] = fma(fma(e0.x, dn * ri2, e0.y), ri, v[0]);
                 }
             }
         }
