@@ -23,14 +23,23 @@ int cuda_check(ssd_ctx *ctx, cudaError_t e, const char *what) {
 
 int launch_check(ssd_ctx *ctx, const char *what) { return cuda_check(ctx, cudaGetLastError(), what); }
 
-int dev_alloc(ssd_ctx *ctx, size_t bytes, void **p) {
-    bytes = (bytes + 255) & ~size_t(255);
-    if (bytes == 0) bytes = 256;
+// smallest free block of the pool of at least this size, or -1
+static int dev_best(const ssd_ctx *ctx, size_t bytes) {
     int best = -1;
     for (size_t k = 0; k < ctx->pool.size(); ++k) {
         const auto &b = ctx->pool[k];
         if (!b.used && b.bytes >= bytes && (best < 0 || b.bytes < ctx->pool[best].bytes)) best = (int)k;
     }
+    return best;
+}
+
+static size_t dev_round(size_t bytes) { return bytes == 0 ? 256 : (bytes + 255) & ~size_t(255); }
+
+bool dev_cached(const ssd_ctx *ctx, size_t bytes) { return dev_best(ctx, dev_round(bytes)) >= 0; }
+
+int dev_alloc(ssd_ctx *ctx, size_t bytes, void **p) {
+    bytes = dev_round(bytes);
+    const int best = dev_best(ctx, bytes);
     if (best >= 0) {
         ctx->pool[best].used = true;
         *p = ctx->pool[best].p;

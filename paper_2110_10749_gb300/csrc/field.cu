@@ -131,7 +131,7 @@ struct FieldFx {
     const FxI4 *tab;
     int64_t chunk;
     int nsplit;
-    double *part;                 // [split][NC][nt]
+    double *part;                 // [split][NC][nt]; one split: not used
     double *out;
 };
 
@@ -394,6 +394,11 @@ __global__ void __launch_bounds__(kFieldTPB, 2) field_fx_kernel(const FieldFx A)
             for (int c = 0; c < NC; ++c) sum[c] += s_sum[c][threadIdx.x + k * NT];
     }
     if (!act) return;
+    if (A.nsplit == 1) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) A.out[c * A.nt + t] = sum[c] + A.u0[c];
+        return;
+    }
 #pragma unroll
     for (int c = 0; c < NC; ++c) A.part[((int64_t)blockIdx.y * NC + c) * A.nt + t] = sum[c];
 }
@@ -415,7 +420,9 @@ __global__ void __launch_bounds__(64) field_sum_kernel(const FieldFx A) {
     A.out[g] = (s0 + s1) + A.u0[g / A.nt];
 }
 
-// Fixed-point evaluation on a prepared layout; *done is false where it does not serve the point set.
+// Fixed-point evaluation on a prepared layout; *done is false where it does not serve
+// the point set, or has no workspace: a captured call whose pool has no block of the
+// size, a device without the memory.  The kernel in double needs none.
 template <bool VEL> int field_fx(ssd_ctx *ctx, const ssd_points *pts, const FieldArgs &F, cudaStream_t s, bool *done) {
     *done = false;
     if (!pts->layout) return SSD_OK;
@@ -443,9 +450,20 @@ template <bool VEL> int field_fx(ssd_ctx *ctx, const ssd_points *pts, const Fiel
     const size_t o_x = carve(sizeof(l4) * L.n_pad), o_b = carve(sizeof(int4) * 2 * (L.n_pad / kChunk)),
                  o_0 = carve(sizeof(d4) * L.n_pad), o_1 = VEL ? carve(sizeof(d4) * L.n_pad) : 0,
                  o_m = carve(sizeof(unsigned long long) * 2 * A.nblk),
-                 o_p = carve(sizeof(double) * NC * F.nt * A.nsplit);
+                 o_p = A.nsplit > 1 ? carve(sizeof(double) * NC * F.nt * A.nsplit) : 0;
     void *ws = nullptr;
-    SSD_TRY(dev_alloc(ctx, off, &ws));
+    if (!dev_cached(ctx, off)) {
+        if (capturing(s)) return SSD_OK;
+        const int st = dev_alloc(ctx, off, &ws);
+        if (st == SSD_ENOMEM) {
+            ctx->err.clear();
+            cudaGetLastError();
+            return SSD_OK;
+        }
+        SSD_TRY(st);
+    } else {
+        SSD_TRY(dev_alloc(ctx, off, &ws));
+    }
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, ws};
     char *b = static_cast<char *>(ws);
     A.X = reinterpret_cast<l4 *>(b + o_x);
@@ -459,9 +477,12 @@ template <bool VEL> int field_fx(ssd_ctx *ctx, const ssd_points *pts, const Fiel
     SSD_TRY(cuda_check(ctx, groups == 1 ? launch_pdl(field_fx_kernel<VEL, 1>, grid, dim3(kFieldTPB), 0, s, A)
                                         : launch_pdl(field_fx_kernel<VEL, 4>, grid, dim3(kFieldTPB), 0, s, A),
                        "field kernel"));
-    SSD_TRY(cuda_check(ctx, launch_pdl(field_sum_kernel<VEL>, dim3((unsigned)((NC * F.nt + 63) / 64)), dim3(64), 0, s, A),
-                       "field sums"));
-    ctx->launches += 3;
+    ctx->launches += 2;
+    if (A.nsplit > 1) {
+        SSD_TRY(cuda_check(ctx, launch_pdl(field_sum_kernel<VEL>, dim3((unsigned)((NC * F.nt + 63) / 64)), dim3(64), 0, s,
+                                           A), "field sums"));
+        ctx->launches++;
+    }
     *done = true;
     return SSD_OK;
 }

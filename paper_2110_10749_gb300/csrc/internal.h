@@ -141,6 +141,16 @@ int launch_check(ssd_ctx *ctx, const char *what);
 // on one stream at a time.
 int dev_alloc(ssd_ctx *ctx, size_t bytes, void **p);
 void dev_free(ssd_ctx *ctx, void *p);
+bool dev_cached(const ssd_ctx *ctx, size_t bytes);   // dev_alloc would take a block of the pool
+// whether work on s is being captured, where nothing may be allocated
+inline bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {   // the legacy stream while another one captures
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
 
 // Layout handling (ctx.cu).  A temporary (unsorted) layout is built into pool
 // memory when pts->layout is NULL; release it with release_layout.

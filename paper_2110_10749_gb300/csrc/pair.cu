@@ -1779,12 +1779,7 @@ static size_t fx_position_bytes(const Layout &L) { return sizeof(l4) * L.n_pad +
 // a stream order of their own: such calls make the positions in their
 // workspace (about 3 us more).
 static bool fx_keeps(const ssd_ctx *ctx, const Layout &L, cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {   // the legacy stream while another one captures
-        cudaGetLastError();
-        return false;
-    }
-    return L.owner == ctx && st == cudaStreamCaptureStatusNone;
+    return L.owner == ctx && !capturing(s);
 }
 
 // Grid positions of a layout at a smoothing radius: in ws, or (ws NULL) kept
