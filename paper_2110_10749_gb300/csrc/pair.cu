@@ -22,6 +22,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <memory>
+
 #include "internal.h"
 #include "erfcx_coef.h"
 #include "fx_geo.h"
@@ -1585,24 +1587,10 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
         }
         return g2 >= rfar2;
     };
-    std::vector<BItem> near, far2;
+    std::vector<BItem> near;
     std::vector<SymItem> far;
+    std::vector<char> is_far(ordered ? (size_t)nb * nb : 0, 0);
     int64_t far_blocks = 0;
-    if (ordered)   // runs of far blocks of every target block, both directions
-        for (int64_t i = 0; i < nb; ++i)
-            for (int64_t k = 0; k < nb;) {
-                if (k == i || !far_pair(i, k) || k * kSymBlock >= n) { ++k; continue; }
-                int64_t k1 = k;
-                while (k1 < nb && k1 != i && far_pair(i, k1) && k1 * kSymBlock < n) ++k1;
-                for (int64_t t = k * kSymBlock; t < k1 * kSymBlock; t += (int64_t)kSymTiles * kTile) {
-                    int64_t e = t + (int64_t)kSymTiles * kTile;
-                    if (e > k1 * kSymBlock) e = k1 * kSymBlock;
-                    for (int q = 0; q < nsub; ++q)
-                        if (i * kSymBlock + q * sub < n)
-                            far2.push_back(BItem{(int32_t)(i * kSymBlock + q * sub), (int32_t)t, (int32_t)e, 0, 0, 0, 0, 0});
-                }
-                k = k1;
-            }
     auto near_item = [&](int64_t ti, int64_t si) {   // targets of block ti against sources of block si
         for (int q = 0; q < nsub; ++q)
             near.push_back(BItem{(int32_t)(ti * kSymBlock + q * sub), (int32_t)(si * kSymBlock),
@@ -1621,6 +1609,11 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
             int64_t k1 = k;
             while (k1 < nb && far_pair(i, k1)) ++k1;
             far_blocks += k1 - k;
+            if (ordered) {
+                for (int64_t q = k; q < k1; ++q) is_far[i * nb + q] = is_far[q * nb + i] = 1;
+                k = k1;
+                continue;
+            }
             for (int64_t t = k * kSymBlock; t < k1 * kSymBlock; t += (int64_t)kSymTiles * kTile) {
                 int64_t e = t + (int64_t)kSymTiles * kTile;
                 if (e > k1 * kSymBlock) e = k1 * kSymBlock;
@@ -1632,27 +1625,52 @@ int sym_plan(ssd_ctx *ctx, const Layout &L, int slot, double rfar2, const void *
     pl.rfar2 = rfar2;
     // far pairs (both directions) against all ordered pairs
     if (2.0 * (double)far_blocks < 0.5 * (double)nb * (double)nb) return SSD_OK;
+    // `ordered`: runs of far blocks of every target block, both directions; calls f(first
+    // target, first source, end) for every item
+    auto far_items = [&](auto f) {
+        for (int64_t i = 0; i < nb; ++i)
+            for (int64_t k = 0; k < nb;) {
+                if (!is_far[i * nb + k]) { ++k; continue; }
+                int64_t k1 = k;
+                while (k1 < nb && is_far[i * nb + k1]) ++k1;
+                for (int64_t t = k * kSymBlock; t < k1 * kSymBlock; t += (int64_t)kSymTiles * kTile) {
+                    int64_t e = t + (int64_t)kSymTiles * kTile;
+                    if (e > k1 * kSymBlock) e = k1 * kSymBlock;
+                    for (int q = 0; q < nsub; ++q)
+                        if (i * kSymBlock + q * sub < n) f(i * kSymBlock + q * sub, t, e);
+                }
+                k = k1;
+            }
+    };
+    size_t nfar = far.size();
+    if (ordered) far_items([&](int64_t, int64_t, int64_t) { ++nfar; });
     size_t off = 0;
     auto carve = [&](size_t b) { size_t o = off; off += (b + 255) & ~size_t(255); return o; };
     const size_t o_surf = carve(sizeof(BSurf)), o_c = carve(cbytes);
     const size_t o_near = carve(sizeof(BItem) * near.size()),
-                 o_far = carve(ordered ? sizeof(BItem) * far2.size() : sizeof(SymItem) * far.size());
+                 o_far = carve((ordered ? sizeof(BItem) : sizeof(SymItem)) * nfar);
     void *blk = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &blk));
     char *b = static_cast<char *>(blk);
     const BSurf sf{0, n_pad, n, 0, 1, 0, 0, 0};
-    std::vector<char> host(off);
-    memcpy(host.data() + o_surf, &sf, sizeof(sf));
-    memcpy(host.data() + o_c, consts, cbytes);
-    memcpy(host.data() + o_near, near.data(), sizeof(BItem) * near.size());
-    if (ordered) memcpy(host.data() + o_far, far2.data(), sizeof(BItem) * far2.size());
-    else memcpy(host.data() + o_far, far.data(), sizeof(SymItem) * far.size());
-    const int st = cuda_check(ctx, cudaMemcpyAsync(b, host.data(), off, cudaMemcpyHostToDevice, s), "plan copy");
+    std::unique_ptr<char[]> host(new char[off]);
+    memcpy(host.get() + o_surf, &sf, sizeof(sf));
+    memcpy(host.get() + o_c, consts, cbytes);
+    memcpy(host.get() + o_near, near.data(), sizeof(BItem) * near.size());
+    if (ordered) {
+        BItem *item = reinterpret_cast<BItem *>(host.get() + o_far);
+        far_items([&](int64_t ti, int64_t s_beg, int64_t s_end) {
+            *item++ = BItem{(int32_t)ti, (int32_t)s_beg, (int32_t)s_end, 0, 0, 0, 0, 0};
+        });
+    } else {
+        memcpy(host.get() + o_far, far.data(), sizeof(SymItem) * nfar);
+    }
+    const int st = cuda_check(ctx, cudaMemcpyAsync(b, host.get(), off, cudaMemcpyHostToDevice, s), "plan copy");
     if (st == SSD_OK) SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "plan sync"));
     if (st != SSD_OK) { dev_free(ctx, blk); return st; }
     pl.block = blk;
     pl.near = (int64_t)near.size();
-    pl.far = ordered ? (int64_t)far2.size() : (int64_t)far.size();
+    pl.far = (int64_t)nfar;
     pl.use = true;
     return SSD_OK;
 }
