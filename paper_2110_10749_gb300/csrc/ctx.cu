@@ -172,10 +172,11 @@ __global__ void bbox_union_kernel(double *out) {   // one warp
     }
 }
 
-static void launch_bbox(const double *xyz, int64_t n, double *bb, cudaStream_t s) {
+static void launch_bbox(ssd_ctx *ctx, const double *xyz, int64_t n, double *bb, cudaStream_t s) {
     const int blocks = n <= 4096 ? 1 : kBoxBlocks;
     bbox_kernel<<<blocks, 256, 0, s>>>(xyz, n, bb);
     if (blocks > 1) bbox_union_kernel<<<1, kBoxBlocks, 0, s>>>(bb);
+    ctx->launches += blocks > 1 ? 2 : 1;
 }
 
 __device__ __forceinline__ uint32_t spread10(uint32_t v) {
@@ -516,9 +517,9 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
             double *bb = reinterpret_cast<double *>(tb + o_bb);
             const unsigned gn = (unsigned)((n + 255) / 256);
             batch_esurf_kernel<<<gn, 256, 0, s>>>(dmeta, ns, n, out.elem_surf);
-            launch_bbox(b->xyz, n, bb, s);
+            launch_bbox(ctx, b->xyz, n, bb, s);
             batch_key_kernel<<<gn, 256, 0, s>>>(b->xyz, n, bb, out.elem_surf, k0, i0);
-            ctx->launches += 4;
+            ctx->launches += 2;
             st = launch_check(ctx, "batch keys");
             if (st == SSD_OK) {
                 cudaError_t e = cub::DeviceRadixSort::SortPairs(tb + o_cub, cub_bytes, k0, k1, i0, i1, (int)n, 0,
@@ -633,9 +634,9 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cuda
         uint32_t *k0 = reinterpret_cast<uint32_t *>(tb + o_k0), *k1 = reinterpret_cast<uint32_t *>(tb + o_k1);
         int32_t *i0 = reinterpret_cast<int32_t *>(tb + o_i0), *i1 = reinterpret_cast<int32_t *>(tb + o_i1);
         double *bb = reinterpret_cast<double *>(tb + o_bb);
-        launch_bbox(pts->xyz, n, bb, s);
+        launch_bbox(ctx, pts->xyz, n, bb, s);
         morton_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pts->xyz, n, bb, k0, i0);
-        ctx->launches += 3;
+        ctx->launches += 1;
         st = launch_check(ctx, "morton keys");
         if (st == SSD_OK) {
             cudaError_t e = cub::DeviceRadixSort::SortPairs(tb + o_cub, cub_bytes, k0, k1, i0, i1, (int)n, 0, 30, s);
