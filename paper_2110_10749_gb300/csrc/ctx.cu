@@ -716,7 +716,13 @@ int ssd_ctx_create(ssd_ctx **out, int device) {
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return SSD_ECUDA; }
     ctx->num_sms = prop.multiProcessorCount;
     if (cudaMallocHost((void **)&ctx->hbuf, sizeof(double) * (512 + kFrameLen * kHostFrames)) != cudaSuccess) { delete ctx; return SSD_ENOMEM; }
-    if (pair_occupancy(ctx) != SSD_OK) { cudaFreeHost(ctx->hbuf); delete ctx; return SSD_ECUDA; }
+    const int st = pair_occupancy(ctx);
+    if (st != SSD_OK) {
+        for (auto &b : ctx->pool) cudaFree(b.p);
+        cudaFreeHost(ctx->hbuf);
+        delete ctx;
+        return st;
+    }
     // tuning knob: waves of resident CTAs in an FP32C pair-kernel grid
     if (const char *w = getenv("SSD_PAIR_WAVES")) {
         const int v = atoi(w);

@@ -231,7 +231,7 @@ FX_HD double fx_value(const FxMac &a) { return (double)a.h * 16777216.0 + (doubl
 
 // Kernel tables of sigma_1 .. sigma_4 on v in [1, 2^kFxMaxOct), then t^(-1/2) on
 // t in [1, 4): host array of kFxTabEntries entries, built once per process
-// (fx_table.cu).
+// (fx_table.cu); NULL without the memory.
 const FxI4 *fx_table_host();
 
 }  // namespace ssd

@@ -492,8 +492,10 @@ template <int OP, bool FAR = false> cudaError_t fx_attr1() {
 // Uploads the kernel tables of a context and lets the kernels use them.
 int fx_init(ssd_ctx *ctx) {
     const size_t bytes = (size_t)kFxTabEntries * kFxEntry * sizeof(FxI4);
+    const FxI4 *host = fx_table_host();
+    if (!host) return set_error(ctx, SSD_ENOMEM, "kernel tables: no host memory");
     SSD_TRY(dev_alloc(ctx, bytes, &ctx->fx_tab));
-    SSD_TRY(cuda_check(ctx, cudaMemcpy(ctx->fx_tab, fx_table_host(), bytes, cudaMemcpyHostToDevice), "kernel tables"));
+    SSD_TRY(cuda_check(ctx, cudaMemcpy(ctx->fx_tab, host, bytes, cudaMemcpyHostToDevice), "kernel tables"));
     cudaError_t e = fx_attr1<OP_LSL>();
     if (e == cudaSuccess) e = fx_attr1<OP_LDL>();
     if (e == cudaSuccess) e = fx_attr1<OP_SSL>();

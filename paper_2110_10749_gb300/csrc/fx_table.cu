@@ -13,8 +13,9 @@
 #include <math.h>
 
 #include <algorithm>
+#include <exception>
 #include <mutex>
-#include <system_error>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -136,7 +137,7 @@ std::vector<FxI4> build() {
     int first = 1;
     try {
         for (; first < step; ++first) helpers.emplace_back(segments, first, step);
-    } catch (const std::system_error &) {   // no more threads: the rest here
+    } catch (const std::exception &) {   // no more threads: the rest here
     }
     segments(0, step);
     for (; first < step; ++first) segments(first, step);
@@ -149,7 +150,11 @@ std::vector<FxI4> build() {
 const FxI4 *fx_table_host() {
     static std::once_flag once;
     static std::vector<FxI4> tab;
-    std::call_once(once, [] { tab = build(); });
+    try {
+        std::call_once(once, [] { tab = build(); });
+    } catch (const std::bad_alloc &) {   // the next call tries again
+        return nullptr;
+    }
     return tab.data();
 }
 
