@@ -154,7 +154,8 @@ inline bool capturing(cudaStream_t s) {
 
 // Layout handling (ctx.cu).  A temporary (unsorted) layout is built into pool
 // memory when pts->layout is NULL; release it with release_layout.
-int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, Layout *L, cudaStream_t s);
+// `extent`: with L->ext, which the fixed-point kernels need
+int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, bool extent, Layout *L, cudaStream_t s);
 void release_layout(ssd_ctx *ctx, Layout *L);
 struct LayoutRef {
     const Layout *L = nullptr;
@@ -162,7 +163,7 @@ struct LayoutRef {
     ssd_ctx *ctx = nullptr;
     ~LayoutRef() { if (ctx && tmp.block) release_layout(ctx, &tmp); }
 };
-int get_layout(ssd_ctx *ctx, const ssd_points *pts, LayoutRef *ref, cudaStream_t s);
+int get_layout(ssd_ctx *ctx, const ssd_points *pts, LayoutRef *ref, cudaStream_t s, bool extent = true);
 int check_points(ssd_ctx *ctx, const ssd_points *pts);
 
 // Pinned frame of kFrameLen doubles and two events for one GMRES solve, so that

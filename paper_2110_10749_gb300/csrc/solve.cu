@@ -1987,7 +1987,7 @@ int op_entry(ssd_ctx *ctx, const ssd_points *pts, const PairCall &pc, cudaStream
     if (pc.prec != SSD_FP64 && pc.prec != SSD_FP32C) return set_error(ctx, SSD_EINVAL, "unknown precision");
     if (!pc.dens0 || !pc.out) return set_error(ctx, SSD_EINVAL, "NULL density or output");
     LayoutRef lref;
-    SSD_TRY(get_layout(ctx, pts, &lref, s));
+    SSD_TRY(get_layout(ctx, pts, &lref, s, pc.prec == SSD_FP64));
     return pair_apply(ctx, *lref.L, pc, s);
 }
 
@@ -2057,7 +2057,7 @@ int ssd_points_order(ssd_ctx *ctx, const ssd_points *pts, int32_t *order, ssd_st
     SSD_TRY(check_points(ctx, pts));
     cudaStream_t s = (cudaStream_t)stream;
     LayoutRef lref;
-    SSD_TRY(get_layout(ctx, pts, &lref, s));
+    SSD_TRY(get_layout(ctx, pts, &lref, s, false));
     SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(order, lref.L->perm, sizeof(int32_t) * pts->n, cudaMemcpyDeviceToHost, s),
                        "order copy"));
     return cuda_check(ctx, cudaStreamSynchronize(s), "order sync");
