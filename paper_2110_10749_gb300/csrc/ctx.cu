@@ -133,14 +133,14 @@ static int drain_timing(ssd_ctx *ctx) {
 // ------------------------------------------------------------------ layouts
 namespace {
 
-// Bounding box of n points: one block, or 32 partial boxes (block b: out + 6 (1 + b))
+// Bounding box of n points: one block, or 32 partial boxes (block b: part + 6 b)
 // and then their union.  The comparisons are double precision, 1.6 a clock and SM,
 // six a point: preparing 78106 points took 344 us with one block and takes 190,
 // 17070 points 188 and 153; up to 4096 points the second launch costs as much as it
 // saves.
 constexpr int kBoxBlocks = 32;
 
-__global__ void bbox_kernel(const double *xyz, int64_t n, double *out) {
+__global__ void bbox_kernel(const double *xyz, int64_t n, double *out, double *part) {
     __shared__ double red[6][256];   // (lo, -hi)
     double v[6] = {1e300, 1e300, 1e300, 1e300, 1e300, 1e300};
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
@@ -157,11 +157,11 @@ __global__ void bbox_kernel(const double *xyz, int64_t n, double *out) {
         __syncthreads();
     }
     if (threadIdx.x < 6)
-        out[6 * (gridDim.x > 1 ? 1 + blockIdx.x : 0) + threadIdx.x] = threadIdx.x < 3 ? red[threadIdx.x][0] : -red[threadIdx.x][0];
+        (gridDim.x > 1 ? part + 6 * blockIdx.x : out)[threadIdx.x] = threadIdx.x < 3 ? red[threadIdx.x][0] : -red[threadIdx.x][0];
 }
 
-__global__ void bbox_union_kernel(double *out) {   // one warp
-    const double *p = out + 6 * (1 + threadIdx.x);
+__global__ void bbox_union_kernel(double *out, const double *part) {   // one warp
+    const double *p = part + 6 * threadIdx.x;
     for (int k = 0; k < 6; ++k) {
         double v = p[k];
         for (int off = 16; off > 0; off >>= 1) {
@@ -172,10 +172,10 @@ __global__ void bbox_union_kernel(double *out) {   // one warp
     }
 }
 
-static void launch_bbox(ssd_ctx *ctx, const double *xyz, int64_t n, double *bb, cudaStream_t s) {
+static void launch_bbox(ssd_ctx *ctx, const double *xyz, int64_t n, double *bb, double *part, cudaStream_t s) {
     const int blocks = n <= 4096 ? 1 : kBoxBlocks;
-    bbox_kernel<<<blocks, 256, 0, s>>>(xyz, n, bb);
-    if (blocks > 1) bbox_union_kernel<<<1, kBoxBlocks, 0, s>>>(bb);
+    bbox_kernel<<<blocks, 256, 0, s>>>(xyz, n, bb, part);
+    if (blocks > 1) bbox_union_kernel<<<1, kBoxBlocks, 0, s>>>(bb, part);
     ctx->launches += blocks > 1 ? 2 : 1;
 }
 
@@ -266,41 +266,57 @@ __device__ void wsum_block(const double *w, int64_t n, double *red, double *out)
 }
 
 // Extent (see internal.h) of points [off[y], off[y + 1]) of surface y =
-// blockIdx.y (off NULL: all n points), block x of kExtentBlocks partials each.
-// With wsum, block 0 of one more sums the weights beside them (a launch of its own made
-// the layout of 1062 points take 7 us longer, with one block for the box).
+// blockIdx.y (off NULL: all n points), one partial per block x.  With wsum, block 0 of
+// one more sums the weights beside them (a launch of its own made the layout of 1062
+// points take 7 us longer, with one block for the box).  BOX: with the box of the points,
+// six double-precision minima a point; prepared sets have it already.  The magnitudes
+// are compared as integers, which order like the nonnegative doubles they are the
+// bits of, with infinities and NaN above all finite ones.
+// Preparing and releasing 1062 points takes 78 us (86 with a second box and eight
+// double-precision minima through shared memory, 77 without an extent).
+template <bool BOX>
 __global__ void extent_kernel(const double *xyz, const double *nrm, const double *w, int64_t n, const int64_t *off,
                               Extent *out, double *wsum) {
-    __shared__ double red[8][256];
+    __shared__ double red[BOX ? 6 : 1][256];
+    __shared__ unsigned long long top[2][8];
     const int64_t nb = (int64_t)gridDim.x - (wsum ? 1 : 0), blk = (int64_t)blockIdx.x - (wsum ? 1 : 0);
     if (blk < 0) {
         wsum_block(w, n, red[0], wsum);
         return;
     }
     const int64_t beg = off ? off[blockIdx.y] : 0, end = off ? off[blockIdx.y + 1] : n;
-    double v[8] = {1e308, 1e308, 1e308, 1e308, 1e308, 1e308, 0.0, 1.0};   // lo, -hi (minima), -mmax, fin
+    double v[6] = {1e308, 1e308, 1e308, 1e308, 1e308, 1e308};   // lo, -hi
+    unsigned long long mx = 0, mm = 0;                          // largest |x|, |w n|
+    auto bits = [](double a) { return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull; };
     for (int64_t i = beg + blk * 256 + threadIdx.x; i < end; i += nb * 256) {
         for (int c = 0; c < 3; ++c) {
-            const double x = xyz[c * n + i], m = w[i] * nrm[c * n + i];
-            v[c] = fmin(v[c], x);
-            v[3 + c] = fmin(v[3 + c], -x);
-            v[6] = fmin(v[6], -fabs(m));
-            if (!isfinite(x) || !isfinite(m)) v[7] = 0.0;
+            const double x = xyz[c * n + i];
+            if (BOX) { v[c] = fmin(v[c], x); v[3 + c] = fmin(v[3 + c], -x); }
+            mx = max(mx, bits(x));
+            mm = max(mm, bits(w[i] * nrm[c * n + i]));
         }
     }
-    for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = v[q];
-    __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
-        if (threadIdx.x < st)
-            for (int q = 0; q < 8; ++q)
-                red[q][threadIdx.x] = fmin(red[q][threadIdx.x], red[q][threadIdx.x + st]);
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, o));
     }
+    if ((threadIdx.x & 31) == 0) { top[0][threadIdx.x >> 5] = mx; top[1][threadIdx.x >> 5] = mm; }
+    if (BOX)
+        for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = v[q];
+    __syncthreads();
+    if (BOX)
+        for (int st = 128; st > 0; st >>= 1) {
+            if (threadIdx.x < st)
+                for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = fmin(red[q][threadIdx.x], red[q][threadIdx.x + st]);
+            __syncthreads();
+        }
     if (threadIdx.x == 0) {
-        Extent e;
-        for (int c = 0; c < 3; ++c) { e.lo[c] = red[c][0]; e.hi[c] = -red[3 + c][0]; }
-        e.mmax = -red[6][0];
-        e.fin = red[7][0];
+        Extent e{};
+        if (BOX)
+            for (int c = 0; c < 3; ++c) { e.lo[c] = red[c][0]; e.hi[c] = -red[3 + c][0]; }
+        for (int k = 1; k < 8; ++k) { mx = max(mx, top[0][k]); mm = max(mm, top[1][k]); }
+        e.fin = mx < 0x7ff0000000000000ull && mm < 0x7ff0000000000000ull ? 1.0 : 0.0;
+        e.mmax = __longlong_as_double((long long)mm);
         out[blockIdx.y * nb + blk] = e;
     }
 }
@@ -517,7 +533,7 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
             double *bb = reinterpret_cast<double *>(tb + o_bb);
             const unsigned gn = (unsigned)((n + 255) / 256);
             batch_esurf_kernel<<<gn, 256, 0, s>>>(dmeta, ns, n, out.elem_surf);
-            launch_bbox(ctx, b->xyz, n, bb, s);
+            launch_bbox(ctx, b->xyz, n, bb, bb + 6, s);
             batch_key_kernel<<<gn, 256, 0, s>>>(b->xyz, n, bb, out.elem_surf, k0, i0);
             ctx->launches += 2;
             st = launch_check(ctx, "batch keys");
@@ -536,7 +552,7 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
                 batch_chunk_box_kernel<<<(unsigned)((np / kChunk + 127) / 128), 128, 0, s>>>(out.L);
                 batch_wsum_kernel<<<ns, 256, 0, s>>>(b->w, dmeta, out.d_wsum);
                 for (int k = 0; k < ns; k += 65535)   // grid.y limit
-                    extent_kernel<<<dim3(1, (unsigned)(ns - k < 65535 ? ns - k : 65535)), 256, 0, s>>>(
+                    extent_kernel<true><<<dim3(1, (unsigned)(ns - k < 65535 ? ns - k : 65535)), 256, 0, s>>>(
                         b->xyz, b->nrm, b->w, n, dmeta + k, dext + k, nullptr);
                 ctx->launches += 4;
                 st = launch_check(ctx, "batch fill");
@@ -597,8 +613,8 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, bool extent, La
     const size_t o_p64 = carve(sizeof(d4) * n_pad);
     const size_t o_w64 = carve(sizeof(d4) * n_pad);
     const size_t o_cb = carve(sizeof(float4) * 2 * (n_pad / kChunk));
-    // weight sum, then the extent partials: one host read
-    const size_t o_ws = carve(sizeof(double) * 8 + sizeof(Extent) * kExtentBlocks);
+    // weight sum, box of the points, extent partials: one host read
+    const size_t o_ws = carve(sizeof(double) * 16 + sizeof(Extent) * kExtentBlocks);
     void *blk = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &blk));
     char *b = static_cast<char *>(blk);
@@ -615,6 +631,8 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, bool extent, La
     out.cbox = reinterpret_cast<float4 *>(b + o_cb);
     double *dsum = reinterpret_cast<double *>(b + o_ws);
 
+    // blocks of the extent: some 256 points each on small sets
+    const int eb = !extent ? 0 : (n < 256 * kExtentBlocks ? (int)((n + 255) / 256) : kExtentBlocks);
     int32_t *sorted = nullptr;
     void *tmp = nullptr;
     int st = SSD_OK;
@@ -627,14 +645,14 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, bool extent, La
         auto tcarve = [&](size_t bb) { size_t o = t_off; t_off += (bb + 255) & ~size_t(255); return o; };
         const size_t o_k0 = tcarve(sizeof(uint32_t) * n), o_k1 = tcarve(sizeof(uint32_t) * n);
         const size_t o_i0 = tcarve(sizeof(int32_t) * n), o_i1 = tcarve(sizeof(int32_t) * n);
-        const size_t o_bb = tcarve(sizeof(double) * 6 * (1 + kBoxBlocks)), o_cub = tcarve(cub_bytes);
+        const size_t o_bb = tcarve(sizeof(double) * 6 * kBoxBlocks), o_cub = tcarve(cub_bytes);
         st = dev_alloc(ctx, t_off, &tmp);
         if (st != SSD_OK) { release_layout(ctx, &out); return st; }
         char *tb = static_cast<char *>(tmp);
         uint32_t *k0 = reinterpret_cast<uint32_t *>(tb + o_k0), *k1 = reinterpret_cast<uint32_t *>(tb + o_k1);
         int32_t *i0 = reinterpret_cast<int32_t *>(tb + o_i0), *i1 = reinterpret_cast<int32_t *>(tb + o_i1);
-        double *bb = reinterpret_cast<double *>(tb + o_bb);
-        launch_bbox(ctx, pts->xyz, n, bb, s);
+        double *bb = dsum + 8;
+        launch_bbox(ctx, pts->xyz, n, bb, reinterpret_cast<double *>(tb + o_bb), s);
         morton_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pts->xyz, n, bb, k0, i0);
         ctx->launches += 1;
         st = launch_check(ctx, "morton keys");
@@ -650,21 +668,26 @@ int build_layout(ssd_ctx *ctx, const ssd_points *pts, bool sort, bool extent, La
                                                                           sorted, out);
         // (without the extent's blocks the Stokes double layer in FP32C on 2406 plain points
         // takes 146.2 us, 147.8 with them)
-        extent_kernel<<<1 + (extent ? kExtentBlocks : 0), 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, nullptr,
-                                                                       reinterpret_cast<Extent *>(dsum + 8), dsum);
+        Extent *part = reinterpret_cast<Extent *>(dsum + 16);
+        if (sort) extent_kernel<false><<<1 + eb, 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, nullptr, part, dsum);
+        else extent_kernel<true><<<1 + eb, 256, 0, s>>>(pts->xyz, pts->nrm, pts->w, n, nullptr, part, dsum);
         chunk_box_kernel<<<(unsigned)((n_pad / kChunk + 127) / 128), 128, 0, s>>>(out);
         ctx->launches += 3;
         st = launch_check(ctx, "layout fill");
     }
-    static_assert(8 + 8 * kExtentBlocks <= 512, "the read fits the pinned scratch");
+    static_assert(16 + 8 * kExtentBlocks <= 512, "the read fits the pinned scratch");
     if (st == SSD_OK) st = cuda_check(ctx, cudaMemcpyAsync(ctx->hbuf, dsum,
-                                                           sizeof(double) * 8 + (extent ? sizeof(Extent) * kExtentBlocks : 0),
+                                                           eb ? sizeof(double) * 16 + sizeof(Extent) * eb : sizeof(double),
                                                            cudaMemcpyDeviceToHost, s), "wsum copy");
     if (st == SSD_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "layout sync");
     if (tmp) dev_free(ctx, tmp);
     if (st != SSD_OK) { release_layout(ctx, &out); return st; }
     out.wsum = ctx->hbuf[0];
-    if (extent) out.ext = merge_extents(reinterpret_cast<const Extent *>(ctx->hbuf + 8), kExtentBlocks);
+    if (extent) {
+        out.ext = merge_extents(reinterpret_cast<const Extent *>(ctx->hbuf + 16), eb);
+        if (sort)
+            for (int c = 0; c < 3; ++c) { out.ext.lo[c] = ctx->hbuf[8 + c]; out.ext.hi[c] = ctx->hbuf[11 + c]; }
+    }
     if (!(out.wsum > 0.0)) {
         release_layout(ctx, &out);
         return set_error(ctx, SSD_EINVAL, "quadrature weights must have a positive sum");

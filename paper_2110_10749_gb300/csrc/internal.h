@@ -203,8 +203,7 @@ struct PairCall {
 };
 int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s);
 int pair_occupancy(ssd_ctx *ctx);
-// reduces the extent of points [beg, end) of SoA arrays over `blocks` blocks, one partial each (ctx.cu)
-constexpr int kExtentBlocks = 32;
+constexpr int kExtentBlocks = 32;   // partial extents of a layout, at most (ctx.cu)
 size_t fx_geo_bytes(int nsurf);
 
 // ------------------------------------------------------------ batched layout
