@@ -104,6 +104,7 @@ struct ssd_ctx {
     int device = 0;
     int num_sms = 0;
     int occ32 = 1, occ64 = 1;  // resident CTAs per SM of the pair kernels
+    int occ32t = 1;            // of the generic kernel in FP32 (transposes)
     int waves32 = 12;          // FP32C grid: about this many waves of resident CTAs (tuned)
     int lpt = 1;               // pair grids in near-first order on prepared layouts
     int sym = 1;               // layer operators (both precisions): far block pairs once for both directions

@@ -1743,14 +1743,17 @@ cudaError_t launch_sym64(const Layout &L, const d4 *d0, double *acc, FxArgs *fx,
 }
 
 int pair_occupancy(ssd_ctx *ctx) {
-    int o32 = 0, o64 = 0;
+    int o32 = 0, o64 = 0, o32t = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o32, pair32_kernel<OP_SSLDL>, kTPB32, 0);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o64, pair_kernel<double, OP_SSLDL, kTPB64, kTPT64>,
                                                           kTPB64, 0);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o32t, pair_kernel<float, OP_SDLT, kTPB64, kTPT64>, kTPB64, 0);
     if (e != cudaSuccess) return cuda_check(ctx, e, "occupancy query");
     ctx->occ32 = o32 > 0 ? o32 : 1;
     ctx->occ64 = o64 > 0 ? o64 : 1;
+    ctx->occ32t = o32t > 0 ? o32t : 1;
     return fx_init(ctx);
 }
 
@@ -1848,7 +1851,9 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     // splits: enough CTAs for several waves of resident CTAs, so that the
     // uneven cost of near and far target tiles evens out (FP32C: tuned on the
     // h = 1/32 sphere, where it reaches one 128-source tile per CTA)
-    const int occ = packed32 ? ctx->occ32 : ctx->occ64;
+    // (FP32C transposes by their own kernel: Laplace double layer at N = 17070 377 us, 418
+    // with a grid for the resident CTAs of the kernel in double)
+    const int occ = packed32 ? ctx->occ32 : (f32 ? ctx->occ32t : ctx->occ64);
     int64_t want = (int64_t)ctx->num_sms * occ * (packed32 ? ctx->waves32 : ctx->waves64);
     int64_t nsplit = (want + ntiles_t - 1) / ntiles_t;
     if (nsplit < 1) nsplit = 1;
