@@ -2,6 +2,7 @@
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <algorithm>
 #include <cub/device/device_radix_sort.cuh>
@@ -267,8 +268,8 @@ __device__ void wsum_block(const double *w, int64_t n, double *red, double *out)
 
 // Extent (see internal.h) of points [off[y], off[y + 1]) of surface y =
 // blockIdx.y (off NULL: all n points), one partial per block x.  With wsum, block 0 of
-// one more sums the weights beside them (a launch of its own made the layout of 1062
-// points take 7 us longer, with one block for the box).  BOX: with the box of the points,
+// one more sums the weights beside them, to wsum[y] (a launch of its own made the layout
+// of 1062 points take 7 us longer, with one block for the box).  BOX: with the box of the points,
 // six double-precision minima a point; prepared sets have it already.  The magnitudes
 // are compared as integers, which order like the nonnegative doubles they are the
 // bits of, with infinities and NaN above all finite ones.
@@ -280,11 +281,11 @@ __global__ void extent_kernel(const double *xyz, const double *nrm, const double
     __shared__ double red[BOX ? 6 : 1][256];
     __shared__ unsigned long long top[2][8];
     const int64_t nb = (int64_t)gridDim.x - (wsum ? 1 : 0), blk = (int64_t)blockIdx.x - (wsum ? 1 : 0);
+    const int64_t beg = off ? off[blockIdx.y] : 0, end = off ? off[blockIdx.y + 1] : n;
     if (blk < 0) {
-        wsum_block(w, n, red[0], wsum);
+        wsum_block(w + beg, end - beg, red[0], wsum + blockIdx.y);
         return;
     }
-    const int64_t beg = off ? off[blockIdx.y] : 0, end = off ? off[blockIdx.y + 1] : n;
     double v[6] = {1e308, 1e308, 1e308, 1e308, 1e308, 1e308};   // lo, -hi
     unsigned long long mx = 0, mm = 0;                          // largest |x|, |w n|
     auto bits = [](double a) { return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull; };
@@ -412,21 +413,6 @@ __global__ void batch_chunk_box_kernel(Layout L) {
     L.cbox[2 * c + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
 }
 
-// weight sum per surface, fixed order (one block per surface)
-__global__ void batch_wsum_kernel(const double *w, const int64_t *off, double *out) {
-    __shared__ double red[256];
-    const int s = blockIdx.x;
-    double acc = 0.0;
-    for (int64_t i = off[s] + threadIdx.x; i < off[s + 1]; i += blockDim.x) acc += w[i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[s] = red[0];
-}
-
 __global__ void batch_esurf_kernel(const int64_t *off, int32_t nsurf, int64_t n, int32_t *esurf) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -481,9 +467,8 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
     const size_t o_perm = carve(sizeof(int32_t) * np), o_p32 = carve(sizeof(float4) * np),
                  o_w32 = carve(sizeof(float4) * np), o_p64 = carve(sizeof(d4) * np),
                  o_w64 = carve(sizeof(d4) * np), o_cb = carve(sizeof(float4) * 2 * (np / kChunk)),
-                 o_es = carve(sizeof(int32_t) * n), o_ws = carve(sizeof(double) * ns),
-                 o_sc = carve(sizeof(double) * ns), o_meta = carve(sizeof(int64_t) * (4 * ns + 1)),
-                 o_ex = carve(sizeof(Extent) * ns), o_geo = carve(fx_geo_bytes(ns));
+                 o_es = carve(sizeof(int32_t) * n), o_ws = carve((sizeof(double) + sizeof(Extent)) * ns),
+                 o_meta = carve(sizeof(int64_t) * (4 * ns + 1) + sizeof(double) * ns);
     void *blk = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &blk));
     char *bp = static_cast<char *>(blk);
@@ -498,20 +483,18 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
     out.L.cbox = reinterpret_cast<float4 *>(bp + o_cb);
     out.elem_surf = reinterpret_cast<int32_t *>(bp + o_es);
     out.d_wsum = reinterpret_cast<double *>(bp + o_ws);
-    out.d_selfc = reinterpret_cast<double *>(bp + o_sc);
     int64_t *dmeta = reinterpret_cast<int64_t *>(bp + o_meta);   // off[ns+1], cnt[ns], poff[ns]
-    Extent *dext = reinterpret_cast<Extent *>(bp + o_ex);
-    out.fx_geo = bp + o_geo;
-    std::vector<int64_t> hmeta(4 * ns + 1, 0);
+    out.d_selfc = reinterpret_cast<double *>(dmeta + 4 * ns + 1);
+    Extent *dext = reinterpret_cast<Extent *>(out.d_wsum + ns);   // behind the weight sums: one host read
+    std::vector<int64_t> hmeta(5 * ns + 1, 0);
     for (int k = 0; k <= ns; ++k) hmeta[k] = b->offsets[k];
     for (int k = 0; k < ns; ++k) { hmeta[ns + 1 + k] = out.n[k]; hmeta[2 * ns + 1 + k] = out.poff[k]; }
-    std::vector<double> selfc(ns);
-    for (int k = 0; k < ns; ++k) selfc[k] = 16.0 / (3.0 * sqrt(M_PI) * out.delta[k]);
+    for (int k = 0; k < ns; ++k) {
+        const double selfc = 16.0 / (3.0 * sqrt(M_PI) * out.delta[k]);
+        memcpy(&hmeta[4 * ns + 1 + k], &selfc, sizeof(selfc));
+    }
     int st = cuda_check(ctx, cudaMemcpyAsync(dmeta, hmeta.data(), sizeof(int64_t) * hmeta.size(),
                                              cudaMemcpyHostToDevice, s), "batch meta copy");
-    if (st == SSD_OK)
-        st = cuda_check(ctx, cudaMemcpyAsync(out.d_selfc, selfc.data(), sizeof(double) * ns,
-                                             cudaMemcpyHostToDevice, s), "batch self copy");
     // sort by (surface, Morton)
     void *tmp = nullptr;
     if (st == SSD_OK) {
@@ -550,24 +533,25 @@ int batch_layout_build(ssd_ctx *ctx, const ssd_batch *b, BatchLayout *B, cudaStr
                 fa.sorted = i1;
                 batch_fill_kernel<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(fa, out.L);
                 batch_chunk_box_kernel<<<(unsigned)((np / kChunk + 127) / 128), 128, 0, s>>>(out.L);
-                batch_wsum_kernel<<<ns, 256, 0, s>>>(b->w, dmeta, out.d_wsum);
-                for (int k = 0; k < ns; k += 65535)   // grid.y limit
-                    extent_kernel<true><<<dim3(1, (unsigned)(ns - k < 65535 ? ns - k : 65535)), 256, 0, s>>>(
-                        b->xyz, b->nrm, b->w, n, dmeta + k, dext + k, nullptr);
-                ctx->launches += 4;
+                ctx->launches += 2;
+                for (int k = 0; k < ns; k += 65535) {   // grid.y limit
+                    extent_kernel<true><<<dim3(2, (unsigned)(ns - k < 65535 ? ns - k : 65535)), 256, 0, s>>>(
+                        b->xyz, b->nrm, b->w, n, dmeta + k, dext + k, out.d_wsum + k);
+                    ctx->launches++;
+                }
                 st = launch_check(ctx, "batch fill");
             }
         }
     }
     out.wsum.resize(ns);
     out.ext.resize(ns);
+    std::vector<char> sums((sizeof(double) + sizeof(Extent)) * ns);
     if (st == SSD_OK)
-        st = cuda_check(ctx, cudaMemcpyAsync(out.ext.data(), dext, sizeof(Extent) * ns, cudaMemcpyDeviceToHost, s),
-                        "extent copy");
-    if (st == SSD_OK)
-        st = cuda_check(ctx, cudaMemcpyAsync(out.wsum.data(), out.d_wsum, sizeof(double) * ns,
-                                             cudaMemcpyDeviceToHost, s), "wsum copy");
+        st = cuda_check(ctx, cudaMemcpyAsync(sums.data(), out.d_wsum, sums.size(), cudaMemcpyDeviceToHost, s),
+                        "wsum copy");
     if (st == SSD_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "batch layout sync");
+    memcpy(out.wsum.data(), sums.data(), sizeof(double) * ns);
+    memcpy(out.ext.data(), sums.data() + sizeof(double) * ns, sizeof(Extent) * ns);
     if (tmp) dev_free(ctx, tmp);
     if (st == SSD_OK) {
         for (int k = 0; k < ns; ++k)

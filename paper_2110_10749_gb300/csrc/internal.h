@@ -205,7 +205,6 @@ struct PairCall {
 int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s);
 int pair_occupancy(ssd_ctx *ctx);
 constexpr int kExtentBlocks = 32;   // partial extents of a layout, at most (ctx.cu)
-size_t fx_geo_bytes(int nsurf);
 
 // ------------------------------------------------------------ batched layout
 // Many surfaces concatenated (caller order: surface s owns caller indices
@@ -217,7 +216,7 @@ struct BatchLayout {
     std::vector<int64_t> off, n, poff, n_pad;   // host copies
     std::vector<double> delta, wsum;
     std::vector<Extent> ext;
-    void *fx_geo = nullptr;   // per-surface constants of the fixed-point kernel (in block)
+    void *fx_geo = nullptr;   // per-surface constants of the fixed-point kernel (beside the FP64 items)
     void *fx_pos = nullptr;   // grid positions and chunk boxes
     int fx_noct = 0;          // octaves of the kernel tables the surfaces need; 0: some surface is out of range
     Layout L;                 // concatenated padded arrays; L.perm maps to caller indices

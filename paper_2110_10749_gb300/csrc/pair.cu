@@ -1757,8 +1757,6 @@ int pair_occupancy(ssd_ctx *ctx) {
     return fx_init(ctx);
 }
 
-size_t fx_geo_bytes(int nsurf) { return sizeof(FxGeo) * nsurf; }
-
 // Grid of the fixed-point kernel.  Every pair costs the same, so it only has to
 // fill the SMs evenly.  Small sets: at most one round of two CTAs per SM, the
 // grouped form where its finer items leave less to the fullest CTA (N = 1062:
@@ -2108,8 +2106,6 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
         if (!fx_geo(B->ext[k], B->delta[k], &geos[k], &noct)) { B->fx_noct = 0; break; }
         B->fx_noct = noct > B->fx_noct ? noct : B->fx_noct;
     }
-    SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(B->fx_geo, geos.data(), sizeof(FxGeo) * ns, cudaMemcpyHostToDevice, s),
-                       "surface constants copy"));
     for (int pr = 0; pr < 2; ++pr) {   // 0: FP32C, 1: FP64
         const bool fx = pr == 1 && B->fx_noct > 0;
         const int64_t unit = fx ? kChunk : kTile;   // sources come in multiples of this
@@ -2153,7 +2149,7 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
         size_t off = 0;
         auto carve = [&](size_t bb) { size_t o = off; off += (bb + 255) & ~size_t(255); return o; };
         const size_t o_it = carve(sizeof(BItem) * items.size()), o_sf = carve(sizeof(BSurf) * ns),
-                     o_c = carve(csz * ns);
+                     o_c = carve(csz * ns), o_geo = fx ? carve(sizeof(FxGeo) * ns) : 0;
         void *blk = nullptr;
         SSD_TRY(dev_alloc(ctx, off, &blk));
         char *bp = static_cast<char *>(blk);
@@ -2162,22 +2158,26 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
         B->consts[pr] = bp + o_c;
         B->nitems[pr] = (int64_t)items.size();
         B->ptotal[pr] = pb;
-        std::vector<char> cbuf(csz * ns);
+        // one copy of everything; the host buffer stays until it has been read
+        std::unique_ptr<char[]> host(new char[off]);
+        struct Wait { cudaStream_t s; bool on; ~Wait() { if (on) cudaStreamSynchronize(s); } } wait{s, false};
+        memcpy(host.get() + o_it, items.data(), sizeof(BItem) * items.size());
+        memcpy(host.get() + o_sf, surfs.data(), sizeof(BSurf) * ns);
         for (int k = 0; k < ns; ++k) {
             if (pr == 0) {
                 const Consts<float> c = make_consts<float>(B->delta[k], kRhoFar32);
-                memcpy(cbuf.data() + k * csz, &c, csz);
+                memcpy(host.get() + o_c + k * csz, &c, csz);
             } else {
                 const Consts<double> c = make_consts<double>(B->delta[k], kRhoFar64);
-                memcpy(cbuf.data() + k * csz, &c, csz);
+                memcpy(host.get() + o_c + k * csz, &c, csz);
             }
         }
-        SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(bp + o_it, items.data(), sizeof(BItem) * items.size(),
-                                                cudaMemcpyHostToDevice, s), "items copy"));
-        SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(bp + o_sf, surfs.data(), sizeof(BSurf) * ns,
-                                                cudaMemcpyHostToDevice, s), "surfs copy"));
-        SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(bp + o_c, cbuf.data(), csz * ns, cudaMemcpyHostToDevice, s),
-                           "consts copy"));
+        if (fx) {
+            memcpy(host.get() + o_geo, geos.data(), sizeof(FxGeo) * ns);
+            B->fx_geo = bp + o_geo;
+        }
+        wait.on = true;
+        SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(bp, host.get(), off, cudaMemcpyHostToDevice, s), "items copy"));
         if (fx) {
             SSD_TRY(dev_alloc(ctx, sizeof(l4) * B->n_pad_total + sizeof(int4) * 2 * (B->n_pad_total / kChunk),
                               &B->fx_pos));
@@ -2188,8 +2188,6 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
             ctx->launches++;
             SSD_TRY(launch_check(ctx, "grid positions"));
         }
-        // the host vectors go out of scope: wait for the copies
-        SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "items sync"));
         if (pr == 0 && ctx->lpt && !items.empty()) {
             // FP32C items in decreasing order of near work, so that cheap far
             // items fill the last wave; each item keeps its own partial slot
@@ -2206,6 +2204,7 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
             SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(hk.data(), kd, sizeof(int32_t) * ni, cudaMemcpyDeviceToHost, s),
                                "key copy"));
             SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "key sync"));
+            wait.on = false;
             int32_t kmax = 0;
             for (int64_t i = 0; i < ni; ++i) kmax = hk[i] > kmax ? hk[i] : kmax;
             std::vector<int64_t> start(kmax + 2, 0);
@@ -2216,6 +2215,9 @@ int pair_batch_items(ssd_ctx *ctx, BatchLayout *B, cudaStream_t s) {
             SSD_TRY(cuda_check(ctx, cudaMemcpyAsync(bp + o_it, sorted.data(), sizeof(BItem) * ni,
                                                     cudaMemcpyHostToDevice, s), "items copy"));
             SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "items sync"));
+        } else {
+            SSD_TRY(cuda_check(ctx, cudaStreamSynchronize(s), "items sync"));
+            wait.on = false;
         }
     }
     return SSD_OK;
