@@ -580,6 +580,12 @@ __global__ void __launch_bounds__(kTPB32, pair32_min_cta(OP)) pair32_kernel(cons
     static_assert(kChunks * kTPT32 <= 32, "one lane per (chunk, patch)");
     const int64_t patch = (tbase + (threadIdx.x & ~31) + (lane % kTPT32) * kTPB32) / kChunk;
     const float4 tlo = a.cbox[2 * patch], thi = a.cbox[2 * patch + 1];
+    // The scalar path's vote comes first, where the boxes allow such close pairs, and is
+    // left out elsewhere: on small sets those chunks are most of the time, and one vote more
+    // before it cost a batch of two sets of 822 points up to 5% (Stokes single layer 78.6
+    // us, 83.2).  The Stokes layers with a double layer vote after the near test, which
+    // serves large sets (Stokes double layer at N = 17070 279.5 us, 280.5).
+    constexpr bool kSerFirst = OP != OP_SDL && OP != OP_SSLDL;
     // a patch of padding is near nothing (its sums are not read; against chunks of
     // padding its pairs would all take the scalar path: Stokes double layer at N = 1062
     // 94 us a call, 67 without them)
@@ -602,17 +608,22 @@ __global__ void __launch_bounds__(kTPB32, pair32_min_cta(OP)) pair32_kernel(cons
         float2 part[NP][3];
 #pragma unroll
         for (int k = 0; k < NP; ++k) part[k][0] = part[k][1] = part[k][2] = make_float2(0.f, 0.f);
-        uint32_t nearmask;
+        uint32_t nearmask, sermask = 0;
         {
             const int64_t cidx = tile / kChunk + (lane / kTPT32) % kChunks;
             const float4 clo = a.cbox[2 * cidx], chi = a.cbox[2 * cidx + 1];
             const float gx = fmaxf(0.f, fmaxf(clo.x - thi.x, tlo.x - chi.x));
             const float gy = fmaxf(0.f, fmaxf(clo.y - thi.y, tlo.y - chi.y));
             const float gz = fmaxf(0.f, fmaxf(clo.z - thi.z, tlo.z - chi.z));
-            nearmask = __ballot_sync(0xffffffffu, real && !(gx * gx + gy * gy + gz * gz >= c.rfar2));
+            const float g2 = gx * gx + gy * gy + gz * gz;
+            nearmask = __ballot_sync(0xffffffffu, real && !(g2 >= c.rfar2));
+            if constexpr (kSerFirst)   // 1%: the box gap and r^2 round differently
+                sermask = __ballot_sync(0xffffffffu, real && !(OP == OP_LSL ? g2 >= 1.01f * c.rvec2
+                                                                            : g2 * c.inv_d2 >= 1.01f * c.tser));
         }
         for (int ch = 0; ch < kChunks; ++ch) {
             const uint32_t bits = (nearmask >> (ch * kTPT32)) & ((1u << kTPT32) - 1u);   // near patches
+            const bool ser = (sermask >> (ch * kTPT32)) & ((1u << kTPT32) - 1u);
             const int j0 = ch * kChunk;
             if (bits == 0) {
 #pragma unroll 4
@@ -646,14 +657,14 @@ __global__ void __launch_bounds__(kTPB32, pair32_min_cta(OP)) pair32_kernel(cons
                         m[k] = fminf(R2[k].x, R2[k].y);
                         mall = fminf(mall, m[k]);
                     }
-                    if (!__any_sync(0xffffffffu, mall < c.rfar2)) {
+                    if (!kSerFirst && !__any_sync(0xffffffffu, mall < c.rfar2)) {
 #pragma unroll
                         for (int k = 0; k < NP; ++k)
                             pair2<OP, false>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
                         continue;
                     }
                     const bool serv = OP == OP_LSL ? mall < c.rvec2 : mall * c.inv_d2 < c.tser;
-                    if (__any_sync(0xffffffffu, serv)) {
+                    if ((ser || !kSerFirst) && __any_sync(0xffffffffu, serv)) {
                         // a target of the warp is within 0.5 delta of this source
                         // (the self pair or a close neighbour): scalar path with
                         // the Taylor branch
@@ -680,6 +691,10 @@ __global__ void __launch_bounds__(kTPB32, pair32_min_cta(OP)) pair32_kernel(cons
                                 }
                             }
                         }
+                    } else if (kSerFirst && !__any_sync(0xffffffffu, mall < c.rfar2)) {
+#pragma unroll
+                        for (int k = 0; k < NP; ++k)
+                            pair2<OP, false>(DX[k], DY[k], DZ[k], R2[k], dt[k], sw, s0, s1, c, part[k]);
                     } else {
                         // smoothed terms only for the target pairs that need them (they
                         // equal the bare ones bit for bit beyond rho_far)
