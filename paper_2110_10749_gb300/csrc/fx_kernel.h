@@ -25,7 +25,14 @@
 // SDLT 4.4, SSLDL 6.
 //
 // Densities are scaled by their largest magnitude, which the packing kernel
-// leaves per block; the kernel reduces those at its start.  When that scale
+// leaves per block; the kernel reduces those at its start.  The double layers see
+// differences of densities only.  Where a constant can cost digits (more than one
+// component, or a single layer beside it) the packing also leaves the densities less the
+// surface's first one, and where these are smaller by 2^5 or more the kernel takes them:
+// the scale is then that of the variation, and what a component keeps of its constant
+// subtracts exactly (Sterbenz).  (Errors with a constant 1 and a variation of 1e-8 in
+// another component 2e-10 without, 4e-16 with it; beside a constant in the fused
+// layers the single layer keeps its digits.)  When the scale
 // does not exist (a NaN, an infinity, or a magnitude outside 2^+-400) the CTA
 // evaluates its pairs in double precision instead, as the generic kernel
 // does, so non-finite densities give the same results as there.  Point sets
@@ -38,7 +45,7 @@ constexpr int kFxUnit = 8;     // and the granularity of their chunks of sources
 struct FxArgs {
     const l4 *X;
     const int4 *cbox;            // per 32-point chunk: (lo, hi) of X >> 32
-    const unsigned long long *bmax;   // [rhs][pack block][2]: bits of the largest |d0|, |d1|
+    const unsigned long long *bmax;   // [rhs][pack block][2], see fx_pack
     int64_t nblk;                // pack blocks per right-hand side
     const FxI4 *tab;
     int noct;
@@ -51,18 +58,52 @@ struct FxArgs {
 // what the packing kernels leave for it: the densities' block maxima
 struct FxPack {
     unsigned long long *bmax = nullptr;   // NULL: not wanted
-    int two = 0;                          // LSLDL: .y of the first record is the second density
+    int two = 0;                 // LSLDL: .y of the first record is the second density
+    d4 *rest = nullptr;          // double layers: first records less the surface's first one
+    const int32_t *elem_surf = nullptr;   // batched: surface of a caller index, and the surfaces
+    const BSurf *surfs = nullptr;
 };
 
-// block maxima (every thread of a 256-thread block calls this)
-__device__ __forceinline__ void fx_pack(const FxPack &P, const d4 &r0, const d4 &r1, int rhs, int64_t nblk) {
+// magnitude of a double for comparisons and its exponent: the high word without the
+// sign, 0 for zero only
+__device__ __forceinline__ uint32_t fx_mag(double v) {
+    return ((uint32_t)__double2hiint(v) & 0x7fffffffu) | (__double2loint(v) != 0 ? 1u : 0u);
+}
+__device__ __forceinline__ uint32_t fx_mag(double x, double y, double z) { return max(fx_mag(x), max(fx_mag(y), fx_mag(z))); }
+
+// a record less the first point's, s v; both are rounded records (no contraction)
+__device__ __forceinline__ double fx_rest(double r, double s, double v) { return __dsub_rn(r, __dmul_rn(s, v)); }
+
+// Block maxima (every thread of a 256-thread block calls this), 16 bytes per block: the
+// bits of the largest |d0| and |d1|, or, with P.rest, a uint4 of fx_mag of the first
+// density, of the second one and of the first one's rest.  rest: record r0 less the
+// surface's first one (zero for padding); it goes to P.rest[i].
+__device__ __forceinline__ void fx_pack(const FxPack &P, const d4 &r0, const d4 &r1, const d4 &rest, int64_t i, int rhs,
+                                        int64_t nblk) {
     __shared__ unsigned long long smax[2][8];
+    __shared__ uint32_t smag[3][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (P.rest) {
+        P.rest[i] = rest;
+        const uint32_t m[3] = {P.two ? fx_mag(r0.x) : fx_mag(r0.x, r0.y, r0.z), P.two ? fx_mag(r0.y) : fx_mag(r1.x, r1.y, r1.z),
+                               P.two ? fx_mag(rest.x) : fx_mag(rest.x, rest.y, rest.z)};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t v = __reduce_max_sync(0xffffffffu, m[k]);
+            if (lane == 0) smag[k][warp] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t t[3] = {0u, 0u, 0u};
+            for (int w = 0; w < 8; ++w)
+                for (int k = 0; k < 3; ++k) t[k] = max(t[k], smag[k][w]);
+            reinterpret_cast<uint4 *>(P.bmax)[(int64_t)rhs * nblk + blockIdx.x] = make_uint4(t[0], t[1], t[2], 0u);
+        }
+        return;
+    }
     const unsigned long long am = 0x7fffffffffffffffull;
     auto bits = [&](double v) { return (unsigned long long)__double_as_longlong(v) & am; };
-    unsigned long long m0 = bits(r0.x), m1 = 0;
-    if (P.two) m1 = bits(r0.y);
-    else { m0 = max(m0, max(bits(r0.y), bits(r0.z))); m1 = max(bits(r1.x), max(bits(r1.y), bits(r1.z))); }
+    unsigned long long m0 = max(bits(r0.x), max(bits(r0.y), bits(r0.z))), m1 = max(bits(r1.x), max(bits(r1.y), bits(r1.z)));
     for (int off = 16; off > 0; off >>= 1) {
         m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, off));
         m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
@@ -161,7 +202,7 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
     __shared__ int4 s_mh[M ? kTile : 1], s_ml[M ? kTile : 1];
     __shared__ int4 s_uh[VU ? kTile : 1], s_ul[VU ? kTile : 1];
     __shared__ int4 s_fh[VF ? kTile : 1], s_fl[VF ? kTile : 1];
-    __shared__ unsigned long long s_max[2][kFxTPB / 32];
+    __shared__ __align__(16) unsigned long long s_max[2][kFxTPB / 32];   // or a uint4 per warp
     __shared__ int64_t s_acc[GROUPS > 1 ? 2 * NC : 1][GROUPS > 1 ? kFxTPB : 1];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -227,7 +268,44 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
     pdl_release();
     if constexpr (kEarly) Yd = d0[i];
     // largest densities of this surface and right-hand side
-    {
+    int ee[2];
+    bool bad = false;
+    if constexpr (T::rest) {
+        uint4 *s_mag = reinterpret_cast<uint4 *>(s_max);
+        uint4 m = make_uint4(0u, 0u, 0u, 0u);
+        const uint4 *bm = reinterpret_cast<const uint4 *>(a.bmax) + (a.geos ? blockIdx.y : 0) * a.nblk;
+        for (int64_t b = b0 + threadIdx.x; b < b1; b += kFxTPB) {
+            const uint4 v = bm[b];
+            m.x = max(m.x, v.x);
+            m.y = max(m.y, v.y);
+            m.z = max(m.z, v.z);
+        }
+        m.x = __reduce_max_sync(0xffffffffu, m.x);
+        m.y = __reduce_max_sync(0xffffffffu, m.y);
+        m.z = __reduce_max_sync(0xffffffffu, m.z);
+        if (lane == 0) s_mag[warp] = m;
+        __syncthreads();
+        m = s_mag[0];
+#pragma unroll
+        for (int w = 1; w < kFxTPB / 32; ++w) {
+            const uint4 v = s_mag[w];
+            m.x = max(m.x, v.x);
+            m.y = max(m.y, v.y);
+            m.z = max(m.z, v.z);
+        }
+        // the rest where it is smaller by 2^5 (not below the range)
+        if (m.x < 0x7ff00000u && m.z + (5u << 20) <= m.x && (m.z == 0u || m.z >= (uint32_t)(1022 - kFxExpMax) << 20)) {
+            m.x = m.z;
+            d0 += (a.geos ? (int64_t)gridDim.y : 1) * a.k.n_pad;
+            if constexpr (kEarly) Yd = d0[i];
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t t = k ? m.y : m.x;
+            ee[k] = t == 0u ? -kFxExpMax : (int)(t >> 20) - 1022;   // all zero: any scale
+            bad |= t != 0u && (ee[k] > kFxExpMax || ee[k] < -kFxExpMax);
+        }
+    } else {
         unsigned long long m0 = 0, m1 = 0;
         const unsigned long long *bm = a.bmax + (a.geos ? blockIdx.y : 0) * a.nblk * 2;
         for (int64_t b = b0 + threadIdx.x; b < b1; b += kFxTPB) { m0 = max(m0, bm[2 * b]); m1 = max(m1, bm[2 * b + 1]); }
@@ -236,18 +314,16 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
         }
         if (lane == 0) { s_max[0][warp] = m0; s_max[1][warp] = m1; }
-    }
-    __syncthreads();
-    int ee[2];
-    bool bad = false;
+        __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        unsigned long long m = 0;
+        for (int k = 0; k < 2; ++k) {
+            unsigned long long m = 0;
 #pragma unroll
-        for (int w = 0; w < kFxTPB / 32; ++w) m = max(m, s_max[k][w]);
-        const int ex = (int)(m >> 52);
-        ee[k] = m == 0 ? -kFxExpMax : ex - 1022;            // all zero: any scale
-        bad |= m != 0 && (ee[k] > kFxExpMax || ee[k] < -kFxExpMax);
+            for (int w = 0; w < kFxTPB / 32; ++w) m = max(m, s_max[k][w]);
+            const int ex = (int)(m >> 52);
+            ee[k] = m == 0 ? -kFxExpMax : ex - 1022;            // all zero: any scale
+            bad |= m != 0 && (ee[k] > kFxExpMax || ee[k] < -kFxExpMax);
+        }
     }
     double sum[3] = {0.0, 0.0, 0.0}, low[3] = {0.0, 0.0, 0.0};
     if (bad) {

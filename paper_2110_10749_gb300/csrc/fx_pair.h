@@ -23,6 +23,7 @@ template <int OP> struct FxOp {
     static constexpr bool sl = OP == OP_LSL || OP == OP_SSL || OP == OP_SSLDL || OP == OP_LSLDL;
     static constexpr bool tr = OP == OP_LDLT || OP == OP_SDLT;
     static constexpr bool fused = OP == OP_SSLDL || OP == OP_LSLDL;
+    static constexpr bool rest = fused || OP == OP_SDL;   // densities less the first one where those are smaller
     static constexpr int k1 = sl ? 0 : -1;                                   // index among the staged tables
     static constexpr int k3 = vec && sl ? 1 : -1;
     static constexpr int kd = dl ? (fused ? (vec ? 2 : 1) : 0) : -1;

@@ -1069,9 +1069,18 @@ __global__ void pack_kernel(const PackArgs a) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double wd = 0.0;
     V4 r0 = {R(0), R(0), R(0), R(0)}, r1 = {R(0), R(0), R(0), R(0)};
+    // the first point's density, requested beside the thread's own
+    double c[3] = {0.0, 0.0, 0.0};
+    if (sizeof(R) == 8 && a.fx.rest) {
+        const int32_t f = a.perm[0];
+        c[0] = a.d0[f];
+        if (a.op != OP_LSLDL) { c[1] = a.d0[a.n + f]; c[2] = a.d0[2 * a.n + f]; }
+    }
+    bool real = false;
     if (i < a.n_pad) {
         const int32_t o = a.perm[i];
-        if (o >= 0) {
+        real = o >= 0;
+        if (real) {
             const double w = a.no_weight ? 1.0 : a.pos64[i].w;
             switch (a.op) {
                 case OP_LSL: r0.x = R(a.s0 * w * a.d0[o]); break;
@@ -1113,7 +1122,15 @@ __global__ void pack_kernel(const PackArgs a) {
         if (a.out1) reinterpret_cast<V4 *>(a.out1)[i] = r1;
     }
     if constexpr (sizeof(R) == 8) {   // n_pad is a multiple of 512: whole blocks
-        if (a.fx.bmax) fx_pack(a.fx, r0, r1, 0, gridDim.x);
+        if (a.fx.bmax) {
+            d4 rest = {0.0, 0.0, 0.0, 0.0};
+            if (a.fx.rest && real) {
+                rest = r0;
+                rest.x = fx_rest(r0.x, a.s0, c[0]);
+                if (a.op != OP_LSLDL) { rest.y = fx_rest(r0.y, a.s0, c[1]); rest.z = fx_rest(r0.z, a.s0, c[2]); }
+            }
+            fx_pack(a.fx, r0, r1, rest, i, 0, gridDim.x);
+        }
     }
     if (a.wdot_part) {
         red[threadIdx.x] = wd;
@@ -1393,7 +1410,17 @@ __global__ void bpack_kernel(const BPackArgs a) {
         if (a.out1) reinterpret_cast<V4 *>(a.out1)[(int64_t)r * a.n_pad + i] = r1;
     }
     if constexpr (sizeof(R) == 8) {
-        if (a.fx.bmax) fx_pack(a.fx, r0, r1, r, gridDim.x);
+        if (a.fx.bmax) {
+            d4 rest = {0.0, 0.0, 0.0, 0.0};
+            const int32_t o = a.perm[i];
+            if (a.fx.rest && o >= 0) {
+                const int32_t f = a.perm[a.fx.surfs[a.fx.elem_surf[o]].poff];
+                rest = r0;
+                rest.x = fx_rest(r0.x, a.s0, d0[f]);
+                if (a.nc0 == 3) { rest.y = fx_rest(r0.y, a.s0, d0[n + f]); rest.z = fx_rest(r0.z, a.s0, d0[2 * n + f]); }
+            }
+            fx_pack(a.fx, r0, r1, rest, (int64_t)r * a.n_pad + i, r, gridDim.x);
+        }
     }
     if (a.want_wdot) {
         red[threadIdx.x] = wd;
@@ -1885,7 +1912,9 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     const int pack_blocks = (int)((n_pad + 255) / 256);
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
-    const size_t o_d0 = carve(rec * n_pad);
+    // (FP64, FxOp::rest: the records less the first one behind them)
+    const bool rest = use_fx && (op == OP_SDL || op == OP_SSLDL || op == OP_LSLDL);
+    const size_t o_d0 = carve(rec * n_pad * (rest ? 2 : 1));
     const size_t o_d1 = two_rec ? carve(rec * n_pad) : 0;
     const size_t o_part = carve(rsz * nslot * nc * nsplit * n_pad);
     const size_t o_wdot = carve(sizeof(double) * pack_blocks);
@@ -1906,7 +1935,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
         use_sym = L.sym[f32 ? 0 : 1].use;
     }
     const size_t o_acc = use_sym ? carve(sizeof(double) * nc * n_pad) : 0;
-    const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks) : 0;
+    const size_t o_fxm = use_fx ? carve(sizeof(uint4) * pack_blocks) : 0;
     const bool fx_kept = use_fx && fx_keeps(ctx, L, s);
     const size_t o_fxx = use_fx ? carve(fx_position_bytes(L)) : 0;   // always: a captured call cannot grow the pool
     void *ws = nullptr;
@@ -1950,6 +1979,7 @@ int pair_apply(ssd_ctx *ctx, const Layout &L, const PairCall &pc, cudaStream_t s
     if (use_fx) {
         SSD_TRY(fx_positions(ctx, L, pc.delta, geo, fx_kept ? nullptr : base + o_fxx, &fa.X, &fa.cbox, s));
         pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
+        if (rest) pa.fx.rest = reinterpret_cast<d4 *>(base + o_d0) + n_pad;
         pa.fx.two = op == OP_LSLDL ? 1 : 0;
         fa.bmax = pa.fx.bmax;
         fa.nblk = pack_blocks; fa.tab = static_cast<const FxI4 *>(ctx->fx_tab); fa.noct = noct;
@@ -2254,13 +2284,15 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
     const int64_t part_stride = (int64_t)nc * nslot * B.ptotal[pr];
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
-    const size_t o_d0 = carve(rec * n_pad * nrhs);
+    const bool use_fx = !f32 && B.fx_noct > 0;
+    // (FP64, FxOp::rest: the records less each surface's first one behind them)
+    const bool rest = use_fx && (op == OP_SDL || op == OP_SSLDL || op == OP_LSLDL);
+    const size_t o_d0 = carve(rec * n_pad * nrhs * (rest ? 2 : 1));
     const size_t o_d1 = two_rec ? carve(rec * n_pad * nrhs) : 0;
     const size_t o_part = carve(rsz * part_stride * nrhs);
     const size_t o_wdot = carve(sizeof(double) * pack_blocks * nrhs);
     const size_t o_r1 = carve(sizeof(double) * B.nsurf * nrhs);
-    const bool use_fx = !f32 && B.fx_noct > 0;
-    const size_t o_fxm = use_fx ? carve(sizeof(unsigned long long) * 2 * pack_blocks * nrhs) : 0;
+    const size_t o_fxm = use_fx ? carve(sizeof(uint4) * pack_blocks * nrhs) : 0;
     void *ws = nullptr;
     SSD_TRY(dev_alloc(ctx, off, &ws));
     struct Release { ssd_ctx *c; void *p; ~Release() { dev_free(c, p); } } release{ctx, ws};
@@ -2297,6 +2329,9 @@ int pair_apply_batch(ssd_ctx *ctx, const BatchLayout &B, const BatchCall &bc, cu
     FxArgs fa{};
     if (use_fx) {
         pa.fx.bmax = reinterpret_cast<unsigned long long *>(base + o_fxm);
+        if (rest) pa.fx.rest = reinterpret_cast<d4 *>(base + o_d0) + nrhs * n_pad;
+        pa.fx.elem_surf = B.elem_surf;
+        pa.fx.surfs = reinterpret_cast<const BSurf *>(B.surfs[pr]);
         pa.fx.two = op == OP_LSLDL ? 1 : 0;
         fa.X = static_cast<const l4 *>(B.fx_pos);
         fa.cbox = reinterpret_cast<const int4 *>(fa.X + n_pad);
