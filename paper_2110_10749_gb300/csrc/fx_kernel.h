@@ -31,8 +31,8 @@
 // surface's first one, and where these are smaller by 2^5 or more the kernel takes them:
 // the scale is then that of the variation, and what a component keeps of its constant
 // subtracts exactly (Sterbenz).  (Errors with a constant 1 and a variation of 1e-8 in
-// another component 2e-10 without, 4e-16 with it; beside a constant in the fused
-// layers the single layer keeps its digits.)  When the scale
+// another component: 1.4e-10 without, 1e-16 with it; of a single layer of 1e-8 beside a
+// constant double-layer density 3e-12 and 1e-16.)  When the scale
 // does not exist (a NaN, an infinity, or a magnitude outside 2^+-400) the CTA
 // evaluates its pairs in double precision instead, as the generic kernel
 // does, so non-finite densities give the same results as there.  Point sets
@@ -445,8 +445,9 @@ __global__ void __launch_bounds__(kFxTPB, 2) fx_kernel(const FxArgs a) {
             // 4 pairs in flight fill the wide multiplier's latency (Stokes double layer
             // 3.10 clocks per pair and SM against 3.50 unrolled once; the transposed
             // Stokes layer has no registers left beyond 2).  3 resident CTAs of the Laplace
-            // layers with 2 pairs in flight are slower: 2.29 ms against 2.20 at N = 17070.
-            constexpr int kUnroll = OP == OP_SDLT ? 2 : 4;
+            // layers with 2 pairs in flight are slower: 2.29 ms against 2.20 at N = 17070.  The
+            // fused Laplace layers keep their values in registers with 2: 3.52 ms, 3.54 with 4.
+            constexpr int kUnroll = OP == OP_SDLT || OP == OP_LSLDL ? 2 : 4;
 #pragma unroll kUnroll
             for (int j = grp; j < cnt; j += GROUPS) {
                 FxPoint<OP> x;
