@@ -23,7 +23,9 @@
  * - prec selects the arithmetic of the pair sums: SSD_FP64 (double precision:
  *   the pair terms in 62-bit fixed point where the extent of the points is
  *   between 1/16 and 256 delta, in double elsewhere; errors at or below plain
- *   double's) or SSD_FP32C (single precision pair terms, compensated two-float
+ *   double's, relative to the largest value of the set's density, for the
+ *   double layers of its variation where a constant outweighs that, and in
+ *   the fused operators to the larger of the two layers) or SSD_FP32C (single precision pair terms, compensated two-float
  *   accumulation per target, FP64 epilogue).  Krylov and interface
  *   arithmetic is always FP64.
  * - Non-finite scalar arguments, n <= 0, delta <= 0, mu <= 0, kappa <= 0,
@@ -481,7 +483,9 @@ int ssd_hessenberg_eigenvalues(int n, const double *h /* host */, int ldh, doubl
  * the surface: the paper gives no near-surface correction).  Field points
  * targets[3][nt] and outputs are device arrays; nt may be 0.  On prepared
  * points the velocity and the Darcy pressure run in fixed point as the
- * operators do; the Stokes pressure, and unprepared points, in double.
+ * operators do; the Stokes pressure, unprepared points, and calls that
+ * cannot have a workspace (captured ones on a pool without a block of the
+ * size) in double.
  *
  * Darcy pressure inside the body, Green's representation (eq. Greens) with
  * dp/dn = -(mu/kappa) q (Darcy's law, the interface flux q = u . n):

@@ -3,7 +3,8 @@
 // This device issues 32 32x32+64-bit integer multiply-adds per clock and SM
 // against 1.6 double-precision FMAs (measured), so the FP64 operators run
 // their pair terms in 59 to 62-bit fixed point on the integer pipes: more
-// significant bits than a double carries, at a fraction of the cost.  The
+// significant bits than a double carries, at a fraction of the cost.  (The kernel
+// tables are good to 2^-53.7, sigma_4 to 2^-51.9, of a value: fx_table.cu.)  The
 // building blocks here are host and device code:
 //
 //   positions   in units of delta, 2^-ps grid, int64; differences are exact
@@ -42,8 +43,7 @@ constexpr int kFxEBias = 8;                     // bias of the stored exponent
 // delta; below 1/16 all terms are small against the bounds that fix the units
 constexpr double kFxMinExt = 0.0625, kFxMaxExt = 256.0;
 
-// 32 x 32 + 64 bits: one IMAD.WIDE (spelled out: where an operand is known to
-// be nonnegative the compiler otherwise takes the product apart as 64 x 64 bits)
+// 32 x 32 + 64 bits: mad.wide.s32 (a x b in full, plus c), as one instruction
 FX_HD int64_t fx_mw(int a, int b, int64_t c) {
 #ifdef __CUDA_ARCH__
     int64_t d;

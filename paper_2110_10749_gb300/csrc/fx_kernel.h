@@ -6,8 +6,9 @@
 // of them replacing 31 double-precision operations that issue at 1.6 per
 // clock and SM; a smoothed pair costs the same as a bare one, where the
 // double-precision kernel also evaluates erf and exp (33 clocks per pair and
-// SM).  So there is no near/far split here, every tile costs the same, and
-// the grid needs no launch order.
+// SM).  So there is no near/far split within a launch, every tile costs the same,
+// and the grid needs no launch order.  (On a plan the far block pairs are a launch of
+// their own, the FAR form below.)
 //
 // A CTA holds 256 targets, one per thread, and walks its sources 128 at a time
 // in shared memory next to the kernel tables (3 KB per octave of 1 + rho^2 and
@@ -16,11 +17,12 @@
 // their order does not matter); they enter a double accumulator once per tile.
 // Tables are read by lane-dependent index, sources by broadcast.
 // Measured on the h = 1/32 sphere (N = 17070), against the double-precision
-// kernel: Laplace double layer 2.20 ms (18.9), and on small sets, where every
+// kernel: Laplace double layer 2.21 ms (18.9), and on small sets, where every
 // pair is smoothed, with packing and epilogue: Stokes double layer 0.028 ms
 // (0.62) at N = 1062, fused Stokes layers 0.095 ms (1.44) at N = 1742, transposed
 // Stokes double layer 0.334 ms (3.7) at N = 4302; errors against long double at
-// or below the double kernel's.  The wide multiplier is 71% busy (32 a clock and
+// or below the double kernel's, on densities whose values are within a few orders
+// of magnitude (below).  The wide multiplier is 71% busy (32 a clock and
 // SM) on large sets, the ALU that shifts and adds 64%; clocks per pair and SM: LSL 1.6, LDL 2.2, SDL 3.3, SSL 4.0,
 // SDLT 4.4, SSLDL 6.
 //
@@ -32,7 +34,9 @@
 // the scale is then that of the variation, and what a component keeps of its constant
 // subtracts exactly (Sterbenz).  (Errors with a constant 1 and a variation of 1e-8 in
 // another component: 1.4e-10 without, 1e-16 with it; of a single layer of 1e-8 beside a
-// constant double-layer density 3e-12 and 1e-16.)  When the scale
+// constant double-layer density 3e-12 and 1e-16.)  What remains is relative to the
+// largest value: a source 1e12 times the others costs the targets that its kernel
+// vanishes on, as those of one plane do for a double layer, 6e-6 of their sums.  When the scale
 // does not exist (a NaN, an infinity, or a magnitude outside 2^+-400) the CTA
 // evaluates its pairs in double precision instead, as the generic kernel
 // does, so non-finite densities give the same results as there.  Point sets
@@ -179,10 +183,7 @@ __device__ __noinline__ void fx_fallback(const KArgs<double> *ap, const Consts<d
 // plan).  Only the octaves from there on are staged, and the Stokes single
 // layer takes sigma_3 from sigma_1: one table of noct - 6 octaves instead of two
 // of noct.  Stokes single layer at N = 68166: 58.9 ms with the plan against 64.9
-// with every tile on the general kernel; the other layers gain 1-2%.  (The
-// double-precision symmetric kernel that ran the far pairs before left this
-// operator at 164 ms at N = 78106, nearly all of it in that kernel; both directions
-// in fixed point take it to 76 ms.)
+// with every tile on the general kernel; the other layers gain 1-2%.
 constexpr int kFxFarOct = 6;                     // 1 + 8^2 > 2^6
 template <int OP, bool FAR> constexpr int fx_ntab() { return FAR && OP == OP_SSL ? 1 : FxOp<OP>::ntab; }
 

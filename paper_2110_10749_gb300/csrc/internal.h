@@ -49,8 +49,9 @@ struct alignas(16) l4 { int64_t x, y, z, w; };
 // largest |w n| component; fin is 0 when any of it is not finite.
 struct Extent { double lo[3], hi[3], mmax, fin; };
 
-// Plan that evaluates the far block pairs of a layout once for both
-// directions, cached for the last rho_far delta it was built for: near items
+// Plan with the far block pairs of a layout on a kernel of their own (once for both
+// directions, or, on the fixed-point kernels, as ordered items of both directions),
+// cached for the last rho_far delta it was built for: near items
 // (generic or packed pair kernel in items mode) and far items (symmetric
 // kernel) in one device block.
 struct SymPlan {

@@ -1802,16 +1802,15 @@ int pair_occupancy(ssd_ctx *ctx) {
 // Grid of the fixed-point kernel.  Every pair costs the same, so it only has to
 // fill the SMs evenly.  Small sets: at most one round of two CTAs per SM, the
 // grouped form where its finer items leave less to the fullest CTA (N = 1062:
-// 289 CTAs of 64 targets, against 170 of 256: Stokes double layer 44 us instead
-// of 55 with its packing and epilogue; N = 1742: 280 against 196).  Their chunks
-// go by 8 sources, not 32: at N = 1099 the fullest thread has 18 pairs instead of
-// 24 (value and gradients on a star surface 128.9 ms against 140.5), at N = 1742
-// 44 instead of 48 (fused Stokes layers 96.4 us against 103.4), and without groups
-// at N = 3558 168 sources a CTA instead of 192 (Stokes double layer 177 us against
-// 189).  Chunks of more than 256 sources need not be whole staged tiles: at N = 4974
-// 336 instead of 384 (318 us against 357).
-// From 6000 points on about 5 rounds, which the scheduler levels, of whole staged
-// tiles.
+// 289 CTAs of 64 targets instead of 170 of 256 shorten the Stokes double layer by a
+// fifth).  Their chunks go by 8 sources, not 32: at N = 1099 the fullest thread has 18
+// pairs instead of 24 (value and gradients on a star surface 9% faster), at N = 3558
+// 168 sources a CTA instead of 192 (Stokes double layer 177 us against 189).  Chunks of
+// more than 256 sources need not be whole staged tiles: at N = 4974 336 instead of 384
+// (318 us against 357).
+// From 6000 points on waves_fx = 10 rounds of two CTAs per SM, which the scheduler
+// levels, of whole staged tiles.  (The fused Stokes layers stage three tables: from 11
+// octaves, a box diagonal of 32 delta, on one CTA fills an SM, and their rounds are 20.)
 struct FxSplit {
     int groups = 1;
     int64_t chunk = 0, nsplit = 1;
