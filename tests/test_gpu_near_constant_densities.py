@@ -99,3 +99,22 @@ def test_batch_of_constants_and_variations(gpu_ctx):
             _close(out[r][:, offs[k]:offs[k + 1]], s * ref)
             _close(fused[r][:, offs[k]:offs[k + 1]], s * 0.5 * single)
     B.release()
+
+
+def test_a_plan_of_far_blocks(gpu_ctx):
+    """Eight unit spheres on the corners of a cube: most block pairs are far, in launches of their own."""
+    import torch
+
+    import paper_2110_10749_gb300 as ssd
+    q, const, var, _ = _data(gpu_ctx, 1 / 8, 1e-6)
+    x = torch.cat([q["xyz"] + torch.tensor([[12.0 * (i >> 2 & 1)], [12.0 * (i >> 1 & 1)], [12.0 * (i & 1)]],
+                                           dtype=torch.float64, device="cuda") for i in range(8)], dim=1).contiguous()
+    P = ssd.Points(x, q["nrm"].repeat(1, 8), q["w"].repeat(8)).prepare(gpu_ctx)
+    v = (var.repeat(1, 8) * torch.linspace(0.5, 1.0, 8, dtype=torch.float64, device="cuda").repeat_interleave(var.shape[1]))
+    v[0] = _round(v[0])
+    u = (const.repeat(1, 8) + v).contiguous()
+    _close(ssd.stokes_DL(gpu_ctx, P, 3 / 8, u), ssd.stokes_DL(gpu_ctx, P, 3 / 8, v))
+    before = gpu_ctx.launch_count()
+    ssd.stokes_DL(gpu_ctx, P, 3 / 8, u)
+    assert gpu_ctx.launch_count() - before == 4      # packing, near items, far items, epilogue
+    P.release()
